@@ -167,11 +167,16 @@ __global__ void __launch_bounds__(kRedThreads) k_transition_group(const C* __res
     write_partial2(re, im, part);
 }
 
-// sum of |psi_x|^2 over the x whose measured bits are fixed: i runs over the free qubits, its
-// bits deposited at their positions, the measured ones set from `set`
+// sum of |psi_x|^2 over the x whose measured bits are fixed: i runs over the free qubits in
+// ascending order, the measured bits set from `set`. x is formed from i by the shorter of two
+// loops, the same x either way: one free bit deposited per step, or a zero inserted at each
+// measured position (ascending). At n = 28 with 4 measured qubits (24 free): 201 us with 24
+// deposits per amplitude, 155 us with 4 insertions (four loads in
+// flight per thread measured no faster).
 struct FreeBits {
     uint64_t set;
-    int32_t nfree;
+    int32_t nfree, nfix;
+    int32_t insert;  // 1: pos holds the measured positions, 0: the free ones
     int8_t pos[64];
 };
 template <typename C>
@@ -182,7 +187,18 @@ __global__ void __launch_bounds__(kRedThreads) k_norm2_sub(const C* __restrict__
     const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
     for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n_iter; i += stride) {
         uint64_t x = F.set;
-        for (int j = 0; j < F.nfree; j++) x |= ((i >> j) & 1ull) << F.pos[j];
+        if (F.insert) {
+            uint64_t y = i;
+#pragma unroll 1
+            for (int j = 0; j < F.nfix; j++) {
+                const uint64_t lo = y & ((1ull << F.pos[j]) - 1ull);
+                y = ((y ^ lo) << 1) | lo;
+            }
+            x |= y;
+        } else {
+#pragma unroll 1
+            for (int j = 0; j < F.nfree; j++) x |= ((i >> j) & 1ull) << F.pos[j];
+        }
         const double2 v = widen(psi[x]);
         acc = fma(v.x, v.x, acc);
         acc = fma(v.y, v.y, acc);
@@ -190,11 +206,85 @@ __global__ void __launch_bounds__(kRedThreads) k_norm2_sub(const C* __restrict__
     write_partial2(acc, 0.0, part);
 }
 
-// sampling, step 1: probability mass of each chunk of 2^chunk_log amplitudes (one block each)
-template <typename C>
+// |v|^2 of an amplitude as an unevaluated FP32 pair (2^-45 relative): the parts split on the integer
+// pipes, exact hi x hi products
+__device__ __forceinline__ void df_square_sum(float xh, float xl, float yh, float yl, float& s, float& c) {
+    const float p = __fmul_rn(xh, xh), q = __fmul_rn(yh, yh);
+    const float e = __fmaf_rn(__fadd_rn(xh, xh), xl, __fmaf_rn(xh, xh, -p));
+    const float f = __fmaf_rn(__fadd_rn(yh, yh), yl, __fmaf_rn(yh, yh, -q));
+    float t;
+    DFArith::two_sum(p, q, s, t);
+    c = __fadd_rn(t, __fadd_rn(e, f));
+}
+__device__ __forceinline__ void df_mass(double2 v, float& s, float& c) {
+    float xh, xl, yh, yl;
+    split_double_int(v.x, xh, xl);
+    split_double_int(v.y, yh, yl);
+    df_square_sum(xh, xl, yh, yl, s, c);
+}
+__device__ __forceinline__ void df_mass(float2 v, float& s, float& c) { df_square_sum(v.x, 0.f, v.y, 0.f, s, c); }
+__device__ __forceinline__ void df_mass(float4 v, float& s, float& c) { df_square_sum(v.x, v.y, v.z, v.w, s, c); }
+// (s, c) += (os, oc)
+__device__ __forceinline__ void df_pair_add(float& s, float& c, float os, float oc) {
+    float h, e;
+    DFArith::two_sum(s, os, h, e);
+    s = h;
+    c = __fadd_rn(c, __fadd_rn(oc, e));
+}
+
+constexpr int kSampleChunkLog = 12;                       // amplitudes per sampling chunk
+constexpr int kSegsPerChunk = (1 << kSampleChunkLog) / 32;  // segments of 32 amplitudes
+
+// sampling, step 1: probability mass of each chunk of 2^chunk_log amplitudes (one block each).
+// kSegs (chunks of 2^12): also the mass of every 32-amplitude segment as an FP32 pair, for
+// k_sample_pick. The FP64 chunk mass bounds the kernel (two FMA per amplitude, GB300's FP64 rate),
+// the segment sums run on the idle FP32 and integer pipes beside it: 1060 us without
+// them at n = 28 (complex128), 1441 us with them.
+template <typename C, bool kSegs>
 __global__ void __launch_bounds__(kRedThreads) k_chunk_mass(const C* __restrict__ psi, uint64_t N, int chunk_log,
-                                                            double* mass) {
+                                                            double* mass, float2* __restrict__ segs) {
     const uint64_t base = uint64_t(blockIdx.x) << chunk_log;
+    if constexpr (kSegs) {
+        constexpr int J = (1 << kSampleChunkLog) / kRedThreads;  // amplitudes per thread
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        C v[J];
+#pragma unroll
+        for (int j = 0; j < J; j++) v[j] = psi[base + threadIdx.x + j * kRedThreads];
+        double acc = 0.0;
+        float s[J], c[J];
+#pragma unroll
+        for (int j = 0; j < J; j++) {
+            const double2 w = widen(v[j]);
+            acc = fma(w.x, w.x, acc);
+            acc = fma(w.y, w.y, acc);
+            df_mass(v[j], s[j], c[j]);
+        }
+        // J sums over the warp's lanes at once: in each of the first four stages a lane keeps half of
+        // its sums and gives the other half away, so lane l ends with segment j(l)'s sum over 16
+        // lanes, and a last stage adds the two halves
+        int own = 0;
+#pragma unroll
+        for (int half = J / 2, bit = 1; half >= 1; half /= 2, bit <<= 1) {
+            const bool up = (lane & bit) != 0;
+            own = own * 2 + (up ? 1 : 0);
+#pragma unroll
+            for (int j = 0; j < half; j++) {
+                const float gs = up ? s[j] : s[j + half], gc = up ? c[j] : c[j + half];
+                if (up) {
+                    s[j] = s[j + half];
+                    c[j] = c[j + half];
+                }
+                df_pair_add(s[j], c[j], __shfl_xor_sync(0xffffffffu, gs, bit), __shfl_xor_sync(0xffffffffu, gc, bit));
+            }
+        }
+        df_pair_add(s[0], c[0], __shfl_xor_sync(0xffffffffu, s[0], 16), __shfl_xor_sync(0xffffffffu, c[0], 16));
+        // segment (j, warp) covers amplitudes j * 256 + warp * 32 ..
+        if (lane < 16) segs[size_t(blockIdx.x) * kSegsPerChunk + own * (kRedThreads / 32) + warp] = make_float2(s[0], c[0]);
+        __shared__ double sh[kRedThreads / 32];
+        const double r = block_sum<kRedThreads>(acc, sh);
+        if (threadIdx.x == 0) mass[blockIdx.x] = r;
+        return;
+    }
     const uint64_t end = N < base + (1ull << chunk_log) ? N : base + (1ull << chunk_log);
     double acc = 0.0;
     for (uint64_t x = base + threadIdx.x; x < end; x += blockDim.x) {
@@ -207,17 +297,30 @@ __global__ void __launch_bounds__(kRedThreads) k_chunk_mass(const C* __restrict_
     if (threadIdx.x == 0) mass[blockIdx.x] = r;
 }
 
-// sampling, step 2: one warp per sample finds, inside its chunk, the first x whose running mass
-// (lanes own consecutive stretches, summed in order) exceeds the residual target
+// sampling, step 2: each sample's chunk (the first whose cumulative mass exceeds u * total; at the
+// top, where rounding may leave none, the last chunk with mass) and residual target
+__global__ void __launch_bounds__(kRedThreads) k_sample_chunk(const double* __restrict__ cum, uint64_t B,
+                                                              const double* __restrict__ u, double total,
+                                                              uint64_t last, int count, uint64_t* __restrict__ chunk,
+                                                              double* __restrict__ resid) {
+    const int k = int(blockIdx.x * blockDim.x + threadIdx.x);
+    if (k >= count) return;
+    const double target = __dmul_rn(u[k], total);
+    uint64_t lo = 0, hi = B;  // first c in [0, B) with cum[c + 1] > target, B if none
+    while (lo < hi) {
+        const uint64_t mid = (lo + hi) >> 1;
+        if (cum[mid + 1] > target) hi = mid; else lo = mid + 1;
+    }
+    const uint64_t c = lo < B ? lo : last;
+    chunk[k] = c;
+    resid[k] = __dsub_rn(target, cum[c]);
+}
+
+// sampling, step 3: one warp finds, inside the sample's chunk, the first x whose running mass
+// (lanes own consecutive stretches, summed in order, FP64) exceeds the residual target
 template <typename C>
-__global__ void __launch_bounds__(kRedThreads) k_sample_find(const C* __restrict__ psi, uint64_t N, int chunk_log,
-                                                             const uint64_t* __restrict__ chunk,
-                                                             const double* __restrict__ resid, int count,
-                                                             uint64_t* __restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    const int s = int((uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5);
-    if (s >= count) return;
-    const uint64_t base = chunk[s] << chunk_log;
+__device__ __forceinline__ void sample_find_warp(const C* __restrict__ psi, uint64_t N, int chunk_log, uint64_t base,
+                                                 double r, int lane, uint64_t* __restrict__ out) {
     const uint64_t len = N - base < (1ull << chunk_log) ? N - base : (1ull << chunk_log);
     const uint64_t per = (len + 31) / 32;
     const uint64_t lo = len < uint64_t(lane) * per ? len : uint64_t(lane) * per;
@@ -233,7 +336,6 @@ __global__ void __launch_bounds__(kRedThreads) k_sample_find(const C* __restrict
         const double v = __shfl_up_sync(0xffffffffu, incl, d);
         if (lane >= d) incl += v;
     }
-    const double r = resid[s];
     const unsigned over = __ballot_sync(0xffffffffu, incl > r);
     const unsigned nonzero = __ballot_sync(0xffffffffu, own > 0.0);
     // the lane whose stretch crosses r; past the end (rounding) the last lane with mass
@@ -252,8 +354,107 @@ __global__ void __launch_bounds__(kRedThreads) k_sample_find(const C* __restrict
                 break;
             }
         }
-        out[s] = base + (found ? pick : last);
+        *out = base + (found ? pick : last);
     }
+}
+template <typename C>
+__global__ void __launch_bounds__(kRedThreads) k_sample_find(const C* __restrict__ psi, uint64_t N, int chunk_log,
+                                                             const uint64_t* __restrict__ chunk,
+                                                             const double* __restrict__ resid, int count,
+                                                             uint64_t* __restrict__ out) {
+    const int s = int((uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5);
+    if (s >= count) return;
+    sample_find_warp(psi, N, chunk_log, chunk[s] << chunk_log, resid[s], threadIdx.x & 31, out + s);
+}
+
+// The same from the segment masses: the segment by a scan of the chunk's 128 segment sums (FP32
+// pairs, four per lane), then the amplitude by a scan of the segment's 32 masses: 1.5 KB read per
+// sample instead of the chunk's 64 KB (complex128), and no FP64. The pick stands only where r lies
+// further than 2^-38 of the chunk's mass from both of its edges, which is beyond what the FP64 sums
+// of k_sample_find (under 2^-44) and the pairs here (under 2^-40) can be off, so both kernels return
+// the same index; any other sample (about 1 in 2^25, and every one of a chunk whose mass leaves the
+// range where FP32 pairs hold it) is found as there. 10^5 samples at n = 28: 4254 us by the
+// chunk search, 91 us here.
+template <typename C>
+__global__ void __launch_bounds__(kRedThreads) k_sample_pick(const C* __restrict__ psi, uint64_t N,
+                                                             const uint64_t* __restrict__ chunk,
+                                                             const double* __restrict__ resid,
+                                                             const float2* __restrict__ segs, int count,
+                                                             uint64_t* __restrict__ out) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int k = int((uint64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5);
+    if (k >= count) return;
+    const uint64_t ch = chunk[k], base = ch << kSampleChunkLog;
+    const double r = resid[k];
+    float rh, rl;
+    split_double(r, rh, rl);
+    auto scan = [&](float& s, float& c) {  // inclusive over the lanes
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const float os = __shfl_up_sync(kAll, s, d), oc = __shfl_up_sync(kAll, c, d);
+            if (lane >= d) df_pair_add(s, c, os, oc);
+        }
+    };
+    auto above = [&](float s, float c) { return __fadd_rn(__fsub_rn(s, rh), __fsub_rn(c, rl)); };  // (s + c) - r
+    constexpr int kPer = kSegsPerChunk / 32;
+    float s[kPer], c[kPer];
+#pragma unroll
+    for (int j = 0; j < kPer; j++) {
+        const float2 v = segs[ch * kSegsPerChunk + lane * kPer + j];
+        s[j] = v.x;
+        c[j] = v.y;
+        if (j) df_pair_add(s[j], c[j], s[j - 1], c[j - 1]);
+    }
+    float ts = s[kPer - 1], tc = c[kPer - 1];
+    scan(ts, tc);
+    const float total = __shfl_sync(kAll, ts, 31);
+    float es = __shfl_up_sync(kAll, ts, 1), ec = __shfl_up_sync(kAll, tc, 1);  // exclusive
+    if (lane == 0) es = ec = 0.f;
+    bool fine = total > 0x1p-60f && total < 0x1p60f && r >= 0.0;
+    // first segment whose inclusive sum exceeds r
+    int j = kPer;
+    float ps = es, pc = ec;  // its exclusive sum
+#pragma unroll
+    for (int i = kPer - 1; i >= 0; i--) {
+        float is = s[i], ic = c[i];
+        df_pair_add(is, ic, es, ec);
+        if (above(is, ic) > 0.f) j = i;
+    }
+#pragma unroll
+    for (int i = 0; i < kPer - 1; i++)
+        if (j == i + 1) {
+            ps = s[i];
+            pc = c[i];
+            df_pair_add(ps, pc, es, ec);
+        }
+    const unsigned over = __ballot_sync(kAll, j < kPer);
+    fine = fine && over != 0u;
+    const int L = over ? __ffs(over) - 1 : 0;
+    const int seg = L * kPer + min(__shfl_sync(kAll, j, L), kPer - 1);
+    ps = __shfl_sync(kAll, ps, L);
+    pc = __shfl_sync(kAll, pc, L);
+    // first amplitude of the segment whose inclusive sum exceeds r
+    const uint64_t x = base + uint64_t(seg) * 32 + lane;
+    float ms, mc;
+    df_mass(psi[x], ms, mc);
+    scan(ms, mc);
+    df_pair_add(ms, mc, ps, pc);
+    float bs = __shfl_up_sync(kAll, ms, 1), bc = __shfl_up_sync(kAll, mc, 1);
+    if (lane == 0) {
+        bs = ps;
+        bc = pc;
+    }
+    const unsigned hit = __ballot_sync(kAll, above(ms, mc) > 0.f);
+    const int lx = hit ? __ffs(hit) - 1 : 0;
+    const float margin = total * 0x1p-38f;
+    const bool clear = lane != lx || (above(ms, mc) > margin && above(bs, bc) < -margin);
+    fine = fine && hit != 0u && __all_sync(kAll, clear);
+    if (fine) {
+        if (lane == lx) out[k] = x;
+        return;
+    }
+    sample_find_warp(psi, N, kSampleChunkLog, base, r, lane, out + k);
 }
 
 // sum of `nslots` (re, im) partials in a fixed order -> out[0..1]
@@ -550,12 +751,16 @@ void reduce_marginal(const qs_state* st, const int32_t* measured, double* out) {
     qs_state* s = const_cast<qs_state*>(st);
     FreeBits F;
     F.set = 0;
-    F.nfree = 0;
+    F.nfree = F.nfix = 0;
     for (int q = 0; q < s->n; q++) {
         QS_REQUIRE(measured[q] >= 0 && measured[q] <= 2, "measured values must be 0, 1 or 2 (any)");
-        if (measured[q] == 2) F.pos[F.nfree++] = int8_t(q);
-        else if (measured[q] == 1) F.set |= 1ull << q;
+        F.nfree += measured[q] == 2;
+        F.nfix += measured[q] != 2;
+        if (measured[q] == 1) F.set |= 1ull << q;
     }
+    F.insert = F.nfix < F.nfree ? 1 : 0;
+    for (int q = 0, j = 0; q < s->n; q++)
+        if ((measured[q] == 2) != (F.insert == 1)) F.pos[j++] = int8_t(q);
     const uint64_t work = 1ull << F.nfree;
     const unsigned g = red_grid(work);
     ensure_scratch(s, 2 * g + 2);
@@ -566,29 +771,54 @@ void reduce_marginal(const qs_state* st, const int32_t* measured, double* out) {
     *out = r[0];
 }
 
+// Sampling: chunk masses (FP64), their cumulative sums in order on the host (a sequential sum, so
+// that its rounding is one order whatever the GPU), then per sample the chunk by bisection and the
+// index inside it. The mass pass also forms the segment sums that k_sample_pick reads where they
+// save more than they cost: 370 us per 65536 chunks, against k_sample_find's 0.054 us per sample and
+// about 60 us of its serial chain, so from count + 1024 >= chunks / 8 on. Whole calls, chunk search /
+// segment sums: 194 / 157 us for 256 samples at n = 24, 126 / 65 us for 16 at n = 20; at n = 28,
+// 1428 us for 4095 samples by the chunk search and 1578 us for 4096 with segment sums.
+
 void sample_state(const qs_state* st, int count, const double* uniforms, uint64_t* out) {
     qs_state* s = const_cast<qs_state*>(st);
     if (count == 0) return;
     for (int k = 0; k < count; k++) QS_REQUIRE(uniforms[k] >= 0.0 && uniforms[k] < 1.0, "uniforms must lie in [0, 1)");
     const uint64_t N = 1ull << s->n;
-    const int chunk_log = std::min(s->n, 12);
+    const int chunk_log = std::min(s->n, kSampleChunkLog);
     const uint64_t B = N >> chunk_log;
-    double* d_mass = nullptr;
-    uint64_t* d_chunk = nullptr;
-    double* d_resid = nullptr;
-    uint64_t* d_out = nullptr;
+    bool segs = chunk_log == kSampleChunkLog && uint64_t(count) + 1024 >= B / 8;
+    // one allocation: masses, cumulative masses, uniforms, residuals, chunks, results, segment sums
+    // (1/64 of a complex128 state; without them where that much memory is not left)
+    const size_t nc = size_t(count);
+    const size_t doubles = B + (B + 1) + 4 * nc;
+    double* d = nullptr;
     auto cleanup = [&]() {
-        if (d_mass) dev_free_async(d_mass, s->stream);
-        if (d_chunk) dev_free_async(d_chunk, s->stream);
-        if (d_resid) dev_free_async(d_resid, s->stream);
-        if (d_out) dev_free_async(d_out, s->stream);
+        if (d) dev_free_async(d, s->stream);
     };
     try {
-        QS_TRY_CUDA(dev_malloc_async(reinterpret_cast<void**>(&d_mass), B * sizeof(double), s->stream));
+        if (segs && dev_malloc_async(reinterpret_cast<void**>(&d), (doubles + B * kSegsPerChunk) * sizeof(double),
+                                     s->stream) != cudaSuccess) {
+            cudaGetLastError();
+            d = nullptr;
+            segs = false;
+        }
+        if (!d) QS_TRY_CUDA(dev_malloc_async(reinterpret_cast<void**>(&d), doubles * sizeof(double), s->stream));
+        double* d_mass = d;
+        double* d_cum = d_mass + B;
+        double* d_u = d_cum + (B + 1);
+        double* d_resid = d_u + nc;
+        uint64_t* d_chunk = reinterpret_cast<uint64_t*>(d_resid + nc);
+        uint64_t* d_out = d_chunk + nc;
+        float2* d_segs = reinterpret_cast<float2*>(d_out + nc);
         with_type(arith_of(s), s->data, [&](auto p) {
-            k_chunk_mass<<<unsigned(B), kRedThreads, 0, s->stream>>>(p, N, chunk_log, d_mass);
+            using C = std::remove_const_t<std::remove_pointer_t<decltype(p)>>;
+            if (segs)
+                k_chunk_mass<C, true><<<unsigned(B), kRedThreads, 0, s->stream>>>(p, N, chunk_log, d_mass, d_segs);
+            else
+                k_chunk_mass<C, false><<<unsigned(B), kRedThreads, 0, s->stream>>>(p, N, chunk_log, d_mass, nullptr);
         });
         QS_TRY_CUDA(cudaGetLastError());
+        QS_TRY_CUDA(cudaMemcpyAsync(d_u, uniforms, nc * sizeof(double), cudaMemcpyHostToDevice, s->stream));
         // cumulative distribution over chunks, in order, on the host
         std::vector<double> mass(B), cum(B + 1, 0.0);
         QS_TRY_CUDA(cudaMemcpyAsync(mass.data(), d_mass, B * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
@@ -596,32 +826,23 @@ void sample_state(const qs_state* st, int count, const double* uniforms, uint64_
         for (uint64_t b = 0; b < B; b++) cum[b + 1] = cum[b] + mass[b];
         const double total = cum[B];
         if (!(total > 0.0)) throw Error{QS_ERR_NUMERIC, "sampling a zero state"};
-        std::vector<uint64_t> chunk(count);
-        std::vector<double> resid(count);
-        for (int k = 0; k < count; k++) {
-            const double target = uniforms[k] * total;
-            // first chunk whose cumulative mass exceeds the target
-            uint64_t c = uint64_t(std::upper_bound(cum.begin() + 1, cum.end(), target) - (cum.begin() + 1));
-            if (c >= B) {  // rounding at the top: the last chunk with mass
-                c = B - 1;
-                while (c > 0 && !(mass[c] > 0.0)) c--;
-            }
-            chunk[k] = c;
-            resid[k] = target - cum[c];
-        }
-        QS_TRY_CUDA(dev_malloc_async(reinterpret_cast<void**>(&d_chunk), count * sizeof(uint64_t), s->stream));
-        QS_TRY_CUDA(dev_malloc_async(reinterpret_cast<void**>(&d_resid), count * sizeof(double), s->stream));
-        QS_TRY_CUDA(dev_malloc_async(reinterpret_cast<void**>(&d_out), count * sizeof(uint64_t), s->stream));
-        QS_TRY_CUDA(cudaMemcpyAsync(d_chunk, chunk.data(), count * sizeof(uint64_t), cudaMemcpyHostToDevice, s->stream));
-        QS_TRY_CUDA(cudaMemcpyAsync(d_resid, resid.data(), count * sizeof(double), cudaMemcpyHostToDevice, s->stream));
+        uint64_t last = B - 1;
+        while (last > 0 && !(mass[last] > 0.0)) last--;
+        QS_TRY_CUDA(cudaMemcpyAsync(d_cum, cum.data(), (B + 1) * sizeof(double), cudaMemcpyHostToDevice, s->stream));
+        k_sample_chunk<<<unsigned((nc + kRedThreads - 1) / kRedThreads), kRedThreads, 0, s->stream>>>(
+            d_cum, B, d_u, total, last, count, d_chunk, d_resid);
         const unsigned blocks = unsigned((uint64_t(count) * 32 + kRedThreads - 1) / kRedThreads);
         with_type(arith_of(s), s->data, [&](auto p) {
-            k_sample_find<<<blocks, kRedThreads, 0, s->stream>>>(p, N, chunk_log, d_chunk, d_resid, count, d_out);
+            if (segs)
+                k_sample_pick<<<blocks, kRedThreads, 0, s->stream>>>(p, N, d_chunk, d_resid, d_segs, count, d_out);
+            else
+                k_sample_find<<<blocks, kRedThreads, 0, s->stream>>>(p, N, chunk_log, d_chunk, d_resid, count, d_out);
         });
         QS_TRY_CUDA(cudaGetLastError());
-        QS_TRY_CUDA(cudaMemcpyAsync(out, d_out, count * sizeof(uint64_t), cudaMemcpyDeviceToHost, s->stream));
+        QS_TRY_CUDA(cudaMemcpyAsync(out, d_out, nc * sizeof(uint64_t), cudaMemcpyDeviceToHost, s->stream));
         QS_TRY_CUDA(cudaStreamSynchronize(s->stream));
     } catch (...) {
+        cudaStreamSynchronize(s->stream);  // copies in flight may still read this call's host vectors
         cleanup();
         throw;
     }
