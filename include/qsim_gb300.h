@@ -204,7 +204,8 @@ qs_status qs_apply_gate(qs_state* s, const qs_gate* g);
 /* psi <- K psi for a dense k-qubit matrix (k in 1..6), as produced by gate fusion
  * (Sec. 5.4 merge). Equivalent to qs_apply_gate with a QS_GATE_DENSE gate. */
 qs_status qs_apply_fused(qs_state* s, int k, const int* targets, const double* mat);
-/* Applies every gate of c in order. fusion_k = 0 applies gate by gate; 1..6 first merges
+/* Applies every gate of c in order. fusion_k = 0 applies gate by gate (each gate its own update,
+ * several gates per pass over the state where their qubits allow); 1..6 first merges
  * gates into dense blocks of at most fusion_k qubits (Sec. 5.4 merge; the planner keeps the
  * partition with fewer blocks of two: an open-block greedy one, where a gate joins the open
  * block while the union of qubits stays within the width, and a frontier-growth one, which

@@ -149,12 +149,40 @@ void apply_single(qs_state* s, const Op& op) {
     launch_op(op, s->data, s->n, s->dt, s->stream, stage_of(s));
 }
 
+// Ops applied gate by gate, several per pass over the state (qsim_pass.cu). A pass whose gates move
+// less than a full pass as launches of their own (one controlled phase, say) is launched gate by
+// gate from the size on where traffic counts more than launches.
+constexpr int kPassTrafficQubits = 18;
+void run_ops(qs_state* s, const std::vector<Op>& ops) {
+    const bool df_run = use_df(s) && !s->df;
+    const Arith ar = df_run ? Arith::DF : arith_of(s);
+    const std::vector<GatePass> passes = schedule_passes(ops, s->n, ar);
+    if (passes.empty()) {  // a double-float run rounds the state to that format whatever its gates
+        DFScope df(s, df_run);
+        return;
+    }
+    auto single = [&](const GatePass& p) { return !p.local || (p.share < 1.0 && s->n >= kPassTrafficQubits); };
+    // a double-float run changes the layout in its first and last passes where those are tile passes
+    const bool in = df_run && !single(passes.front()), out = df_run && !single(passes.back());
+    DFScope df(s, df_run, in);
+    for (size_t i = 0; i < passes.size(); i++) {
+        const GatePass& p = passes[i];
+        const bool last = i + 1 == passes.size();
+        if (single(p)) {
+            for (size_t k : p.ops) launch_op_arith(ops[k], s->data, s->n, ar, s->stream, stage_of(s));
+        } else {
+            launch_gate_pass(p, ops, s->data, s->n, ar, in && i == 0, out && last, s->stream);
+            if (in && i == 0) df.entered();
+            if (out && last) df.left();
+        }
+    }
+}
+
 void run_gates(qs_state* s, const qs_circuit* c, const double* theta) {
     std::vector<Op> ops;
     ops.reserve(c->n_gates);
     for (int i = 0; i < c->n_gates; i++) ops.push_back(op_of_gate(c->gates[i], s->n, theta));
-    DFScope df(s, use_df(s));
-    for (const Op& op : ops) launch_op_arith(op, s->data, s->n, arith_of(s), s->stream, stage_of(s));
+    run_ops(s, ops);
 }
 
 }  // namespace
@@ -395,13 +423,18 @@ Op trotter_op(const qs_pauli_obs* H, int k, double angle, int n_slices) {
     return op;
 }
 
-// one pass per term and slice
+// term by term, several per pass over the state
 void trotter_by_terms(qs_state* s, const qs_pauli_obs* H, double angle, int n_slices) {
     std::vector<Op> ops;
     for (int k = 0; k < H->n_terms; k++) ops.push_back(trotter_op(H, k, angle, n_slices));
-    DFScope df(s, use_df(s));
-    for (int r = 0; r < n_slices; r++)
-        for (const Op& op : ops) launch_op_arith(op, s->data, s->n, arith_of(s), s->stream, stage_of(s));
+    // slices in batches of a bounded number of ops
+    const int per = int(std::max<size_t>(1, 1024 / std::max<size_t>(1, ops.size())));
+    DFScope df(s, use_df(s) && n_slices > per);
+    for (int r = 0; r < n_slices; r += per) {
+        std::vector<Op> some;
+        for (int j = r; j < std::min(n_slices, r + per); j++) some.insert(some.end(), ops.begin(), ops.end());
+        run_ops(s, some);
+    }
 }
 
 // Where a pass over the state costs more than preparing a block on the host, the terms of up to 6

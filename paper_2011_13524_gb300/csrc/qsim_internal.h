@@ -212,6 +212,20 @@ void launch_from_df(void* psi, int n, cudaStream_t st);
 size_t kernel_entry_bytes(Arith ar);
 void encode_entries(Arith ar, const std::vector<cplx>& m, unsigned char* dst);
 
+// Several gates per pass over the state (qsim_pass.cu): the gates of a run in application order,
+// grouped into passes. local == 0: a single op that takes a launch of its own.
+struct GatePass {
+    std::vector<size_t> ops;  // indices into the run's ops
+    uint64_t local = 0;       // the tile's qubits
+    size_t data = 0;          // matrix entries
+    double share = 0.0;       // traffic of the ops as single launches, in full passes
+};
+int gate_pass_bits(int n, Arith ar);
+std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith ar);
+// ieee_in / ieee_out (double-float): psi holds / is left in IEEE complex128
+void launch_gate_pass(const GatePass& p, const std::vector<Op>& ops, void* psi, int n, Arith ar, bool ieee_in,
+                      bool ieee_out, cudaStream_t st);
+
 // Reductions: write results into the state's scratch and copy to host; synchronise.
 void reduce_norm2(qs_state* s, double* out);
 void reduce_inner(const qs_state* a, const qs_state* b, double out[2]);

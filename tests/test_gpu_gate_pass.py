@@ -1,0 +1,94 @@
+"""Several gates per pass (gate-by-gate circuit runs) against the same gates applied one call at a
+time, over tile edges, low, high and scattered qubits, controls, strings longer than a tile, and the
+layout changes folded into the first and last pass."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+# per gate 2^-46 (double-float; FP64 below it) or 2^-23 (complex64) of amplitudes <= 1, at most 400 gates
+TOL = {"df": 1e-12, "f64": 1e-12, "c64": 1e-5}
+
+
+def random_tensor(n, dtype, seed):
+    import torch
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    v = torch.randn(1 << n, dtype=dtype, device="cuda", generator=g)
+    return v / torch.linalg.vector_norm(v)
+
+
+def mixed_circuit(n, seed):
+    """Every gate kind twice in shuffled order, long Pauli rotations among them, between layers."""
+    rng = W.SplitMix64(seed)
+    gates = W.u3cz_circuit(n, 2, seed).gates
+    if n >= 6:
+        suite = W.random_gate_suite(n, seed) + W.random_gate_suite(n, seed + 1)
+        for i in range(len(suite) - 1, 0, -1):
+            j = rng.randint(0, i)
+            suite[i], suite[j] = suite[j], suite[i]
+        gates += suite
+        ids = tuple(rng.randint(1, 3) for _ in range(6))
+        gates.append(W.Gate("PAULIROT", tuple(range(n - 6, n)), pauli=ids, params=(0.4,)))
+    gates += W.hea_circuit(n, 1, seed).gates
+    return W.Circuit(n, gates)
+
+
+@pytest.mark.parametrize("arith", ["df", "f64", "c64"])
+@pytest.mark.parametrize("n", [1, 2, 5, 8, 9, 10, 12, 15, 18, 19, 21])
+def test_passes_equal_single_gates(n, arith):
+    import torch
+    import paper_2011_13524_gb300 as qs
+    dt, tdt = (qs.QS_C64, torch.complex64) if arith == "c64" else (qs.QS_C128, torch.complex128)
+    v = random_tensor(n, tdt, n)
+    a, b = qs.State(n, dt, tensor=v.clone()), qs.State(n, dt, tensor=v)
+    math = qs.QS_MATH_FP64 if arith == "f64" else qs.QS_MATH_DF
+    a.set_arith(math=math)
+    b.set_arith(math=qs.QS_MATH_FP64)
+    c = mixed_circuit(n, 3 + n) if n > 1 else W.Circuit(1, [W.Gate("H", (0,)), W.Gate("T", (0,)), W.Gate("RX", (0,), params=(0.3,))])
+    a.run(c, 0)
+    for g in c.gates:
+        b.apply_gate(g)
+    a.synchronize()
+    b.synchronize()
+    assert float((a.tensor - b.tensor).abs().max()) < TOL[arith]
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("arith", ["df", "c64"])
+def test_one_gate_runs(arith):
+    """Runs of a single gate of each kind: one pass that changes the layout on both sides."""
+    import torch
+    import paper_2011_13524_gb300 as qs
+    n = 13
+    dt, tdt = (qs.QS_C64, torch.complex64) if arith == "c64" else (qs.QS_C128, torch.complex128)
+    for i, g in enumerate(W.random_gate_suite(n, 8)):
+        v = random_tensor(n, tdt, i)
+        a, b = qs.State(n, dt, tensor=v.clone()), qs.State(n, dt, tensor=v)
+        b.set_arith(math=qs.QS_MATH_FP64)
+        a.run(W.Circuit(n, [g]), 0)
+        b.apply_gate(g)
+        a.synchronize()
+        b.synchronize()
+        assert float((a.tensor - b.tensor).abs().max()) < TOL[arith], g
+        a.close()
+        b.close()
+
+
+def test_long_runs_and_many_slices():
+    """More gates than the scheduler looks at together, and Trotter slices in batches."""
+    import paper_2011_13524_gb300 as qs
+    import oracle
+    c = W.u3cz_circuit(9, 90, 4)  # 1170 gates
+    st = qs.State(9, qs.QS_C128)
+    st.run(c, 0)
+    assert float(np.max(np.abs(st.get_vector() - oracle.run_circuit(c)))) < 2e-12
+    obs = W.random_pauli_observable(9, 9, 5)
+    psi = W.random_state(9, 3)
+    st.load(psi)
+    st.apply_observable_rotation(obs, 0.9, 150)  # 1350 rotations
+    assert float(np.max(np.abs(st.get_vector() - oracle.observable_rotation(psi, 9, obs, 0.9, 150)))) < 2e-12
+    st.close()
