@@ -902,6 +902,8 @@ void pack_tiles(const std::vector<PauliGroup>& groups, int n, int tbits, ExpectP
         for (const Chunk& c : B.ch) build(c, tpos, b, B.T, P);
         plan.passes.push_back(P);
         plan.tmask.push_back(B.T);
+        plan.chunks.emplace_back();
+        for (const Chunk& c : B.ch) plan.chunks.back().push_back(HeavyChunk{c.g, c.t0, c.t1});
     }
 }
 

@@ -320,6 +320,7 @@ struct DiagObsParams {
 struct ExpectPlan {
     std::vector<TileParams> passes;
     std::vector<uint64_t> tmask;     // qubits of each pass's tile
+    std::vector<std::vector<HeavyChunk>> chunks;  // each pass's groups
     std::vector<HeavyChunk> heavy;   // terms [t0, t1) of groups that fit no tile
     bool diag = false;               // a diagonal observable read in one streaming pass (dp)
     DiagObsParams dp;

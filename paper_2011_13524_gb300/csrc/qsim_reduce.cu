@@ -121,6 +121,101 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_group(const C* __restric
     write_partial2(re, im, part);
 }
 
+// One term per flip group (general Pauli strings): sum over the pairs (y, y ^ f) of
+// (-1)^popc(y & z) Re A or Im A with A = conj(psi_{y^f}) psi_y, whichever the string takes, many terms
+// in one launch (blockIdx.y). The coefficient and the pair's factor enter once per block.
+//  * complex128: two FP64 FMA per pair, the FP64 rate being the bound (the group kernel below takes
+//    seven per pair and term).
+//  * complex64: products exact in FP32 pairs, summed with two levels of compensation (TwoSum of the
+//    sums and of their errors: nothing above 2^-70 of a thread's sum is dropped), both components of a
+//    pair side by side in packed instructions; one FP64 conversion per thread.
+// 24 random strings, whole call, one launch per group / here: complex64 1.62 / 0.33 ms at n = 23 (284 us
+// of kernel, L2 reads and packed FP32 arithmetic about equal) and 67.8 / 12.9 ms at n = 28, complex128
+// 0.75 / 0.36 ms at n = 22 and 50.9 / 25.4 ms at n = 28.
+constexpr int kMaxSingles = 64;
+struct SingleTerm {
+    uint64_t f, z;
+    double coef;     // with the pair's factor +-2
+    int32_t pivot;   // lowest bit of f, clear in y
+    int32_t imag;    // 1: Im A
+};
+struct SingleParams {
+    uint64_t pairs;
+    SingleTerm t[kMaxSingles];
+};
+
+__device__ __forceinline__ float2 two_sum2(float2 a, float2 b, float2& e) {
+    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 h = __fadd2_rn(a, b);
+    const float2 bp = __ffma2_rn(a, m1, h);
+    e = __fadd2_rn(__ffma2_rn(__ffma2_rn(bp, m1, h), m1, a), __ffma2_rn(bp, m1, b));
+    return h;
+}
+struct SingleAccF {  // complex64
+    float2 s = make_float2(0.f, 0.f), c = make_float2(0.f, 0.f), d = make_float2(0.f, 0.f);
+    __device__ __forceinline__ void add(float2 a, float2 b, bool imag, int neg) {
+        const uint32_t sg = uint32_t(neg) << 31;
+        float2 u = imag ? make_float2(a.y, -a.x) : a;
+        u.x = __uint_as_float(__float_as_uint(u.x) ^ sg);
+        u.y = __uint_as_float(__float_as_uint(u.y) ^ sg);
+        const float2 p = __fmul2_rn(u, b);
+        float2 e, e2;
+        s = two_sum2(s, p, e);
+        e = __fadd2_rn(e, __ffma2_rn(u, b, make_float2(-p.x, -p.y)));
+        c = two_sum2(c, e, e2);
+        d = __fadd2_rn(d, e2);
+    }
+    __device__ double value() const {
+        return (double(s.x) + double(s.y)) + ((double(c.x) + double(c.y)) + (double(d.x) + double(d.y)));
+    }
+};
+struct SingleAccD {  // complex128
+    double s = 0.0, c = 0.0;
+    __device__ __forceinline__ void add(double2 a, double2 b, bool imag, int neg) {
+        const long long sg = static_cast<long long>(uint64_t(neg) << 63);
+        const double ux = imag ? a.y : a.x, uy = imag ? -a.x : a.y;
+        s = fma(__longlong_as_double(__double_as_longlong(ux) ^ sg), b.x, s);
+        c = fma(__longlong_as_double(__double_as_longlong(uy) ^ sg), b.y, c);
+    }
+    __device__ double value() const { return s + c; }
+};
+
+template <typename C, typename Acc>
+__global__ void __launch_bounds__(kRedThreads) k_expect_singles(const C* __restrict__ psi,
+                                                                const __grid_constant__ SingleParams P, double* part) {
+    const SingleTerm T = P.t[blockIdx.y];
+    const uint64_t lowmask = (1ull << T.pivot) - 1ull;
+    const bool imag = T.imag != 0;
+    Acc acc;
+    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
+    constexpr int kU = 4;  // pairs in flight per thread
+    for (uint64_t i0 = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i0 < P.pairs; i0 += kU * stride) {
+        C a[kU], b[kU];
+        int neg[kU];
+#pragma unroll
+        for (int u = 0; u < kU; u++) {
+            const uint64_t i = i0 + u * stride;
+            if (i >= P.pairs) break;
+            const uint64_t lo = i & lowmask, y = ((i ^ lo) << 1) | lo;
+            a[u] = psi[y];
+            b[u] = psi[y ^ T.f];
+            neg[u] = parity64(y & T.z);
+        }
+#pragma unroll
+        for (int u = 0; u < kU; u++) {
+            if (i0 + u * stride >= P.pairs) break;
+            acc.add(a[u], b[u], imag, neg[u]);
+        }
+    }
+    __shared__ double sh[kRedThreads / 32];
+    const double r = block_sum<kRedThreads>(acc.value(), sh);
+    if (threadIdx.x == 0) {
+        const size_t slot = size_t(blockIdx.y) * gridDim.x + blockIdx.x;
+        part[2 * slot] = T.coef * r;
+        part[2 * slot + 1] = 0.0;
+    }
+}
+
 // <lam| P |psi> = sum_y conj(lam_y) i^{#Y} s(y ^ f) psi_{y ^ f}
 template <typename C>
 __global__ void __launch_bounds__(kRedThreads) k_transition(const C* __restrict__ lam, const C* __restrict__ psi,
@@ -614,29 +709,77 @@ void reduce_inner(const qs_state* a, const qs_state* b, double out[2]) {
     finish2(s, int(g), out);
 }
 
-// Launches of one expectation: the tile passes, then one launch per heavy chunk. With a cap on
-// the block partials the grids shrink proportionally (the kernels loop over their work).
+// Launches of one expectation: the tile passes, one launch per heavy chunk, and the terms that are
+// alone in their flip group together (k_expect_singles): those that fit no tile, and one that a tile
+// pass would stage the state for alone (whole calls, tile pass / single term: 173 / 135 us at n = 25 and
+// 1138 / 790 us at n = 28 in complex128, 111 / 86 and 654 / 433 us in complex64; with two terms the tile
+// pass is the faster one, 740 / 1052 us at n = 28 in complex64). With a
+// cap on the block partials the grids shrink proportionally (the kernels loop over their work).
 struct ExpectLaunches {
     std::vector<unsigned> pass_grid, heavy_grid;  // a diagonal observable: its one streaming pass in pass_grid
+    std::vector<size_t> passes, heavy;            // indices into the plan
+    std::vector<SingleTerm> singles;
+    unsigned single_grid = 0;                     // blocks per single term
     size_t slots = 0;
 };
+SingleTerm single_term(const HeavyChunk& c) {
+    SingleTerm t;
+    t.f = c.g->xmask;
+    t.z = c.g->zmask[c.t0];
+    t.pivot = __builtin_ctzll(t.f);
+    const int nY = __builtin_popcountll(t.f & t.z);
+    t.imag = nY & 1;
+    t.coef = (((nY + 1) / 2) & 1) ? -2.0 * c.g->coef[c.t0] : 2.0 * c.g->coef[c.t0];
+    return t;
+}
 ExpectLaunches expectation_launches(const ExpectPlan& plan, int n, Arith ar, size_t cap) {
-    ExpectLaunches L;
-    if (plan.diag) L.pass_grid.push_back(expect_diag_grid(n, ar));
-    for (const TileParams& P : plan.passes) L.pass_grid.push_back(expect_pass_grid(P, ar));
-    for (const HeavyChunk& h : plan.heavy) L.heavy_grid.push_back(red_grid((1ull << n) >> (h.g->xmask ? 1 : 0)));
-    size_t tot = 0;
+    auto is_single = [&](const HeavyChunk& c) { return c.g->xmask && c.g->coef.size() == 1 && ar != Arith::DF; };
+    auto build = [&](bool take_light) {
+        ExpectLaunches L;
+        if (plan.diag) L.pass_grid.push_back(expect_diag_grid(n, ar));
+        for (size_t p = 0; p < plan.passes.size(); p++) {
+            const auto& ch = plan.chunks[p];
+            if (take_light && ch.size() == 1 && is_single(ch[0])) {
+                L.singles.push_back(single_term(ch[0]));
+                continue;
+            }
+            L.passes.push_back(p);
+            L.pass_grid.push_back(expect_pass_grid(plan.passes[p], ar));
+        }
+        for (size_t h = 0; h < plan.heavy.size(); h++) {
+            if (is_single(plan.heavy[h])) {
+                L.singles.push_back(single_term(plan.heavy[h]));
+                continue;
+            }
+            L.heavy.push_back(h);
+            L.heavy_grid.push_back(red_grid((1ull << n) >> (plan.heavy[h].g->xmask ? 1 : 0)));
+        }
+        return L;
+    };
+    ExpectLaunches L = build(true);
+    auto launches = [&]() { return L.pass_grid.size() + L.heavy_grid.size() + L.singles.size(); };
+    if (launches() > cap) L = build(false);
+    if (!L.singles.empty()) {
+        // eight pairs per thread, at most 256 blocks per term unless few terms leave the GPU idle (2432
+        // blocks per term measured no faster on states beyond L2: 25.4 / 25.9 ms for 24 strings at n = 28)
+        const uint64_t want = ((1ull << (n - 1)) + kRedThreads * 8 - 1) / (kRedThreads * 8);
+        const uint64_t most = std::max<uint64_t>(256, uint64_t(sms()) * 8 / L.singles.size());
+        L.single_grid = unsigned(std::max<uint64_t>(1, std::min(want, most)));
+    }
+    size_t tot = L.singles.size() * size_t(L.single_grid);
     for (unsigned g : L.pass_grid) tot += g;
     for (unsigned g : L.heavy_grid) tot += g;
     if (tot > cap) {
-        const size_t nl = L.pass_grid.size() + L.heavy_grid.size();
+        const size_t nl = launches();
         QS_REQUIRE(nl <= cap, "observable needs more kernel launches than the partial-sum scratch holds");
         const size_t per = cap / nl;
         for (unsigned& g : L.pass_grid) g = unsigned(std::min<size_t>(g, per));
         for (unsigned& g : L.heavy_grid) g = unsigned(std::min<size_t>(g, per));
+        L.single_grid = unsigned(std::min<size_t>(L.single_grid, per));
     }
     for (unsigned g : L.pass_grid) L.slots += g;
     for (unsigned g : L.heavy_grid) L.slots += g;
+    L.slots += L.singles.size() * size_t(L.single_grid);
     return L;
 }
 
@@ -647,12 +790,25 @@ void launch_expectation(const ExpectPlan& plan, const ExpectLaunches& L, const v
         launch_expect_diag(plan.dp, psi, ar, part, L.pass_grid[0], st);
         return;
     }
-    for (size_t p = 0; p < plan.passes.size(); p++) {
-        launch_expect_pass(plan.passes[p], psi, ar, part + 2 * slots, L.pass_grid[p], st);
+    for (size_t p = 0; p < L.passes.size(); p++) {
+        launch_expect_pass(plan.passes[L.passes[p]], psi, ar, part + 2 * slots, L.pass_grid[p], st);
         slots += L.pass_grid[p];
     }
-    for (size_t h = 0; h < plan.heavy.size(); h++) {
-        const HeavyChunk& c = plan.heavy[h];
+    for (size_t t0 = 0; t0 < L.singles.size(); t0 += kMaxSingles) {
+        SingleParams P;
+        P.pairs = 1ull << (n - 1);
+        const unsigned nt = unsigned(std::min<size_t>(kMaxSingles, L.singles.size() - t0));
+        for (unsigned t = 0; t < nt; t++) P.t[t] = L.singles[t0 + t];
+        const dim3 grid(L.single_grid, nt);
+        if (ar == Arith::F32)
+            k_expect_singles<float2, SingleAccF><<<grid, kRedThreads, 0, st>>>(static_cast<const float2*>(psi), P, part + 2 * slots);
+        else
+            k_expect_singles<double2, SingleAccD><<<grid, kRedThreads, 0, st>>>(static_cast<const double2*>(psi), P, part + 2 * slots);
+        QS_TRY_CUDA(cudaGetLastError());
+        slots += size_t(nt) * L.single_grid;
+    }
+    for (size_t h = 0; h < L.heavy.size(); h++) {
+        const HeavyChunk& c = plan.heavy[L.heavy[h]];
         TermParams P;
         P.xmask = c.g->xmask;
         std::vector<int> fixed;
