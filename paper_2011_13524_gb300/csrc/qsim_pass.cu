@@ -13,14 +13,16 @@
 // gate), large complex64 states by shared-memory traffic and index work, each instead of HBM.
 // Measured, random U3 + CZ circuits of depth 10 gate by gate, one pass per gate / several: complex128
 // 783 / 142 us at n = 12 (175 gates), 1047 / 197 us at n = 16, 5.11 / 4.36 ms at n = 22, 1936 / 1434 ms
-// at n = 30; complex64 1168 / 229 us at n = 18, 50.4 / 20.0 ms at n = 26, 913 / 365 ms at n = 30.
+// at n = 30; complex64 1168 / 302 us at n = 18, 50.4 / 20.5 ms at n = 26, 913 / 368 ms at n = 30.
 // Two CTAs per SM (106 registers) measured 2 % faster than three and 3 % faster than four (spills);
 // staging the gate records in shared memory instead of the parameter bank gave 31 -> 29 us per pass at
 // n = 12 and lost 7 % in complex64 at n = 26, so the records stay in the parameter bank.
 //
 // Passes are formed on the host by list scheduling: the gates in order, each taken when it commutes
 // with every gate skipped before it (no shared qubit, or only diagonal action on the shared ones)
-// and its changed qubits fit L.
+// and its changed qubits fit L. In complex64 a pass ends at the first gate that does not fit: every
+// amplitude then sees its gates in circuit order with the roundings of single launches (an FP32 value
+// computed from the state would otherwise change in its seventh digit with the order).
 #include <algorithm>
 #include <memory>
 
@@ -173,6 +175,18 @@ __device__ __forceinline__ uint32_t insert_zero(uint32_t j, int p) {
     return ((j ^ lo) << 1) | lo;
 }
 
+// k v, rounded as k_phase and k_diag do
+template <typename P>
+__device__ __forceinline__ typename P::C pass_mul(const typename P::K& k, const typename P::C& v) {
+    typename P::Acc a = P::zero();
+    P::mac(a, k, v);
+    return P::out(a);
+}
+template <>
+__device__ __forceinline__ float4 pass_mul<DFArith>(const float4& k, const float4& v) {
+    return DFArith::out(DFArith::first(k, v));
+}
+
 template <typename P>
 __device__ __forceinline__ void pass_elementwise(typename P::C& v, int& sign, const PassOp& o,
                                                  const typename P::K* data, uint32_t l, uint64_t base) {
@@ -185,7 +199,7 @@ __device__ __forceinline__ void pass_elementwise(typename P::C& v, int& sign, co
     if (!on) return;
     switch (o.kind) {
         case kPassPhase:
-            v = o.mode == 0 ? P::out(P::first(data[o.data], v)) : P::ipow(v, o.mode);
+            v = o.mode == 0 ? pass_mul<P>(data[o.data], v) : P::ipow(v, o.mode);
             break;
         case kPassDiag: {
             uint32_t r = 0;
@@ -193,7 +207,7 @@ __device__ __forceinline__ void pass_elementwise(typename P::C& v, int& sign, co
                 const int p = o.pos[j];
                 r |= uint32_t(p < 128 ? (l >> p) & 1u : uint32_t(base >> (p - 128)) & 1u) << j;
             }
-            v = P::out(P::first(data[o.data + r], v));
+            v = pass_mul<P>(data[o.data + r], v);
             break;
         }
         case kPassZSign:
@@ -526,7 +540,8 @@ void launch_pass_p(const Op* const* ops, int nops, size_t ndata, uint64_t local,
 // Tile bits: up to a 32 KB tile (fewer passes) once 2^8 tiles fill the SMs, never below 8 (9 in FP32)
 // bits: under that the extra passes cost more than the wider spread over SMs gives. Whole calls of the
 // depth-10 circuit with at least 7 / 8 / 9 bits: 147 / 142 / 152 us at n = 12 and 173 / 162 / 175 at
-// n = 14 in complex128, 138 / 123 / 124 us at n = 12 and 159 / 147 / 145 at n = 14 in complex64.
+// n = 14 in complex128, 138 / 123 / 124 us at n = 12 and 159 / 147 / 145 at n = 14 in complex64 (with
+// passes in any order).
 int gate_pass_bits(int n, Arith ar) {
     const int most = ar == Arith::F32 ? 12 : 11, least = ar == Arith::F32 ? 9 : 8;
     return std::min(n, std::max(least, std::min(most, n - 8)));
@@ -564,10 +579,11 @@ std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith a
         size_t data = 0;
         double share = 0.0;
         keep.clear();
+        bool ended = false;
         for (size_t i : rem) {
             const Op& op = ops[i];
             const size_t e = pass_entries(op);
-            if ((q[i].x & (bx | bd)) == 0 && (q[i].d & bx) == 0 && p.ops.size() < size_t(kPassOps) &&
+            if (!ended && (q[i].x & (bx | bd)) == 0 && (q[i].d & bx) == 0 && p.ops.size() < size_t(kPassOps) &&
                 data + e <= size_t(kPassData) && __builtin_popcountll(L | q[i].x) <= t && fits_alone(op, q[i])) {
                 L |= q[i].x;
                 data += e;
@@ -577,6 +593,7 @@ std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith a
                 bx |= q[i].x;
                 bd |= q[i].d;
                 keep.push_back(i);
+                ended = ar == Arith::F32;
             }
         }
         for (int b = 0; b < n && __builtin_popcountll(L) < t; b++) L |= 1ull << b;
