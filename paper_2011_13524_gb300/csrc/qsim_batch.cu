@@ -15,6 +15,18 @@
 //    the state one chunk of 2^13 amplitudes at a time (the chunk fixes the other qubits), each
 //    chunk staged in shared memory, so a whole pass costs one read and one write of the state.
 //  * n <= 13: the whole state (and lambda) stays in shared memory for the entire circuit.
+//  * A thread holds 16 amplitudes of psi (and of lambda) in registers for a stage. Z and CZ gates between
+//    two others are one sign per amplitude; a rotation is one body (gradient chain, both
+//    un-applications, the warp sum of the rotation before it) chosen by one branch, its two real
+//    products per part in packed FP32 pairs. The order of the roundings is the circuit's.
+//  * What bounds it: instruction issue (about 42 % of the slots, 16 warps per SM at 128 registers) and
+//    the stage barriers; 1100 instructions per amplitude and layer at 18 qubits, a third of them FP32.
+//    The next chunk's claim, look-ups and L2 prefetch run beside the current one's gates.
+//    512 circuits of 8..20 qubits: 64.0 ms with a loop over separate gates (per-register phase signs,
+//    one pass of negations per CZ, three branches per rotation), 48.0 ms with merged signs, packed
+//    pairs and uniform signs, 47.0 ms with one body per rotation and the claim ahead. Merging the RZ
+//    of a layer into one factor per amplitude measured 40.0 ms but changes the rounding of every
+//    amplitude in FP32; it is not used.
 //  * Forward sweep; lambda = H psi and E = Re <psi|lambda>; reverse sweep over passes and gates:
 //    at a rotation exp(i theta P/2) the gradient is -Im <lambda|P|psi>, then the gate is
 //    un-applied from psi and lambda.
@@ -22,6 +34,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <map>
 #include <memory>
 #include <numeric>
 
@@ -37,35 +50,61 @@ constexpr int kLocal = 13;             // qubits per chunk
 constexpr int kChunk = 1 << kLocal;    // 16 warps x 32 lanes x 16 registers
 constexpr int kRegBits = 4;
 constexpr int kRegs = 1 << kRegBits;
-constexpr int kMaxStageParams = 32;
+constexpr int kMaxStageRows = 32;   // gradient rows (sums per warp) of a stage
 constexpr int kClasses = 5;            // groups of 16, 8, 4, 2, 1 warps
+// a chunked pass's records kept in shared memory (larger passes read theirs from global memory)
+constexpr int kUnitOps = 512, kUnitStages = 64, kUnitSigns = 64;
 constexpr int kMaxBatchQubits = 24;
 
-enum BKind : uint8_t { BK_RX = 0, BK_RY = 1, BK_RZ = 2, BK_CZ = 3, BK_CNOT = 4, BK_H = 5, BK_X = 6, BK_Y = 7, BK_Z = 8 };
+enum BKind : uint8_t { BK_RX = 0, BK_RY = 1, BK_RZ = 2, BK_CZ = 3, BK_CNOT = 4, BK_H = 5, BK_X = 6, BK_Y = 7, BK_Z = 8, BK_SIGN = 9 };
 
-// one gate in the local coordinates of its pass
-struct __align__(16) BGate {
+// one gate of a circuit before planning (host)
+struct BGate {
     uint8_t kind;
-    uint8_t a;      // local bit of the target
-    uint8_t b;      // local bit of the second qubit (CZ) or of the control (CNOT)
-    uint8_t ja;     // register bit holding the target, or kNoReg when it is not a register bit
-    uint8_t jb;     // register bit holding the second qubit / control, or kNoReg
-    uint8_t pad[3];
+    uint8_t a;      // target qubit (then the local bit of its pass)
+    uint8_t b;      // second qubit (CZ) or control (CNOT)
     int32_t grad;   // gradient index (parametric rotations), -1 otherwise
-    float c, s;     // cos, sin of theta/2 (rotations; written before every run), else 1, 0
 };
 constexpr uint8_t kNoReg = 0xff;
 
-// gates whose non-diagonal actions stay inside the register sub-cube spanned by act[]
+// one step of a stage: a rotation or fixed gate, or a run of sign gates (Z, CZ)
+struct __align__(16) BOp {
+    float2 cs;      // cos, sin of theta/2 (rotations; written before every run); sign run: its index (bits of x)
+    uint8_t kind;
+    uint8_t j;      // register bit of the target, or kNoReg (RZ)
+    uint8_t b;      // RZ: local bit of the target; CNOT: of the control
+    uint8_t jb;     // CNOT: register bit of the control, or kNoReg
+    int16_t ref;    // rotations: gradient row of the stage (-1: none)
+    uint8_t code;   // what the stage bodies branch on: kCode*
+    uint8_t pad;
+};
+// rotations: their axis and register bit, one body each (RZ outside the registers: bit 4)
+constexpr int kCodeRX = 0, kCodeRY = 4, kCodeRZ = 8, kCodeFixed = 13, kCodeSign = 14, kCodeGrad = 16;
+
+// The signs of a run of Z and CZ gates: amplitude x of a thread (register index r, other local bits
+// `base`) is negated where the parity of its Z bits and CZ pairs is odd.
+struct BSign {
+    uint32_t nbr[4];    // CZ partners of register bit j among the other bits
+    uint32_t zbase;     // Z bits outside the registers
+    uint32_t pat;       // sign of register index r from Z and CZ within the register bits, bit r
+    int32_t cz0, ncz;   // CZ pairs on the other bits, grouped by distance
+};
+struct BCz {
+    uint32_t shift, mask;  // pairs (a, a + shift), bit a set
+};
+
+// gates whose non-diagonal actions stay inside the register sub-cube spanned by act[] (register bit j
+// is local bit act[j]; diagonal gates act on any bit)
 struct BStage {
-    int32_t g0, g1;
-    int32_t nact;
-    int32_t nparam;
+    int32_t o0, o1;     // steps
+    int32_t p0, np;     // gradient outputs: parameter of each row
     uint8_t act[4];
+    uint8_t sorted[4];  // act, ascending
 };
 
 struct BPass {
     int32_t s0, s1;               // stage range
+    int32_t o0, o1, g0, g1;       // its steps and sign runs
     uint32_t tab_lo[128];         // local index bits 0..6 -> address bits
     uint32_t tab_hi[64];          // local index bits 7..12 -> address bits
     uint32_t nonlocal;            // qubits outside the window (fixed per chunk)
@@ -92,6 +131,8 @@ struct LevelEntry {
     int32_t pass;                 // pass index (forward / reverse levels)
     int32_t unit0;                // first unit of this entry within the level
     int32_t kind;
+    uint64_t ws;                  // psi buffer of the item (amplitudes; lambda follows)
+    int32_t n, first;             // first: a forward pass that starts from |0...0>
 };
 constexpr long long kBarrierSpinLimit = 1ll << 25;  // x 256 ns sleeps: ~10 s
 // test hooks of the grid barrier (kernel arguments): polls before a wait gives up, and CTA 0
@@ -104,10 +145,12 @@ struct BatchDev {
     const int32_t* order;         // resident items grouped by class, longest first within a class
     const BPass* passes;
     const BStage* stages;
-    const BGate* gates;
+    const BOp* ops;
+    const BSign* signs;
+    const BCz* czs;
+    const int32_t* params;
     const BTerm* terms;
     float2* ws;                   // psi and lambda of every circuit wider than the window
-    const uint64_t* ws_off;       // item -> offset of its psi buffer (lambda follows)
     double* energy;
     double* grad;
     double* part_e;               // per wide item: energy partial per chunk
@@ -115,8 +158,10 @@ struct BatchDev {
     double* part_g;               // per wide item: gradient partial per (parameter, chunk)
     const int64_t* part_g_off;
     const LevelEntry* lev_entries;
-    const int32_t* lev_off;       // nlevels + 1
     const int32_t* lev_units;     // units per level
+    const int32_t* lev_pair0;     // level -> first element of lev_pairs
+    const int32_t* lev_pairs;     // entry of units 2 i and 2 i + 1 of a level (an entry has an even
+                                  // number of units; the last level one per entry, see kind)
     int32_t nlevels;
     unsigned int* counters;       // kClasses resident counters, then one per level
     unsigned int* bar_count;
@@ -142,10 +187,6 @@ __device__ __forceinline__ void gbar(int G, int w0) {
 // ones so that lanes spread over the banks whichever bits are in registers
 __device__ __forceinline__ uint32_t swz(uint32_t l) { return l ^ ((l >> 4) & 15u) ^ ((l >> 8) & 15u); }
 
-__device__ __forceinline__ uint32_t chunk_addr(const BPass& P, uint32_t base, uint32_t l) {
-    return base | P.tab_lo[l & 127] | P.tab_hi[l >> 7];
-}
-
 __device__ __forceinline__ uint32_t chunk_base(uint32_t nonlocal, uint32_t c) {
     uint32_t r = 0, m = nonlocal;
     while (m) {
@@ -157,28 +198,50 @@ __device__ __forceinline__ uint32_t chunk_base(uint32_t nonlocal, uint32_t c) {
     return r;
 }
 
-// chunk transfers between global memory and the shared-memory slice (chunked circuits run on
-// the whole CTA: 512 threads x 16 amplitudes); every load is issued before the first store
-__device__ __noinline__ void chunk_load(const BPass& P, uint32_t base, const float2* __restrict__ g, float2* s,
-                                           int tg) {
-    float2 t[kRegs];
+// Chunk transfers between global memory and the shared-memory slice (the whole CTA: 512 threads x 16
+// amplitudes, local index tg + 512 j). Local bits 0..8 are the thread's, 9..12 are j's, so an address
+// is the thread's part OR j's masks, and a shared-memory position (swz is XOR-linear) the thread's
+// XOR a constant.
+struct ChunkMap {
+    uint32_t off, hm[4], sw;
+    __device__ __forceinline__ ChunkMap(const BPass& P, uint32_t base, int tg) {
+        off = base | P.tab_lo[tg & 127] | P.tab_hi[tg >> 7];
 #pragma unroll
-    for (int j = 0; j < kRegs; j++) t[j] = g[chunk_addr(P, base, uint32_t(tg + j * kBT))];
+        for (int k = 0; k < 4; k++) hm[k] = P.tab_hi[4 << k];
+        sw = swz(uint32_t(tg));
+    }
+    __device__ __forceinline__ uint32_t addr(int j) const {
+        uint32_t o = off;
 #pragma unroll
-    for (int j = 0; j < kRegs; j++) s[uint32_t(tg + j * kBT) ^ ((uint32_t(tg + j * kBT) >> 4) & 15u) ^
-                                      ((uint32_t(tg + j * kBT) >> 8) & 15u)] = t[j];
-}
-__device__ __noinline__ void chunk_store(const BPass& P, uint32_t base, float2* __restrict__ g, const float2* s,
-                                            int tg) {
-    float2 t[kRegs];
+        for (int k = 0; k < 4; k++)
+            if ((j >> k) & 1) o |= hm[k];
+        return o;
+    }
+    __device__ __forceinline__ uint32_t pos(int j) const { return sw ^ uint32_t((j << 9) ^ ((2 * j) & 15)); }
+};
+// every load is issued before the first store
+template <bool kBoth>
+__device__ __noinline__ void chunk_load(const ChunkMap m, const float2* __restrict__ g, const float2* __restrict__ h,
+                                           float2* s, float2* t) {
+    float2 v[kRegs], u[kRegs];
 #pragma unroll
-    for (int j = 0; j < kRegs; j++) {
-        const uint32_t l = uint32_t(tg + j * kBT);
-        t[j] = s[l ^ ((l >> 4) & 15u) ^ ((l >> 8) & 15u)];
+    for (int j = 0; j < kRegs; j++) v[j] = __ldcg(g + m.addr(j));
+    if (kBoth) {
+#pragma unroll
+        for (int j = 0; j < kRegs; j++) u[j] = __ldcg(h + m.addr(j));
     }
 #pragma unroll
-    for (int j = 0; j < kRegs; j++) g[chunk_addr(P, base, uint32_t(tg + j * kBT))] = t[j];
+    for (int j = 0; j < kRegs; j++) s[m.pos(j)] = v[j];
+    if (kBoth) {
+#pragma unroll
+        for (int j = 0; j < kRegs; j++) t[m.pos(j)] = u[j];
+    }
 }
+__device__ __noinline__ void chunk_store(const ChunkMap m, float2* __restrict__ g, const float2* s) {
+#pragma unroll
+    for (int j = 0; j < kRegs; j++) __stcg(g + m.addr(j), s[m.pos(j)]);
+}
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // |0...0> restricted to a chunk: amplitude 1 at local index 0 of the chunk with base 0
 __device__ __forceinline__ void sp_init(float2* s, uint32_t l, uint32_t base) {
@@ -189,115 +252,55 @@ __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
 
-// 2x2 complex matrix of a non-diagonal single-qubit gate (or of its adjoint)
-struct M2 {
-    float2 m00, m01, m10, m11;
-};
-__device__ __forceinline__ M2 gate_m2(uint8_t kind, float c, float sn) {
-    M2 m;
-    switch (kind) {
-        case BK_RX:  // [[c, i s], [i s, c]]
-            m.m00 = make_float2(c, 0.f); m.m01 = make_float2(0.f, sn);
-            m.m10 = make_float2(0.f, sn); m.m11 = make_float2(c, 0.f);
-            break;
-        case BK_RY:  // [[c, s], [-s, c]]
-            m.m00 = make_float2(c, 0.f); m.m01 = make_float2(sn, 0.f);
-            m.m10 = make_float2(-sn, 0.f); m.m11 = make_float2(c, 0.f);
-            break;
-        case BK_H: {
+// Rotations on register bit J. The two parts of an amplitude share the real factors, so the updates
+// run on packed FP32 pairs (each lane rounds as the scalar instruction).
+// RY = [[c, s], [-s, c]]
+template <int J>
+__device__ __forceinline__ void pairs_ry(float2 (&v)[kRegs], float c, float sn) {
+    const float2 c2 = make_float2(c, c), s2 = make_float2(sn, sn), m2 = make_float2(-sn, -sn);
+#pragma unroll
+    for (int r = 0; r < kRegs; r++) {
+        if ((r >> J) & 1) continue;
+        const int r1 = r | (1 << J);
+        const float2 u = v[r], w = v[r1];
+        v[r] = __ffma2_rn(c2, u, __fmul2_rn(s2, w));
+        v[r1] = __ffma2_rn(c2, w, __fmul2_rn(m2, u));
+    }
+}
+// RX = [[c, i s], [i s, c]]
+template <int J>
+__device__ __forceinline__ void pairs_rx(float2 (&v)[kRegs], float c, float sn) {
+    const float2 c2 = make_float2(c, c), s2 = make_float2(-sn, sn);
+#pragma unroll
+    for (int r = 0; r < kRegs; r++) {
+        if ((r >> J) & 1) continue;
+        const int r1 = r | (1 << J);
+        const float2 u = v[r], w = v[r1];
+        v[r] = __ffma2_rn(c2, u, __fmul2_rn(s2, make_float2(w.y, w.x)));
+        v[r1] = __ffma2_rn(c2, w, __fmul2_rn(s2, make_float2(u.y, u.x)));
+    }
+}
+// H, X, Y (their own adjoints)
+template <int J>
+__device__ __forceinline__ void pairs_fixed(float2 (&v)[kRegs], uint8_t kind) {
+#pragma unroll
+    for (int r = 0; r < kRegs; r++) {
+        if ((r >> J) & 1) continue;
+        const int r1 = r | (1 << J);
+        const float2 u = v[r], w = v[r1];
+        if (kind == BK_H) {
             const float h = 0.70710678118654752f;
-            m.m00 = make_float2(h, 0.f); m.m01 = make_float2(h, 0.f);
-            m.m10 = make_float2(h, 0.f); m.m11 = make_float2(-h, 0.f);
-            break;
+            v[r] = make_float2(fmaf(h, w.x, h * u.x), fmaf(h, w.y, h * u.y));
+            v[r1] = make_float2(fmaf(-h, w.x, h * u.x), fmaf(-h, w.y, h * u.y));
+        } else if (kind == BK_X) {
+            v[r] = w;
+            v[r1] = u;
+        } else {  // Y = [[0, -i], [i, 0]]
+            v[r] = make_float2(w.y, -w.x);
+            v[r1] = make_float2(-u.y, u.x);
         }
-        case BK_X:
-            m.m00 = make_float2(0.f, 0.f); m.m01 = make_float2(1.f, 0.f);
-            m.m10 = make_float2(1.f, 0.f); m.m11 = make_float2(0.f, 0.f);
-            break;
-        default:  // Y = [[0, -i], [i, 0]]
-            m.m00 = make_float2(0.f, 0.f); m.m01 = make_float2(0.f, -1.f);
-            m.m10 = make_float2(0.f, 1.f); m.m11 = make_float2(0.f, 0.f);
-            break;
-    }
-    return m;
-}
-
-__device__ __forceinline__ float2 cfma2(float2 a, float2 b, float2 acc) {
-    acc.x = fmaf(a.x, b.x, acc.x);
-    acc.x = fmaf(-a.y, b.y, acc.x);
-    acc.y = fmaf(a.x, b.y, acc.y);
-    acc.y = fmaf(a.y, b.x, acc.y);
-    return acc;
-}
-
-// 2x2 update of the register pairs (r, r | 2^J) by a general complex matrix (H, X, Y)
-template <int J>
-__device__ __forceinline__ void pairs_1q(float2 (&v)[kRegs], int R, const M2& m) {
-#pragma unroll
-    for (int r = 0; r < kRegs; r++) {
-        if ((r >> J) & 1) continue;
-        const int r1 = r | (1 << J);
-        const float2 u = v[r], w = v[r1];
-        v[r] = cfma2(m.m01, w, cfma2(m.m00, u, make_float2(0.f, 0.f)));
-        v[r1] = cfma2(m.m11, w, cfma2(m.m10, u, make_float2(0.f, 0.f)));
     }
 }
-
-// RY = [[c, s], [-s, c]] (real): 8 FMA per pair
-template <int J>
-__device__ __forceinline__ void pairs_ry(float2 (&v)[kRegs], int R, float c, float sn) {
-#pragma unroll
-    for (int r = 0; r < kRegs; r++) {
-        if ((r >> J) & 1) continue;
-        const int r1 = r | (1 << J);
-        const float2 u = v[r], w = v[r1];
-        v[r] = make_float2(fmaf(c, u.x, sn * w.x), fmaf(c, u.y, sn * w.y));
-        v[r1] = make_float2(fmaf(c, w.x, -sn * u.x), fmaf(c, w.y, -sn * u.y));
-    }
-}
-
-// RX = [[c, i s], [i s, c]]: 8 FMA per pair
-template <int J>
-__device__ __forceinline__ void pairs_rx(float2 (&v)[kRegs], int R, float c, float sn) {
-#pragma unroll
-    for (int r = 0; r < kRegs; r++) {
-        if ((r >> J) & 1) continue;
-        const int r1 = r | (1 << J);
-        const float2 u = v[r], w = v[r1];
-        v[r] = make_float2(fmaf(c, u.x, -sn * w.y), fmaf(c, u.y, sn * w.x));
-        v[r1] = make_float2(fmaf(c, w.x, -sn * u.y), fmaf(c, w.y, sn * u.x));
-    }
-}
-
-template <int J>
-__device__ __forceinline__ void pairs_kind(float2 (&v)[kRegs], int R, uint8_t kind, float c, float sn) {
-    if (kind == BK_RY) pairs_ry<J>(v, R, c, sn);
-    else if (kind == BK_RX) pairs_rx<J>(v, R, c, sn);
-    else pairs_1q<J>(v, R, gate_m2(kind, c, sn));
-}
-
-// which of the 16 registers have local bit `bit` set: a fixed pattern when the bit is one of the
-// register bits (position j), else all or none according to the thread's base
-__device__ __forceinline__ uint32_t reg_mask(uint8_t j, uint32_t base, uint8_t bit) {
-    const uint32_t pat[kRegBits] = {0xAAAAu, 0xCCCCu, 0xF0F0u, 0xFF00u};
-    if (j != kNoReg) return pat[j & 3];
-    return ((base >> bit) & 1u) ? 0xFFFFu : 0u;
-}
-
-// local index of register r of this thread: the thread's base (its bits outside the register
-// sub-cube) plus the active bits selected by r
-struct LocalMap {
-    uint32_t base;
-    uint32_t am[kRegBits];
-    __device__ __forceinline__ uint32_t at(int r) const {
-        uint32_t o = base;
-#pragma unroll
-        for (int j = 0; j < kRegBits; j++)
-            if ((r >> j) & 1) o |= am[j];
-        return o;
-    }
-};
-
 template <int J>
 __device__ __forceinline__ void pairs_cnot(float2 (&v)[kRegs], uint32_t cmask) {
 #pragma unroll
@@ -311,59 +314,62 @@ __device__ __forceinline__ void pairs_cnot(float2 (&v)[kRegs], uint32_t cmask) {
         }
     }
 }
+template <int J>
+__device__ __forceinline__ void pairs_kind(float2 (&v)[kRegs], const BOp& o, uint32_t cmask) {
+    if (o.kind == BK_CNOT) pairs_cnot<J>(v, cmask);
+    else pairs_fixed<J>(v, o.kind);
+}
 
-// apply g (or its adjoint) to the registers
-__device__ __forceinline__ void apply_reg(float2 (&v)[kRegs], const LocalMap& li, int R, const BGate& g,
-                                          float2 cs, bool adjoint) {
-    const float c = cs.x, sn = adjoint ? -cs.y : cs.y;
-    switch (g.kind) {
-        case BK_RZ: {  // diag(c + i s, c - i s)
-            const uint32_t m = reg_mask(g.ja, li.base, g.a);
-#pragma unroll
-            for (int r = 0; r < kRegs; r++) v[r] = cmulf(make_float2(c, ((m >> r) & 1u) ? -sn : sn), v[r]);
-            break;
-        }
-        case BK_Z: {
-            const uint32_t m = reg_mask(g.ja, li.base, g.a);
-#pragma unroll
-            for (int r = 0; r < kRegs; r++)
-                if ((m >> r) & 1u) v[r] = make_float2(-v[r].x, -v[r].y);
-            break;
-        }
-        case BK_CZ: {
-            const uint32_t m = reg_mask(g.ja, li.base, g.a) & reg_mask(g.jb, li.base, g.b);
-#pragma unroll
-            for (int r = 0; r < kRegs; r++)
-                if ((m >> r) & 1u) v[r] = make_float2(-v[r].x, -v[r].y);
-            break;
-        }
-        case BK_CNOT: {
-            const uint32_t m = reg_mask(g.jb, li.base, g.b);
-            switch (g.ja) {
-                case 0: pairs_cnot<0>(v, m); break;
-                case 1: pairs_cnot<1>(v, m); break;
-                case 2: pairs_cnot<2>(v, m); break;
-                default: pairs_cnot<3>(v, m); break;
-            }
-            break;
-        }
-        default:
-            switch (g.ja) {
-                case 0: pairs_kind<0>(v, R, g.kind, c, sn); break;
-                case 1: pairs_kind<1>(v, R, g.kind, c, sn); break;
-                case 2: pairs_kind<2>(v, R, g.kind, c, sn); break;
-                default: pairs_kind<3>(v, R, g.kind, c, sn); break;
-            }
-            break;
+// register indices with register bit j set
+__device__ __forceinline__ uint32_t reg_pattern(int j) {
+    return j == 0 ? 0xAAAAu : j == 1 ? 0xCCCCu : j == 2 ? 0xF0F0u : 0xFF00u;
+}
+
+// H, X, Y and CNOT (their own adjoints)
+__device__ __forceinline__ void apply_fixed(float2 (&v)[kRegs], uint32_t base, const BOp& o) {
+    uint32_t cmask = 0;
+    if (o.kind == BK_CNOT) cmask = o.jb != kNoReg ? reg_pattern(o.jb) : ((base >> o.b) & 1u) ? 0xFFFFu : 0u;
+    switch (o.j) {
+        case 0: pairs_kind<0>(v, o, cmask); break;
+        case 1: pairs_kind<1>(v, o, cmask); break;
+        case 2: pairs_kind<2>(v, o, cmask); break;
+        default: pairs_kind<3>(v, o, cmask); break;
     }
 }
 
-// Im sum conj(lam) (P psi) over this thread's registers, P the axis of rotation g. The thread's
-// partial (at most 32 products of complex64 data) is an FP32 FMA chain; the sums across threads,
-// warps and chunks are FP64.
+// RZ on register bit J (diag(c + i s, c - i s); the adjoint has -s) or, J == kRegBits, on a bit that
+// is the same for all of the thread's registers (s signed by it)
 template <int J>
-__device__ __forceinline__ void grad_pairs(const float2 (&p)[kRegs], const float2 (&l)[kRegs], int R, uint8_t kind,
-                                           float& im) {
+__device__ __forceinline__ void phases_rz(float2 (&v)[kRegs], float c, float sn) {
+#pragma unroll
+    for (int r = 0; r < kRegs; r++) {
+        const float s = (J < kRegBits && ((r >> J) & 1)) ? -sn : sn;
+        v[r] = cmulf(make_float2(c, s), v[r]);
+    }
+}
+// bit r: the sign of register index r under a run of sign gates
+__device__ __forceinline__ uint32_t run_signs(const BatchDev& B, const BSign& D, uint32_t base) {
+    uint32_t par = __popc(base & D.zbase);
+    for (int k = 0; k < D.ncz; k++) {
+        const BCz z = B.czs[D.cz0 + k];
+        par ^= __popc(base & (base >> z.shift) & z.mask);
+    }
+    uint32_t m = D.pat ^ ((par & 1u) ? 0xFFFFu : 0u);
+#pragma unroll
+    for (int j = 0; j < kRegBits; j++) m ^= (__popc(base & D.nbr[j]) & 1) ? reg_pattern(j) : 0u;
+    return m;
+}
+__device__ __forceinline__ float2 flip_if(float2 v, uint32_t sign, int r) {
+    const uint32_t m = (sign << (31 - r)) & 0x80000000u;
+    return make_float2(__uint_as_float(__float_as_uint(v.x) ^ m), __uint_as_float(__float_as_uint(v.y) ^ m));
+}
+
+// Im sum conj(lam) (P psi) over this thread's registers, P the axis of rotation o. The thread's
+// partial (at most 32 products of complex64 data) is an FP32 FMA chain; the sums across warps and
+// chunks are FP64.
+template <int J>
+__device__ __forceinline__ float grad_pairs(const float2 (&p)[kRegs], const float2 (&l)[kRegs], uint8_t kind) {
+    float im = 0.f;
 #pragma unroll
     for (int r = 0; r < kRegs; r++) {
         if ((r >> J) & 1) continue;
@@ -377,48 +383,63 @@ __device__ __forceinline__ void grad_pairs(const float2 (&p)[kRegs], const float
         im = fmaf(lb.x, p1.y, im);
         im = fmaf(-lb.y, p1.x, im);
     }
+    return im;
 }
-
-__device__ __forceinline__ float grad_reg(const float2 (&p)[kRegs], const float2 (&l)[kRegs], const LocalMap& li,
-                                          int R, const BGate& g) {
+// Z on register bit J; J == kRegBits: without the sign, which is the same for all registers
+template <int J>
+__device__ __forceinline__ float grad_z(const float2 (&p)[kRegs], const float2 (&l)[kRegs]) {
     float im = 0.f;
-    if (g.kind == BK_RZ) {  // Z: (a, -b) by the target bit
-        const uint32_t m = reg_mask(g.ja, li.base, g.a);
 #pragma unroll
-        for (int r = 0; r < kRegs; r++) {
-            const float sg = ((m >> r) & 1u) ? -1.f : 1.f;
-            im = fmaf(sg * l[r].x, p[r].y, im);
-            im = fmaf(-sg * l[r].y, p[r].x, im);
-        }
-    } else {
-        switch (g.ja) {
-            case 0: grad_pairs<0>(p, l, R, g.kind, im); break;
-            case 1: grad_pairs<1>(p, l, R, g.kind, im); break;
-            case 2: grad_pairs<2>(p, l, R, g.kind, im); break;
-            default: grad_pairs<3>(p, l, R, g.kind, im); break;
-        }
+    for (int r = 0; r < kRegs; r++) {
+        const bool neg = J < kRegBits && ((r >> J) & 1);
+        im = fmaf(neg ? -l[r].x : l[r].x, p[r].y, im);
+        im = fmaf(neg ? l[r].y : -l[r].y, p[r].x, im);
     }
     return im;
 }
-
-// local-index map of thread tg in stage S of a window of nl local bits
-__device__ __forceinline__ LocalMap stage_map(const BStage& S, int nl, int tg) {
-    LocalMap m;
-    uint32_t actmask = 0;
-#pragma unroll
-    for (int j = 0; j < kRegBits; j++) {
-        m.am[j] = j < S.nact ? (1u << S.act[j]) : 0u;
-        actmask |= m.am[j];
-    }
-    uint32_t base = 0, t = uint32_t(tg);
-    for (int b = 0; b < nl; b++) {
-        if ((actmask >> b) & 1) continue;
-        if (t & 1u) base |= 1u << b;
-        t >>= 1;
-    }
-    m.base = base;
-    return m;
+// One rotation (its code without the gradient flag): un-applied or applied
+template <int kCode>
+__device__ __forceinline__ void rotate(float2 (&v)[kRegs], float c, float sn, uint32_t bit) {
+    if constexpr (kCode < kCodeRY) pairs_rx<kCode>(v, c, sn);
+    else if constexpr (kCode < kCodeRZ) pairs_ry<kCode - kCodeRY>(v, c, sn);
+    else if constexpr (kCode < kCodeRZ + kRegBits) phases_rz<kCode - kCodeRZ>(v, c, sn);
+    else phases_rz<kRegBits>(v, c, bit ? -sn : sn);
 }
+template <int kCode>
+__device__ __forceinline__ float rotation_grad(const float2 (&p)[kRegs], const float2 (&l)[kRegs], uint32_t bit) {
+    if constexpr (kCode < kCodeRY) return grad_pairs<kCode>(p, l, BK_RX);
+    else if constexpr (kCode < kCodeRZ) return grad_pairs<kCode - kCodeRY>(p, l, BK_RY);
+    else if constexpr (kCode < kCodeRZ + kRegBits) return grad_z<kCode - kCodeRZ>(p, l);
+    else {
+        const float g = grad_z<kRegBits>(p, l);
+        return bit ? -g : g;
+    }
+}
+
+// Thread tg of a stage holds the 16 amplitudes of the register sub-cube at `base` (its bits spread
+// over the local bits outside act, ascending). The shared-memory positions are XOR-linear in the
+// index: one XOR per register from the stage's four masks (in bytes).
+struct StageMap {
+    uint32_t base, a0, am[kRegBits];
+    __device__ __forceinline__ StageMap(const BStage& S, int tg) {
+        uint32_t t = uint32_t(tg);
+#pragma unroll
+        for (int j = 0; j < kRegBits; j++) {
+            const uint32_t lo = t & ((1u << S.sorted[j]) - 1u);
+            t = ((t ^ lo) << 1) | lo;
+            am[j] = swz(1u << S.act[j]) * uint32_t(sizeof(float2));
+        }
+        base = t;
+        a0 = swz(t) * uint32_t(sizeof(float2));
+    }
+    __device__ __forceinline__ float2* at(float2* s, int r) const {
+        uint32_t o = a0;
+#pragma unroll
+        for (int j = 0; j < kRegBits; j++)
+            if ((r >> j) & 1) o ^= am[j];
+        return reinterpret_cast<float2*>(reinterpret_cast<unsigned char*>(s) + o);
+    }
+};
 
 __device__ __forceinline__ float warp_sum_f(float v) {
 #pragma unroll
@@ -433,81 +454,123 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // ---------------------------------------------------------------- stage bodies
+// where a pass's steps are read from: shared memory for a chunked pass that fits, else global
+struct StepSource {
+    const BOp* ops;
+    const BSign* signs;
+};
 // forward: registers <- slice, gates, slice <- registers
-__device__ __forceinline__ void stage_forward(const BatchDev& B, const BStage& S, int nl, int tg, int T, float2* sp) {
+__device__ __forceinline__ void stage_forward(const BatchDev& B, const BStage& S, StepSource src, int tg, int T,
+                                              float2* sp) {
     if (tg >= T) return;
-    const LocalMap li = stage_map(S, nl, tg);
+    const StageMap m(S, tg);
     float2 v[kRegs];
 #pragma unroll
-    for (int r = 0; r < kRegs; r++) v[r] = sp[swz(li.at(r))];
-    BGate g = B.gates[S.g0];
-    for (int gi = S.g0; gi < S.g1; gi++) {
-        const BGate gn = gi + 1 < S.g1 ? B.gates[gi + 1] : g;  // prefetch
-        apply_reg(v, li, kRegs, g, make_float2(g.c, g.s), false);
-        g = gn;
+    for (int r = 0; r < kRegs; r++) v[r] = *m.at(sp, r);
+    BOp o = src.ops[S.o0];
+    for (int i = S.o0; i < S.o1; i++) {
+        const BOp next = i + 1 < S.o1 ? src.ops[i + 1] : o;  // prefetch
+        const float c = o.cs.x, sn = o.cs.y;
+        const uint32_t bit = (m.base >> (o.b & 31)) & 1u;
+        switch (o.code & 15) {
+#define QS_ROT(k) \
+    case k: rotate<k>(v, c, sn, bit); break;
+            QS_ROT(0) QS_ROT(1) QS_ROT(2) QS_ROT(3) QS_ROT(4) QS_ROT(5) QS_ROT(6) QS_ROT(7)
+            QS_ROT(8) QS_ROT(9) QS_ROT(10) QS_ROT(11) QS_ROT(12)
+#undef QS_ROT
+            case kCodeSign: {
+                const uint32_t sign = run_signs(B, src.signs[__float_as_int(c)], m.base);
+#pragma unroll
+                for (int r = 0; r < kRegs; r++) v[r] = flip_if(v[r], sign, r);
+                break;
+            }
+            default: apply_fixed(v, m.base, o); break;
+        }
+        o = next;
     }
 #pragma unroll
-    for (int r = 0; r < kRegs; r++) sp[swz(li.at(r))] = v[r];
+    for (int r = 0; r < kRegs; r++) *m.at(sp, r) = v[r];
 }
 
-// reverse: gradient partials of the stage's rotations into red[slot][warp], un-apply from psi
-// and lambda. Every lane reaches the warp reductions; lanes beyond T hold no amplitudes.
-__device__ __forceinline__ void stage_reverse(const BatchDev& B, const BStage& S, int nl, int tg, int T, float2* sp,
-                                              float2* sl, double (*red)[kWarps], int warp, int lane) {
-    const bool active = tg < T;
-    LocalMap li;
+// reverse: gradient rows of the stage into red[row][warp], un-apply from psi and lambda. Every lane
+// reaches the warp sums; lanes beyond T (never with kFull) hold zeros and store nothing.
+template <bool kFull>
+__device__ __forceinline__ void stage_reverse(const BatchDev& B, const BStage& S, StepSource src, int tg, int T,
+                                              float2* sp, float2* sl, float (*red)[kWarps], int warp, int lane) {
+    const bool active = kFull || tg < T;
+    const StageMap m(S, tg);
     float2 v[kRegs], u[kRegs];
+#pragma unroll
+    for (int r = 0; r < kRegs; r++) {
+        v[r] = active ? *m.at(sp, r) : make_float2(0.f, 0.f);
+        u[r] = active ? *m.at(sl, r) : make_float2(0.f, 0.f);
+    }
+    // One body per rotation: its gradient's FMA chain, both un-applications and the warp sum of the
+    // rotation before it (held back one step) are independent, so that their latencies overlap.
+    float held = 0.f;
+    int held_row = -1;
+    BOp o = src.ops[S.o1 - 1];
+    for (int i = S.o1 - 1; i >= S.o0; i--) {
+        const BOp next = i > S.o0 ? src.ops[i - 1] : o;  // prefetch
+        const float c = o.cs.x, sn = -o.cs.y;
+        const uint32_t bit = (m.base >> (o.b & 31)) & 1u;
+        switch (o.code) {
+#define QS_ROT(k)                                              \
+    case k:                                                    \
+        rotate<k>(v, c, sn, bit);                              \
+        rotate<k>(u, c, sn, bit);                              \
+        break;                                                 \
+    case kCodeGrad + k: {                                      \
+        const float sum = warp_sum_f(held);                    \
+        held = rotation_grad<k>(v, u, bit);                    \
+        rotate<k>(v, c, sn, bit);                              \
+        rotate<k>(u, c, sn, bit);                              \
+        if (lane == 0 && held_row >= 0) red[held_row][warp] = sum; \
+        held_row = o.ref;                                      \
+        break;                                                 \
+    }
+            QS_ROT(0) QS_ROT(1) QS_ROT(2) QS_ROT(3) QS_ROT(4) QS_ROT(5) QS_ROT(6) QS_ROT(7)
+            QS_ROT(8) QS_ROT(9) QS_ROT(10) QS_ROT(11) QS_ROT(12)
+#undef QS_ROT
+            case kCodeSign: {
+                const uint32_t sign = run_signs(B, src.signs[__float_as_int(c)], m.base);
+#pragma unroll
+                for (int r = 0; r < kRegs; r++) {
+                    v[r] = flip_if(v[r], sign, r);
+                    u[r] = flip_if(u[r], sign, r);
+                }
+                break;
+            }
+            default:
+                apply_fixed(v, m.base, o);
+                apply_fixed(u, m.base, o);
+                break;
+        }
+        o = next;
+    }
+    if (held_row >= 0) {
+        const float sum = warp_sum_f(held);
+        if (lane == 0) red[held_row][warp] = sum;
+    }
     if (active) {
-        li = stage_map(S, nl, tg);
 #pragma unroll
         for (int r = 0; r < kRegs; r++) {
-            v[r] = sp[swz(li.at(r))];
-            u[r] = sl[swz(li.at(r))];
-        }
-    }
-    int slot = 0;
-    BGate g = B.gates[S.g1 - 1];
-    for (int gi = S.g1 - 1; gi >= S.g0; gi--) {
-        const BGate gn = gi > S.g0 ? B.gates[gi - 1] : g;  // prefetch
-        const float2 c2 = make_float2(g.c, g.s);
-        if (g.grad >= 0) {
-            // lane partials (<= 32 FP32 products) summed in FP32 across the warp, then FP64
-            const float gw = warp_sum_f(active ? grad_reg(v, u, li, kRegs, g) : 0.f);
-            if (lane == 0) red[slot][warp] = double(gw);
-            slot++;
-        }
-        if (active) {
-            apply_reg(v, li, kRegs, g, c2, true);
-            apply_reg(u, li, kRegs, g, c2, true);
-        }
-        g = gn;
-    }
-    if (active) {
-#pragma unroll
-        for (int r = 0; r < kRegs; r++) {
-            sp[swz(li.at(r))] = v[r];
-            sl[swz(li.at(r))] = u[r];
+            *m.at(sp, r) = v[r];
+            *m.at(sl, r) = u[r];
         }
     }
 }
 
-// after the stage barrier: thread tg < S.nparam owns the tg-th rotation of the stage (reverse
-// order); returns its gradient index and the sum of the warps' partials (fixed order)
-__device__ __forceinline__ int stage_param(const BatchDev& B, const BStage& S, int tg, const double (*red)[kWarps],
-                                           int w0, int G, double* sum) {
-    if (tg >= S.nparam) return -1;
-    int slot = 0, gidx = -1;
-    for (int gi = S.g1 - 1; gi >= S.g0; gi--) {
-        const int gr = B.gates[gi].grad;
-        if (gr >= 0) {
-            if (slot == tg) { gidx = gr; break; }
-            slot++;
-        }
+// after the stage barrier: row k's sum over the group's G warps (FP64, a fixed tree) by warp k mod G of
+// the group, dE/dtheta = -Im <lambda|P|psi> added to out[stride * parameter] (each address belongs to
+// this group; a reduction without a return value does not stall the warp)
+__device__ __forceinline__ void row_sums(const int32_t* params, int np, const float (*red)[kWarps], int w0, int G,
+                                         int warp, int lane, double* out, size_t stride) {
+    for (int k = warp - w0; k < np; k += G) {
+        double v = lane < G ? double(red[k][w0 + lane]) : 0.0;
+        for (int o = G / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) atomicAdd(out + stride * size_t(params[k]), -v);
     }
-    double v = 0.0;
-    for (int w = w0; w < w0 + G; w++) v += red[tg][w];
-    *sum = v;
-    return gidx;
 }
 
 // lambda_y = sum_t coef i^{#Y} s(y ^ f) psi_{y ^ f} for y in [y0, y1) (stride nthr), and this
@@ -577,87 +640,130 @@ __device__ bool grid_barrier(unsigned int* count, unsigned int* gen, int* err, l
     return s_ok != 0;
 }
 
+// a claimed unit of a level (kind < 0: none left)
+struct BUnit {
+    int32_t kind, item, pass, n, first;
+    uint32_t c;
+    uint64_t ws;
+};
+__device__ __noinline__ void claim_unit(const BatchDev& B, int lv, int total, BUnit& out) {
+    const int u = int(atomicAdd(&B.counters[kClasses + lv], 1u));
+    if (u >= total) {
+        out.kind = -1;
+        return;
+    }
+    const int pair = B.lev_pair0[lv];
+    const LevelEntry E = B.lev_entries[pair < 0 ? ~pair + u : B.lev_pairs[pair + (u >> 1)]];
+    out.kind = E.kind;
+    out.item = E.item;
+    out.pass = E.pass;
+    out.n = E.n;
+    out.first = E.first;
+    out.c = uint32_t(u - E.unit0);
+    out.ws = E.ws;
+}
+// a chunk that the next unit reads, into L2: one 128-byte line (16 amplitudes) per thread and buffer
+__device__ __forceinline__ void prefetch_unit(const BatchDev& B, const BUnit& U, int tg) {
+    if (U.kind < 0 || U.first) return;
+    const BPass& P = B.passes[U.pass];
+    const uint32_t l = uint32_t(tg) * 16u;
+    const float2* p = B.ws + U.ws + (chunk_base(P.nonlocal, U.c) | P.tab_lo[l & 127] | P.tab_hi[l >> 7]);
+    prefetch_l2(p);
+    if (U.kind == LV_REV) prefetch_l2(p + (uint64_t(1) << U.n));
+}
+__device__ __forceinline__ void copy_words(void* dst, const void* src, int words, int tg) {
+    for (int i = tg; i < words; i += kBT) static_cast<uint32_t*>(dst)[i] = static_cast<const uint32_t*>(src)[i];
+}
+
 __global__ void __launch_bounds__(kBT, 1) k_batch(const BatchDev B) {
     extern __shared__ __align__(16) unsigned char smem[];
     float2* smem_p = reinterpret_cast<float2*>(smem);
     float2* smem_l = smem_p + kChunk;
-    __shared__ double red[2][kMaxStageParams][kWarps];  // gradient partials per stage parity
+    __shared__ float red[2][kMaxStageRows][kWarps];  // gradient partials per stage parity
     __shared__ double redE[kWarps];
     __shared__ int s_claim[kWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    __shared__ BUnit s_unit[2];
+    __shared__ __align__(16) BOp s_ops[kUnitOps];
+    __shared__ BStage s_stages[kUnitStages];
+    __shared__ BSign s_signs[kUnitSigns];
     int parity = 0;
     bool first_barrier = true;
 
     // ================= circuits wider than the window: level-synchronous over the grid
     for (int lv = 0; lv < B.nlevels; lv++) {
         const int total = B.lev_units[lv];
-        while (true) {
-            if (threadIdx.x == 0) s_claim[0] = int(atomicAdd(&B.counters[kClasses + lv], 1u));
-            __syncthreads();
-            const int u = s_claim[0];
-            __syncthreads();
-            if (u >= total) break;
-            // entry of this unit: last entry with unit0 <= u
-            int lo = B.lev_off[lv], hi = B.lev_off[lv + 1] - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (B.lev_entries[mid].unit0 <= u) lo = mid; else hi = mid - 1;
-            }
-            const LevelEntry E = B.lev_entries[lo];
-            const int item = E.item;
-            const BItem it = B.items[item];
-            const uint32_t c = uint32_t(u - E.unit0);
-            const uint32_t nch = 1u << (it.n - kLocal);
-            float2* gpsi = B.ws + B.ws_off[item];
-            float2* glam = gpsi + (uint64_t(1) << it.n);
+        // units are claimed one ahead: the claim and its look-ups run while the current unit's chunk is
+        // on its way from memory, and the next chunk is fetched into L2 during the current one's gates
+        if (threadIdx.x == 0) claim_unit(B, lv, total, s_unit[0]);
+        __syncthreads();
+        for (int cur = 0; s_unit[cur].kind >= 0; cur ^= 1) {
+            const BUnit E = s_unit[cur];
+            const uint32_t c = E.c;
+            const uint32_t nch = 1u << (E.n - kLocal);
+            float2* gpsi = B.ws + E.ws;
+            float2* glam = gpsi + (uint64_t(1) << E.n);
             const int tg = threadIdx.x;
-            if (E.kind == LV_FWD) {
+            if (E.kind == LV_FWD || E.kind == LV_REV) {
                 const BPass& P = B.passes[E.pass];
-                const uint32_t base = chunk_base(P.nonlocal, c);
-                if (E.pass == it.p0) {
-                    for (uint32_t l = tg; l < kChunk; l += kBT) sp_init(smem_p, l, base);
-                } else {
-                    chunk_load(P, base, gpsi, smem_p, tg);
+                const ChunkMap m(P, chunk_base(P.nonlocal, c), tg);
+                const int ns = P.s1 - P.s0, no = P.o1 - P.o0, ng = P.g1 - P.g0;
+                const bool fits = ns <= kUnitStages && no <= kUnitOps && ng <= kUnitSigns;
+                if (fits) {  // the pass's records, on their way beside the chunk
+                    copy_words(s_stages, B.stages + P.s0, ns * int(sizeof(BStage) / 4), tg);
+                    copy_words(s_ops, B.ops + P.o0, no * int(sizeof(BOp) / 4), tg);
+                    copy_words(s_signs, B.signs + P.g0, ng * int(sizeof(BSign) / 4), tg);
                 }
-                __syncthreads();
-                for (int s = P.s0; s < P.s1; s++) {
-                    stage_forward(B, B.stages[s], kLocal, tg, kBT, smem_p);
+                const BStage* stages = fits ? s_stages - P.s0 : B.stages;
+                const StepSource src{fits ? s_ops - P.o0 : B.ops, fits ? s_signs - P.g0 : B.signs};
+                if (tg == 0) claim_unit(B, lv, total, s_unit[cur ^ 1]);
+                if (E.kind == LV_FWD) {
+                    if (E.first) {
+                        const uint32_t base = chunk_base(P.nonlocal, c);
+                        for (uint32_t l = tg; l < kChunk; l += kBT) sp_init(smem_p, l, base);
+                    } else {
+                        chunk_load<false>(m, gpsi, nullptr, smem_p, nullptr);
+                    }
                     __syncthreads();
+                    prefetch_unit(B, s_unit[cur ^ 1], tg);
+                    for (int s = P.s0; s < P.s1; s++) {
+                        stage_forward(B, stages[s], src, tg, kBT, smem_p);
+                        __syncthreads();
+                    }
+                    chunk_store(m, gpsi, smem_p);
+                } else {
+                    chunk_load<true>(m, gpsi, glam, smem_p, smem_l);
+                    __syncthreads();
+                    prefetch_unit(B, s_unit[cur ^ 1], tg);
+                    double* pg = B.part_g + B.part_g_off[E.item] + c;
+                    for (int s = P.s1 - 1; s >= P.s0; s--) {
+                        const BStage S = stages[s];
+                        stage_reverse<true>(B, S, src, tg, kBT, smem_p, smem_l, red[parity], warp, lane);
+                        __syncthreads();
+                        row_sums(B.params + S.p0, S.np, red[parity], 0, kWarps, warp, lane, pg, nch);
+                        parity ^= 1;
+                    }
+                    chunk_store(m, gpsi, smem_p);
+                    chunk_store(m, glam, smem_l);
                 }
-                chunk_store(P, base, gpsi, smem_p, tg);
                 __syncthreads();
             } else if (E.kind == LV_LAMBDA) {
+                if (tg == 0) claim_unit(B, lv, total, s_unit[cur ^ 1]);
                 const uint32_t y0 = c << kLocal;
-                const double ew = warp_sum(lambda_range<false>(B, it, gpsi, glam, y0, y0 + kChunk, tg, kBT));
+                const double ew = warp_sum(lambda_range<false>(B, B.items[E.item], gpsi, glam, y0, y0 + kChunk, tg, kBT));
                 if (lane == 0) redE[warp] = ew;
                 __syncthreads();
                 if (tg == 0) {
                     double e = 0.0;
                     for (int w = 0; w < kWarps; w++) e += redE[w];
-                    B.part_e[B.part_e_off[item] + c] = e;
+                    B.part_e[B.part_e_off[E.item] + c] = e;
                 }
-                __syncthreads();
-            } else if (E.kind == LV_REV) {
-                const BPass& P = B.passes[E.pass];
-                const uint32_t base = chunk_base(P.nonlocal, c);
-                chunk_load(P, base, gpsi, smem_p, tg);
-                chunk_load(P, base, glam, smem_l, tg);
-                __syncthreads();
-                double* pg = B.part_g + B.part_g_off[item];
-                for (int s = P.s1 - 1; s >= P.s0; s--) {
-                    const BStage S = B.stages[s];
-                    stage_reverse(B, S, kLocal, tg, kBT, smem_p, smem_l, red[parity], warp, lane);
-                    __syncthreads();
-                    double sum;
-                    const int gidx = stage_param(B, S, tg, red[parity], 0, kWarps, &sum);
-                    if (gidx >= 0) pg[size_t(gidx) * nch + c] -= sum;  // dE/dtheta = -Im <lambda|P|psi>
-                    parity ^= 1;
-                }
-                chunk_store(P, base, gpsi, smem_p, tg);
-                chunk_store(P, base, glam, smem_l, tg);
                 __syncthreads();
             } else {  // LV_FINAL: energy and gradients of the item, sums in chunk order
+                const int item = E.item;
+                const BItem it = B.items[item];
                 if (tg == 0) {
+                    claim_unit(B, lv, total, s_unit[cur ^ 1]);
                     double e = 0.0;
                     for (uint32_t k = 0; k < nch; k++) e += B.part_e[B.part_e_off[item] + k];
                     B.energy[item] = e;
@@ -693,15 +799,14 @@ __global__ void __launch_bounds__(kBT, 1) k_batch(const BatchDev B) {
             if (k >= count) break;
             const int item = B.order[B.cls_begin[cls] + k];
             const BItem it = B.items[item];
-            const int nl = it.n;
-            const uint32_t size = 1u << nl;
+            const uint32_t size = 1u << it.n;
             const int T = int(size) / kRegs;
             for (int j = tg; j < it.ngrad; j += nthr) B.grad[it.grad0 + j] = 0.0;
             for (uint32_t l = tg; l < size; l += nthr) sp_init(sp, l, 0u);
             gbar(G, w0);
             const BPass& P = B.passes[it.p0];  // one pass holds the whole circuit
             for (int s = P.s0; s < P.s1; s++) {
-                stage_forward(B, B.stages[s], nl, tg, T, sp);
+                stage_forward(B, B.stages[s], StepSource{B.ops, B.signs}, tg, T, sp);
                 gbar(G, w0);
             }
             {
@@ -717,27 +822,21 @@ __global__ void __launch_bounds__(kBT, 1) k_batch(const BatchDev B) {
             }
             for (int s = P.s1 - 1; s >= P.s0; s--) {
                 const BStage S = B.stages[s];
-                stage_reverse(B, S, nl, tg, T, sp, sl, red[parity], warp, lane);
+                stage_reverse<false>(B, S, StepSource{B.ops, B.signs}, tg, T, sp, sl, red[parity], warp, lane);
                 gbar(G, w0);
-                double sum;
-                const int gidx = stage_param(B, S, tg, red[parity], w0, G, &sum);
-                if (gidx >= 0) B.grad[it.grad0 + gidx] -= sum;
+                row_sums(B.params + S.p0, S.np, red[parity], w0, G, warp, lane, B.grad + it.grad0, 1);
                 parity ^= 1;
             }
         }
     }
 }
 
-// (cos, sin) of theta/2 into every rotation's gate record
-__global__ void k_angles(const double* __restrict__ theta, const int32_t* __restrict__ gate_slot,
-                         BGate* __restrict__ gates, int ng) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ng; i += gridDim.x * blockDim.x) {
-        const int sl = gate_slot[i];
-        if (sl < 0) continue;
+// (cos, sin) of theta/2 of every angle slot into its step
+__global__ void k_angles(const double* __restrict__ theta, const uint32_t* __restrict__ op, BOp* __restrict__ ops, int count) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
         double s, c;
-        sincos(0.5 * theta[sl], &s, &c);
-        gates[i].c = float(c);
-        gates[i].s = float(s);
+        sincos(0.5 * theta[i], &s, &c);
+        ops[op[i]].cs = make_float2(float(c), float(s));
     }
 }
 
@@ -755,8 +854,11 @@ struct qs_batch {
     std::vector<int32_t> order;
     std::vector<qs::BPass> passes;
     std::vector<qs::BStage> stages;
-    std::vector<qs::BGate> gates;
-    std::vector<int32_t> gate_slot;     // emitted gate -> absolute angle slot (or -1)
+    std::vector<qs::BOp> ops;
+    std::vector<qs::BSign> signs;
+    std::vector<qs::BCz> czs;
+    std::vector<int32_t> params;
+    std::vector<uint32_t> angle_op;     // angle slot -> the step it belongs to
     std::vector<qs::BTerm> terms;
     std::vector<int32_t> angle_param;   // angle slot -> parameter index of its circuit (or -1)
     std::vector<double> angle_fixed;    // angle slot -> fixed angle (when not parametric)
@@ -767,7 +869,7 @@ struct qs_batch {
     std::vector<uint64_t> ws_off;       // item -> psi offset (amplitudes)
     std::vector<int64_t> part_e_off, part_g_off;
     std::vector<qs::LevelEntry> lev_entries;
-    std::vector<int32_t> lev_off, lev_units;
+    std::vector<int32_t> lev_units, lev_pair0, lev_pairs;
     uint64_t ws_amps = 0;
     int64_t part_e_total = 0, part_g_total = 0;
     // device buffers
@@ -775,18 +877,21 @@ struct qs_batch {
     void* d_order = nullptr;
     void* d_passes = nullptr;
     void* d_stages = nullptr;
-    void* d_gates = nullptr;
-    void* d_gate_slot = nullptr;
+    void* d_ops = nullptr;
+    void* d_signs = nullptr;
+    void* d_angle_op = nullptr;
+    void* d_czs = nullptr;
+    void* d_params = nullptr;
     void* d_terms = nullptr;
     double* d_theta = nullptr;
     float2* d_ws = nullptr;
-    void* d_ws_off = nullptr;
     double* d_part_e = nullptr;
     void* d_part_e_off = nullptr;
     double* d_part_g = nullptr;
     void* d_part_g_off = nullptr;
     void* d_lev_entries = nullptr;
-    void* d_lev_off = nullptr;
+    void* d_lev_pair0 = nullptr;
+    void* d_lev_pairs = nullptr;
     void* d_lev_units = nullptr;
     unsigned int* d_bar = nullptr;    // count, generation
     int* d_err = nullptr;
@@ -810,6 +915,109 @@ struct qs_batch {
 
 namespace qs {
 namespace {
+
+// The gates of a pass (local bits, circuit order) as stages: a stage takes gates in order until their
+// non-diagonal targets need a fifth register bit, its gradient rows run out or a parameter comes a
+// second time. Z and CZ gates between two gates that are not diagonal become one run of signs at its
+// end: negations are exact and commute with the phases among them.
+void plan_stages(const std::vector<BGate>& gl, const std::vector<int32_t>& slot, int nl, qs_batch& b) {
+    auto diagonal = [](const BGate& g) { return g.kind == BK_RZ || g.kind == BK_Z || g.kind == BK_CZ; };
+    std::vector<int> cur, act, grads;
+    auto close_stage = [&]() {
+        if (cur.empty()) return;
+        for (int q = 0; q < nl && int(act.size()) < kRegBits; q++)
+            if (std::find(act.begin(), act.end(), q) == act.end()) act.push_back(q);
+        BStage st;
+        std::memset(&st, 0, sizeof(st));
+        st.o0 = int(b.ops.size());
+        st.p0 = int(b.params.size());
+        for (int j = 0; j < kRegBits; j++) st.act[j] = st.sorted[j] = uint8_t(act[j]);
+        std::sort(st.sorted, st.sorted + kRegBits);
+        auto regpos = [&](int bit) {
+            const auto f = std::find(act.begin(), act.end(), bit);
+            return f == act.end() ? kNoReg : uint8_t(f - act.begin());
+        };
+        const uint32_t pat[kRegBits] = {0xAAAAu, 0xCCCCu, 0xF0F0u, 0xFF00u};
+        BSign D;
+        std::map<int, uint32_t> pairs;  // distance -> lower bits of the run's CZ pairs outside the registers
+        bool open = false;
+        auto close_run = [&]() {
+            if (!open) return;
+            D.cz0 = int(b.czs.size());
+            for (const auto& pm : pairs)
+                if (pm.second) b.czs.push_back(BCz{uint32_t(pm.first), pm.second});
+            D.ncz = int(b.czs.size()) - D.cz0;
+            pairs.clear();
+            open = false;
+            BOp o;
+            std::memset(&o, 0, sizeof(o));
+            o.kind = BK_SIGN;
+            o.code = kCodeSign;
+            o.ref = -1;
+            const int32_t index = int32_t(b.signs.size());
+            std::memcpy(&o.cs.x, &index, sizeof(index));
+            b.signs.push_back(D);
+            b.ops.push_back(o);
+        };
+        for (int i : cur) {
+            const BGate& g = gl[i];
+            const uint8_t ja = regpos(g.a);
+            if (g.kind == BK_Z || g.kind == BK_CZ) {
+                if (!open) std::memset(&D, 0, sizeof(D));
+                open = true;
+                if (g.kind == BK_Z) {
+                    if (ja != kNoReg) D.pat ^= pat[ja];
+                    else D.zbase ^= 1u << g.a;
+                    continue;
+                }
+                const uint8_t jb = regpos(g.b);
+                if (ja != kNoReg && jb != kNoReg) D.pat ^= pat[ja] & pat[jb];
+                else if (ja != kNoReg) D.nbr[ja] ^= 1u << g.b;
+                else if (jb != kNoReg) D.nbr[jb] ^= 1u << g.a;
+                else pairs[std::abs(int(g.a) - int(g.b))] ^= 1u << std::min(g.a, g.b);
+                continue;
+            }
+            if (g.kind != BK_RZ) close_run();
+            BOp o;
+            std::memset(&o, 0, sizeof(o));
+            o.cs = make_float2(1.f, 0.f);
+            o.kind = g.kind;
+            o.j = ja;
+            o.b = g.kind == BK_CNOT ? g.b : g.a;
+            o.jb = g.kind == BK_CNOT ? regpos(g.b) : kNoReg;
+            o.ref = -1;
+            o.code = uint8_t(g.kind == BK_RX ? kCodeRX + ja : g.kind == BK_RY ? kCodeRY + ja
+                             : g.kind == BK_RZ ? kCodeRZ + (ja == kNoReg ? kRegBits : ja) : kCodeFixed);
+            if (g.grad >= 0) {
+                o.ref = int16_t(int(b.params.size()) - st.p0);
+                o.code |= kCodeGrad;
+                b.params.push_back(g.grad);
+            }
+            if (slot[i] >= 0) b.angle_op[slot[i]] = uint32_t(b.ops.size());
+            b.ops.push_back(o);
+        }
+        close_run();
+        st.o1 = int(b.ops.size());
+        st.np = int(b.params.size()) - st.p0;
+        b.stages.push_back(st);
+        cur.clear();
+        act.clear();
+        grads.clear();
+    };
+    for (size_t i = 0; i < gl.size(); i++) {
+        const BGate& g = gl[i];
+        const bool diag = diagonal(g);
+        const bool have = diag || std::find(act.begin(), act.end(), int(g.a)) != act.end();
+        const bool row = g.grad >= 0;
+        if ((row && int(grads.size()) >= kMaxStageRows) || (!have && int(act.size()) >= kRegBits) ||
+            (row && std::find(grads.begin(), grads.end(), g.grad) != grads.end()))
+            close_stage();
+        if (!diag && std::find(act.begin(), act.end(), int(g.a)) == act.end()) act.push_back(g.a);
+        cur.push_back(int(i));
+        if (row) grads.push_back(g.grad);
+    }
+    close_stage();
+}
 
 // split one circuit into passes over windows of <= kLocal qubits
 void plan_passes(const qs_circuit& c, const std::vector<BGate>& gl, const std::vector<uint32_t>& gmask,
@@ -872,60 +1080,22 @@ void plan_passes(const qs_circuit& c, const std::vector<BGate>& gl, const std::v
             bp.tab_hi[h] = a;
         }
         auto local = [&](int q) { return uint8_t(std::find(lq.begin(), lq.end(), q) - lq.begin()); };
-        // stages: runs of gates whose non-diagonal targets fit a sub-cube of kRegBits local bits
-        // held in registers (diagonal gates act on any bit), at most kMaxStageParams rotations
-        const int nl = int(lq.size());
-        const int na = std::min(kRegBits, nl);
-        bp.s0 = int(b.stages.size());
-        std::vector<BGate> cur;
-        std::vector<int32_t> cur_slot;
-        std::vector<int> act;
-        int nparam = 0;
-        auto close_stage = [&]() {
-            if (cur.empty()) return;
-            for (int q = 0; q < nl && int(act.size()) < na; q++)
-                if (std::find(act.begin(), act.end(), q) == act.end()) act.push_back(q);
-            BStage st;
-            std::memset(&st, 0, sizeof(st));
-            st.g0 = int(b.gates.size());
-            st.nact = na;
-            st.nparam = nparam;
-            for (int j = 0; j < na; j++) st.act[j] = uint8_t(act[j]);
-            auto regpos = [&](int bit) {
-                const auto f = std::find(act.begin(), act.end(), bit);
-                return f == act.end() ? kNoReg : uint8_t(f - act.begin());
-            };
-            for (size_t q = 0; q < cur.size(); q++) {
-                BGate g = cur[q];
-                g.ja = regpos(g.a);
-                g.jb = (g.kind == BK_CZ || g.kind == BK_CNOT) ? regpos(g.b) : kNoReg;
-                b.gates.push_back(g);
-                b.gate_slot.push_back(cur_slot[q]);
-            }
-            st.g1 = int(b.gates.size());
-            b.stages.push_back(st);
-            cur.clear();
-            cur_slot.clear();
-            act.clear();
-            nparam = 0;
-        };
+        std::vector<BGate> pg;
+        std::vector<int32_t> ps;
         for (int gi : p.gates) {
             BGate g = gl[gi];
             g.a = local(g.a);
             if (g.kind == BK_CZ || g.kind == BK_CNOT) g.b = local(g.b);
-            const bool diag = g.kind == BK_RZ || g.kind == BK_Z || g.kind == BK_CZ;
-            const int par = g.grad >= 0 ? 1 : 0;
-            bool fits = nparam + par <= kMaxStageParams;
-            if (!diag && std::find(act.begin(), act.end(), int(g.a)) == act.end() && int(act.size()) >= na)
-                fits = false;
-            if (!fits) close_stage();
-            if (!diag && std::find(act.begin(), act.end(), int(g.a)) == act.end()) act.push_back(g.a);
-            cur.push_back(g);
-            cur_slot.push_back(gslot[gi]);
-            nparam += par;
+            pg.push_back(g);
+            ps.push_back(gslot[gi]);
         }
-        close_stage();
+        bp.s0 = int(b.stages.size());
+        bp.o0 = int(b.ops.size());
+        bp.g0 = int(b.signs.size());
+        plan_stages(pg, ps, int(lq.size()), b);
         bp.s1 = int(b.stages.size());
+        bp.o1 = int(b.ops.size());
+        bp.g1 = int(b.signs.size());
         b.passes.push_back(bp);
     }
     it.p1 = int(b.passes.size());
@@ -935,9 +1105,9 @@ void free_batch(qs_batch* b) {
     if (b->exec) cudaGraphExecDestroy(b->exec);
     if (b->graph) cudaGraphDestroy(b->graph);
     if (b->graph_stream) cudaStreamDestroy(b->graph_stream);
-    void* dev[] = {b->d_items, b->d_order, b->d_passes, b->d_stages, b->d_gates, b->d_gate_slot, b->d_terms,
-                   b->d_theta, b->d_ws, b->d_ws_off, b->d_part_e, b->d_part_e_off, b->d_part_g, b->d_part_g_off,
-                   b->d_lev_entries, b->d_lev_off, b->d_lev_units, b->d_bar, b->d_err, b->d_energy, b->d_grad,
+    void* dev[] = {b->d_items, b->d_order, b->d_passes, b->d_stages, b->d_ops, b->d_signs, b->d_angle_op, b->d_czs, b->d_params, b->d_terms,
+                   b->d_theta, b->d_ws, b->d_part_e, b->d_part_e_off, b->d_part_g, b->d_part_g_off,
+                   b->d_lev_entries, b->d_lev_pair0, b->d_lev_pairs, b->d_lev_units, b->d_bar, b->d_err, b->d_energy, b->d_grad,
                    b->d_counter};
     for (void* p : dev)
         if (p) dev_free(p);
@@ -958,9 +1128,8 @@ void upload(void** d, const std::vector<T>& h) {
 void enqueue(qs_batch* b, cudaStream_t st) {
     QS_TRY_CUDA(cudaMemcpyAsync(b->d_theta, b->h_theta, sizeof(double) * std::max(1, b->total_angles),
                                 cudaMemcpyHostToDevice, st));
-    const int ng = int(b->gates.size());
-    k_angles<<<std::max(1, std::min(1024, (ng + 255) / 256)), 256, 0, st>>>(
-        b->d_theta, static_cast<const int32_t*>(b->d_gate_slot), static_cast<BGate*>(b->d_gates), ng);
+    k_angles<<<std::max(1, std::min(1024, (b->total_angles + 255) / 256)), 256, 0, st>>>(
+        b->d_theta, static_cast<const uint32_t*>(b->d_angle_op), static_cast<BOp*>(b->d_ops), b->total_angles);
     const int nlev = int(b->lev_units.size());
     QS_TRY_CUDA(cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned int) * (kClasses + nlev), st));
     QS_TRY_CUDA(cudaMemsetAsync(b->d_bar, 0, sizeof(unsigned int) * 2, st));
@@ -971,10 +1140,12 @@ void enqueue(qs_batch* b, cudaStream_t st) {
     B.order = static_cast<const int32_t*>(b->d_order);
     B.passes = static_cast<const BPass*>(b->d_passes);
     B.stages = static_cast<const BStage*>(b->d_stages);
-    B.gates = static_cast<const BGate*>(b->d_gates);
+    B.ops = static_cast<const BOp*>(b->d_ops);
+    B.signs = static_cast<const BSign*>(b->d_signs);
+    B.czs = static_cast<const BCz*>(b->d_czs);
+    B.params = static_cast<const int32_t*>(b->d_params);
     B.terms = static_cast<const BTerm*>(b->d_terms);
     B.ws = b->d_ws;
-    B.ws_off = static_cast<const uint64_t*>(b->d_ws_off);
     B.energy = b->d_energy;
     B.grad = b->d_grad;
     B.part_e = b->d_part_e;
@@ -982,7 +1153,8 @@ void enqueue(qs_batch* b, cudaStream_t st) {
     B.part_g = b->d_part_g;
     B.part_g_off = static_cast<const int64_t*>(b->d_part_g_off);
     B.lev_entries = static_cast<const LevelEntry*>(b->d_lev_entries);
-    B.lev_off = static_cast<const int32_t*>(b->d_lev_off);
+    B.lev_pair0 = static_cast<const int32_t*>(b->d_lev_pair0);
+    B.lev_pairs = static_cast<const int32_t*>(b->d_lev_pairs);
     B.lev_units = static_cast<const int32_t*>(b->d_lev_units);
     B.nlevels = nlev;
     B.counters = b->d_counter;
@@ -1074,8 +1246,6 @@ qs_status qs_batch_create(const qs_circuit* circuits, const qs_pauli_obs* observ
             BGate bg;
             std::memset(&bg, 0, sizeof(bg));
             bg.grad = -1;
-            bg.c = 1.f;
-            bg.s = 0.f;
             int32_t aslot = -1;
             bg.a = uint8_t(g.targets[0]);
             uint32_t m = 1u << g.targets[0];
@@ -1121,6 +1291,8 @@ qs_status qs_batch_create(const qs_circuit* circuits, const qs_pauli_obs* observ
             gm.push_back(m);
             gs.push_back(aslot);
         }
+        b->total_angles += slots;
+        b->angle_op.resize(size_t(b->total_angles));
         plan_passes(c, gl, gm, gs, *b, it);
         // observable terms
         QS_REQUIRE(o.n_terms >= 0 && (o.n_terms == 0 || (o.coef && o.x_mask && o.z_mask)), "bad observable");
@@ -1137,7 +1309,6 @@ qs_status qs_batch_create(const qs_circuit* circuits, const qs_pauli_obs* observ
             b->terms.push_back(T);
         }
         it.t1 = int(b->terms.size());
-        b->total_angles += slots;
         b->total_grads += c.n_params;
         param_base += c.n_params;
         const double passes = double(it.p1 - it.p0);
@@ -1194,7 +1365,7 @@ qs_status qs_batch_create(const qs_circuit* circuits, const qs_pauli_obs* observ
     std::stable_sort(wide.begin(), wide.end(), [&](int x, int y) { return cost[x] > cost[y]; });
     auto add_level = [&](int kind, int r) {
         int units = 0;
-        b->lev_off.push_back(int(b->lev_entries.size()));
+        b->lev_pair0.push_back(kind == LV_FINAL ? ~int(b->lev_entries.size()) : int(b->lev_pairs.size()));
         for (int k : wide) {
             const BItem& it = b->items[k];
             const int np_ = it.p1 - it.p0;
@@ -1203,6 +1374,9 @@ qs_status qs_batch_create(const qs_circuit* circuits, const qs_pauli_obs* observ
             e.item = k;
             e.kind = kind;
             e.unit0 = units;
+            e.ws = b->ws_off[k];
+            e.n = it.n;
+            e.first = kind == LV_FWD && r == 0 ? 1 : 0;
             if (kind == LV_FWD) {
                 if (r >= np_) continue;
                 e.pass = it.p0 + r;
@@ -1218,6 +1392,8 @@ qs_status qs_batch_create(const qs_circuit* circuits, const qs_pauli_obs* observ
                 e.pass = -1;
                 units += 1;
             }
+            if (kind != LV_FINAL)  // an even number of units: 2^(n - 13), n > 13
+                b->lev_pairs.insert(b->lev_pairs.end(), size_t(units - e.unit0) / 2, int32_t(b->lev_entries.size()));
             b->lev_entries.push_back(e);
         }
         b->lev_units.push_back(units);
@@ -1227,27 +1403,27 @@ qs_status qs_batch_create(const qs_circuit* circuits, const qs_pauli_obs* observ
         add_level(LV_LAMBDA, 0);
         for (int r = 0; r < maxp; r++) add_level(LV_REV, r);
         add_level(LV_FINAL, 0);
-        b->lev_off.push_back(int(b->lev_entries.size()));
-    } else {
-        b->lev_off.push_back(0);
     }
     try {
         upload(&b->d_items, b->items);
         upload(&b->d_order, b->order);
         upload(&b->d_passes, b->passes);
         upload(&b->d_stages, b->stages);
-        upload(&b->d_gates, b->gates);
-        upload(&b->d_gate_slot, b->gate_slot);
+        upload(&b->d_ops, b->ops);
+        upload(&b->d_signs, b->signs);
+        upload(&b->d_angle_op, b->angle_op);
+        upload(&b->d_czs, b->czs);
+        upload(&b->d_params, b->params);
         upload(&b->d_terms, b->terms);
         QS_TRY_CUDA(dev_malloc(&b->d_theta, sizeof(double) * std::max(1, b->total_angles)));
         QS_TRY_CUDA(dev_malloc(&b->d_ws, sizeof(float2) * std::max<uint64_t>(1, b->ws_amps)));
-        upload(&b->d_ws_off, b->ws_off);
         upload(&b->d_part_e_off, b->part_e_off);
         upload(&b->d_part_g_off, b->part_g_off);
         QS_TRY_CUDA(dev_malloc(&b->d_part_e, sizeof(double) * std::max<int64_t>(1, b->part_e_total)));
         QS_TRY_CUDA(dev_malloc(&b->d_part_g, sizeof(double) * std::max<int64_t>(1, b->part_g_total)));
         upload(&b->d_lev_entries, b->lev_entries);
-        upload(&b->d_lev_off, b->lev_off);
+        upload(&b->d_lev_pair0, b->lev_pair0);
+        upload(&b->d_lev_pairs, b->lev_pairs);
         upload(&b->d_lev_units, b->lev_units);
         QS_TRY_CUDA(dev_malloc(&b->d_bar, sizeof(unsigned int) * 2));
         QS_TRY_CUDA(dev_malloc(&b->d_err, sizeof(int)));
