@@ -229,8 +229,9 @@ qs_status qs_apply_observable_rotation(qs_state* s, const qs_pauli_obs* H, doubl
 qs_status qs_plan_fusion(const qs_circuit* c, int k, qs_fused_circuit** out);
 /* The library keeps the partitions of the last 16 circuit structures it planned (the qubits of
  * each gate, the width): a circuit run again with new angles or matrices is not partitioned
- * again. This forgets them; the next run or plan of any circuit partitions it afresh. The
- * autotuner's per-kernel timings of this GPU are kept. */
+ * again. This forgets them; the next run or plan of any circuit partitions it afresh. It also
+ * gives back the freed device memory that the library's allocation pools keep (at most 256 MiB per
+ * device). The autotuner's per-kernel timings of this GPU are kept. */
 qs_status qs_clear_plan_cache(void);
 /* Number of blocks of a plan and, for block b, its width and targets (ascending) and its
  * FP64 matrix (2^w x 2^w complex, row-major) copied to host memory; any output may be NULL. */

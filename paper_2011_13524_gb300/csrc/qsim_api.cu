@@ -65,18 +65,51 @@ void report_device_errors() {
 }
 
 void* stage_of(qs_state* s) {
-    if (!s->d_stage) QS_TRY_CUDA(dev_malloc(&s->d_stage, kStageBytes));
+    if (!s->d_stage)
+        QS_TRY_CUDA(s->pooled ? dev_malloc_async(&s->d_stage, kStageBytes, s->stream) : dev_malloc(&s->d_stage, kStageBytes));
     return s->d_stage;
 }
 
 void free_state_resources(qs_state* s) {
-    if (s->scratch.d_part) dev_free(s->scratch.d_part);
+    if (s->pooled) {
+        if (s->scratch.d_part) dev_free_async(s->scratch.d_part, s->stream);
+        if (s->d_stage) dev_free_async(s->d_stage, s->stream);
+        if (s->owns && s->data) dev_free_async(s->data, s->stream);
+    } else {
+        if (s->scratch.d_part) dev_free(s->scratch.d_part);
+        if (s->d_stage) dev_free(s->d_stage);
+        if (s->owns && s->data) dev_free(s->data);
+    }
     if (s->scratch.h_out) host_free_pinned(s->scratch.h_out);
-    if (s->d_stage) dev_free(s->d_stage);
-    if (s->owns && s->data) dev_free(s->data);
     s->scratch = Scratch{};
     s->d_stage = nullptr;
     s->data = nullptr;
+}
+
+// A state for the duration of one call (contents undefined). Up to kPooledStateBytes its memory and
+// scratch come from the library's stream-ordered pool: cudaMalloc and cudaFree of a small state cost
+// 0.1 ms each and synchronise the device.
+constexpr size_t kPooledStateBytes = size_t(64) << 20;
+std::unique_ptr<qs_state, void (*)(qs_state*)> scratch_state(int n, qs_dtype dt, cudaStream_t st) {
+    std::unique_ptr<qs_state, void (*)(qs_state*)> s(new qs_state(), [](qs_state* p) {
+        free_state_resources(p);
+        delete p;
+    });
+    s->n = n;
+    s->dt = dt;
+    s->stream = st;
+    s->owns = true;
+    QS_TRY_CUDA(cudaGetDevice(&s->device));
+    const size_t bytes = (size_t(1) << n) * amp_bytes(dt);
+    s->pooled = bytes <= kPooledStateBytes;
+    const cudaError_t e = s->pooled ? dev_malloc_async(&s->data, bytes, st) : dev_malloc(&s->data, bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        s->data = nullptr;
+        throw Error{e == cudaErrorMemoryAllocation ? QS_ERR_OOM : QS_ERR_CUDA,
+                    std::string("state allocation failed: ") + cudaGetErrorString(e)};
+    }
+    return s;
 }
 
 // adjoint of an operator: conjugate transpose (Pauli strings and SWAP are Hermitian)
@@ -258,11 +291,11 @@ WideMats upload_wide(qs_state* s, Arith ar, std::vector<Op>& ops) {
     for (size_t b = 0; b < ops.size(); b++) {
         if (ops[b].kind != OpKind::Dense || ops[b].targets.size() < 4) continue;
         if (ar == Arith::F32 && (ops[b].targets.size() == 5 || ops[b].targets.size() == 6) && tensor_c64x_enabled()) {
-            ops[b] = sort_targets(ops[b]);
+            if (!std::is_sorted(ops[b].targets.begin(), ops[b].targets.end())) ops[b] = sort_targets(ops[b]);
             oz[b] = char(10 + ops[b].targets.size());  // the complex64 form, 15 or 16
         }
         if (ar == Arith::DF && (ops[b].targets.size() == 4 || ops[b].targets.size() == 5) && tensor_c128_enabled()) {
-            ops[b] = sort_targets(ops[b]);
+            if (!std::is_sorted(ops[b].targets.begin(), ops[b].targets.end())) ops[b] = sort_targets(ops[b]);
             oz[b] = char(ops[b].targets.size());
         }
         offs[b] = total;
@@ -290,7 +323,10 @@ WideMats upload_wide(qs_state* s, Arith ar, std::vector<Op>& ops) {
     // the blocks' device forms (sliced for the tensor cores, or encoded entries) are independent:
     // several host threads for long plans
     const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-    const unsigned nth = wide.size() < 8 ? 1u : std::min<unsigned>(std::min(hw, 8u), unsigned(wide.size() / 4));
+    // (a thread costs about 25 us to start, a 64 x 64 real form about 25 us to slice)
+    size_t entries = 0;
+    for (size_t b : wide) entries += ops[b].data.size();
+    const unsigned nth = std::max(1u, std::min<unsigned>(std::min(hw, 8u), unsigned(entries >> 12)));
     if (nth <= 1) {
         for (size_t b : wide) prepare(b);
     } else {
@@ -995,6 +1031,7 @@ qs_status qs_plan_fusion(const qs_circuit* c, int k, qs_fused_circuit** out) {
 qs_status qs_clear_plan_cache(void) {
     API_BEGIN
     clear_partition_cache();
+    trim_pools();
     API_END
 }
 
@@ -1278,29 +1315,16 @@ qs_status qs_adjoint_grad(const qs_circuit* c, const double* theta, const qs_pau
     }
     const std::vector<PauliGroup> groups = group_observable(H, c->n);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    qs_state *psi = nullptr, *lam = nullptr;
-    qs_status rc = qs_create_state(c->n, dt, stream, &psi);
-    if (rc != QS_OK) throw Error{rc, std::string("adjoint: ") + qs_last_error()};
-    rc = qs_create_state(c->n, dt, stream, &lam);
-    if (rc != QS_OK) {
-        qs_destroy_state(psi);
-        throw Error{rc, std::string("adjoint: ") + qs_last_error()};
-    }
-    struct Guard {
-        qs_state *a, *b;
-        ~Guard() {
-            qs_destroy_state(a);
-            qs_destroy_state(b);
-        }
-    } guard{psi, lam};
+    const auto psi_owner = scratch_state(c->n, dt, st), lam_owner = scratch_state(c->n, dt, st);
+    qs_state *psi = psi_owner.get(), *lam = lam_owner.get();
     // both buffers stay in the double-float layout for the whole sweep when that arithmetic
     // is selected (they are scratch states, never seen outside this call)
     if (use_df(psi)) {
         psi->df = 1;
         lam->df = 1;
-        launch_set_basis_arith(psi->data, c->n, Arith::DF, 0, st);
     }
     const Arith ar = arith_of(psi);
+    launch_set_basis_arith(psi->data, c->n, ar, 0, st);
     // The reverse sweep as steps: single-qubit X/Y rotations use the fused reverse step
     // (gradient partials + un-apply in one pass); maximal runs of diagonal gates (CZ, phases,
     // RZ and Z-string rotations, diagonal gates) take one pass for the whole run; other gates

@@ -42,8 +42,29 @@ struct OpenBlock {
     int order = 0;           // creation order (emission order among simultaneous closes)
 };
 
+// out[] (interleaved re, im, D columns) += or = (re + i im) * in[]; real and imaginary factors skip the
+// products by zero
+void row_axpy(double* out, const double* in, double re, double im, int D, bool first) {
+    if (first)
+        for (int j = 0; j < 2 * D; j++) out[j] = 0.0;
+    if (im == 0.0) {
+        for (int j = 0; j < 2 * D; j++) out[j] += re * in[j];
+    } else if (re == 0.0) {
+        for (int j = 0; j < D; j++) {
+            out[2 * j] -= im * in[2 * j + 1];
+            out[2 * j + 1] += im * in[2 * j];
+        }
+    } else {
+        for (int j = 0; j < D; j++) {
+            out[2 * j] += re * in[2 * j] - im * in[2 * j + 1];
+            out[2 * j + 1] += re * in[2 * j + 1] + im * in[2 * j];
+        }
+    }
+}
+
 // Apply dense op d (targets/controls given as positions inside `qubits`) to every column of
-// the 2^w x 2^w row-major matrix M: M <- G M.
+// the 2^w x 2^w row-major matrix M: M <- G M, whole rows at a time (contiguous columns), without the
+// entries of G that are zero and the rows it leaves alone.
 void apply_to_columns(std::vector<cplx>& M, int w, const DenseOp& d, const std::vector<int>& local_t,
                       const std::vector<int>& local_c) {
     const int D = 1 << w;
@@ -55,26 +76,35 @@ void apply_to_columns(std::vector<cplx>& M, int w, const DenseOp& d, const std::
         cmask |= 1ull << local_c[j];
         if (d.cvals[j]) cval |= 1ull << local_c[j];
     }
-    std::vector<uint64_t> off(dm);
+    uint64_t off[1 << QS_MAX_TARGETS];
+    bool keep[1 << QS_MAX_TARGETS];  // the identity's rows
     for (int a = 0; a < dm; a++) {
         uint64_t o = 0;
         for (int j = 0; j < m; j++)
             if ((a >> j) & 1) o |= 1ull << local_t[j];
         off[a] = o;
+        keep[a] = true;
+        for (int b = 0; b < dm; b++) keep[a] = keep[a] && d.mat[size_t(a) * dm + b] == cplx(a == b ? 1.0 : 0.0, 0.0);
     }
-    std::vector<cplx> in(dm), out(dm);
-    for (int col = 0; col < D; col++) {
-        for (int r0 = 0; r0 < D; r0++) {
-            if (uint64_t(r0) & tmask) continue;
-            if ((uint64_t(r0) & cmask) != cval) continue;
-            for (int a = 0; a < dm; a++) in[a] = M[size_t(r0 + off[a]) * D + col];
-            for (int z = 0; z < dm; z++) {
-                cplx acc = 0.0;
-                for (int a = 0; a < dm; a++) acc += d.mat[size_t(z) * dm + a] * in[a];
-                out[z] = acc;
+    double* base = reinterpret_cast<double*>(M.data());
+    std::vector<double> out(size_t(dm) * 2 * D);
+    for (int r0 = 0; r0 < D; r0++) {
+        if (uint64_t(r0) & tmask) continue;
+        if ((uint64_t(r0) & cmask) != cval) continue;
+        for (int z = 0; z < dm; z++) {
+            if (keep[z]) continue;
+            double* o = out.data() + size_t(z) * 2 * D;
+            bool first = true;
+            for (int a = 0; a < dm; a++) {
+                const cplx k = d.mat[size_t(z) * dm + a];
+                if (k == cplx(0.0, 0.0)) continue;
+                row_axpy(o, base + (r0 + off[a]) * 2 * D, k.real(), k.imag(), D, first);
+                first = false;
             }
-            for (int z = 0; z < dm; z++) M[size_t(r0 + off[z]) * D + col] = out[z];
+            if (first) std::fill(o, o + 2 * D, 0.0);
         }
+        for (int z = 0; z < dm; z++)
+            if (!keep[z]) std::copy_n(out.data() + size_t(z) * 2 * D, 2 * D, base + (r0 + off[z]) * 2 * D);
     }
 }
 
@@ -528,7 +558,8 @@ FusionPlan plan_fusion(const qs_circuit* c, int k, const double* theta) {
     size_t work = 0;
     for (const OpenBlock& blk : parts) work += blk.gates.size() << (2 * __builtin_popcountll(blk.mask));
     const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-    const unsigned nth = work < (1u << 16) ? 1u : std::min<unsigned>(std::min(hw, 8u), unsigned(parts.size()));
+    // a thread costs about 25 us to start, a row operation on 2^16 entries about 30 us
+    const unsigned nth = std::max(1u, std::min<unsigned>(std::min(hw, 8u), std::min<unsigned>(unsigned(parts.size()), unsigned(work >> 17))));
     if (nth <= 1) {
         for (size_t i = 0; i < parts.size(); i++) plan.blocks[i] = emit(parts[i], c, theta);
     } else {

@@ -821,6 +821,12 @@ void launch_from_df(void* psi, int n, cudaStream_t st) {
 }
 
 Op sort_targets(const Op& op) {
+    if (std::is_sorted(op.targets.begin(), op.targets.end())) {
+        Op r = op;
+        r.dmat = nullptr;
+        r.dmat_oz = false;
+        return r;
+    }
     const int m = int(op.targets.size());
     std::vector<int> perm(m);
     for (int j = 0; j < m; j++) perm[j] = j;

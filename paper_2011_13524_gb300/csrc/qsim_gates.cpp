@@ -11,6 +11,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <mutex>
 
 #include "qsim_internal.h"
 
@@ -291,15 +292,58 @@ bool injected_failure() {
 }
 }  // namespace
 
+namespace {
+std::mutex g_pool_mu;
+cudaMemPool_t g_pools[kMaxDevices] = {};
+// the current device's pool (nullptr if it cannot be made: the device's default pool serves then)
+cudaMemPool_t device_pool() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pools[dev]) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        uint64_t keep = kPoolKeepBytes;
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        g_pools[dev] = pool;
+    }
+    return g_pools[dev];
+}
+}  // namespace
+
+void trim_pools() {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    for (cudaMemPool_t p : g_pools)
+        if (p) cudaMemPoolTrimTo(p, 0);
+}
+
 cudaError_t dev_malloc_raw(void** p, size_t bytes) {
     if (injected_failure()) return cudaErrorMemoryAllocation;
-    const cudaError_t e = cudaMalloc(p, bytes);
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        trim_pools();
+        e = cudaMalloc(p, bytes);
+    }
     if (e == cudaSuccess) g_alloc_held++;
     return e;
 }
 cudaError_t dev_malloc_async_raw(void** p, size_t bytes, cudaStream_t st) {
     if (injected_failure()) return cudaErrorMemoryAllocation;
-    const cudaError_t e = cudaMallocAsync(p, bytes, st);
+    const cudaMemPool_t pool = device_pool();
+    cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, st) : cudaMallocAsync(p, bytes, st);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        trim_pools();
+        e = cudaMallocAsync(p, bytes, st);
+    }
     if (e == cudaSuccess) g_alloc_held++;
     return e;
 }

@@ -57,6 +57,7 @@ struct qs_state {
     qs_dtype dt = QS_C128;
     void* data = nullptr;
     bool owns = false;
+    bool pooled = false;      // memory and scratch from the stream-ordered pool, freed on `stream`
     cudaStream_t stream = nullptr;
     int device = 0;
     qs::Scratch scratch;
@@ -74,6 +75,11 @@ inline size_t amp_bytes(qs_dtype dt) { return dt == QS_C64 ? 8 : 16; }
 // Every device and pinned-host allocation of the library goes through these: they count the
 // allocations held, and a test hook can make one of them fail as if memory had run out
 // (cudaErrorMemoryAllocation, reported as QS_ERR_OOM), to check that no call leaks on that path.
+// Stream-ordered allocations come from a pool of the library's own per device, which keeps at most
+// kPoolKeepBytes of freed memory; trim_pools() gives that back, and so does an allocation that fails
+// otherwise.
+constexpr uint64_t kPoolKeepBytes = uint64_t(256) << 20;
+void trim_pools();
 cudaError_t dev_malloc_raw(void** p, size_t bytes);
 cudaError_t dev_malloc_async_raw(void** p, size_t bytes, cudaStream_t st);
 cudaError_t host_malloc_pinned_raw(void** p, size_t bytes);

@@ -1438,18 +1438,51 @@ OzDevice& oz_init() {
     return d;
 }
 
-// the real form of K~ (16 x 16 complex): row n = 2z + c_out, column k = 2w + c_in
-double real_form(const std::vector<cplx>& K, int n, int k) {
-    const cplx e = K[size_t(n >> 1) * kOzD + size_t(k >> 1)];
-    if ((n & 1) == 0) return (k & 1) == 0 ? e.real() : -e.imag();
-    return (k & 1) == 0 ? e.imag() : e.real();
-}
-
-uint16_t bf16_bits_exact(double v) {
-    const float f = float(v);
-    uint32_t u;
-    std::memcpy(&u, &f, 4);
-    return uint16_t(u >> 16);  // v has at most 8 significant bits: the low half is zero
+// bf16 slices of a matrix's real form (interleaved re, im indices, R = 2 D): row n scaled by the power
+// of two mu[n] >= max|row| and cut on the grids 2^-8(t+1); place(t, n) gives the byte where slice t of
+// row n starts, 8 columns being contiguous and kOzLbo bytes apart from the next 8.
+template <int NS, typename Place>
+void slice_real_form(const std::vector<cplx>& K, int D, float* mu, unsigned char* out, Place&& place) {
+    const int R = 2 * D;
+    double magic[NS];
+    for (int t = 0; t < NS; t++) magic[t] = 1.5 * std::ldexp(1.0, 52 - 8 * (t + 1));
+    double row[2 << QS_MAX_TARGETS];
+    for (int n = 0; n < R; n++) {
+        const cplx* k = K.data() + size_t(n >> 1) * D;
+        double m = 0.0;
+        for (int j = 0; j < D; j++) {
+            row[2 * j] = (n & 1) ? k[j].imag() : k[j].real();
+            row[2 * j + 1] = (n & 1) ? k[j].real() : -k[j].imag();
+            m = std::max(m, std::max(std::fabs(row[2 * j]), std::fabs(row[2 * j + 1])));
+        }
+        double scale = 1.0;
+        if (m > 0.0) {
+            int e = 0;
+            const double f = std::frexp(m, &e);  // m = f 2^e, f in [0.5, 1)
+            scale = f == 0.5 ? m : std::ldexp(1.0, e);
+        }
+        mu[n] = float(scale);
+        for (int k0 = 0; k0 < R; k0 += 8) {
+            double r[8];
+            for (int i = 0; i < 8; i++) r[i] = row[k0 + i] / scale;  // exact (power of two), |r| <= 1
+            for (int t = 0; t < NS; t++) {
+                // r rounded to a multiple of u = 2^-8(t+1): (r + c) - c with c = 1.5 * 2^52 * u
+                // (|r| is far below 2^51 u, so the sum stays in c's binade; exact in FP64); at most 8
+                // significant bits, so that the low half of its float is zero
+                uint32_t u[8];
+                uint16_t bits[8];
+                float f[8];
+                for (int i = 0; i < 8; i++) {
+                    const double a = (r[i] + magic[t]) - magic[t];
+                    r[i] -= a;
+                    f[i] = float(a);
+                }
+                std::memcpy(u, f, sizeof(u));
+                for (int i = 0; i < 8; i++) bits[i] = uint16_t(u[i] >> 16);
+                std::memcpy(out + place(t, n) + size_t(k0 >> 3) * kOzLbo, bits, sizeof(bits));
+            }
+        }
+    }
 }
 
 }  // namespace
@@ -1460,34 +1493,10 @@ size_t oz4_matrix_bytes() { return kOzMat + kOzR * 4; }
 void prepare_oz4_matrix(const std::vector<cplx>& K, unsigned char* host_out) {
     QS_REQUIRE(K.size() == size_t(kOzD) * kOzD, "tensor-core double-float path takes 4-target matrices");
     std::memset(host_out, 0, oz4_matrix_bytes());
-    float* mu = reinterpret_cast<float*>(host_out + kOzMat);
-    double magic[kOzNS];
-    for (int t = 0; t < kOzNS; t++) magic[t] = 1.5 * std::ldexp(1.0, 52 - 8 * (t + 1));
-    for (int n = 0; n < kOzR; n++) {
-        double m = 0.0;
-        for (int k = 0; k < kOzR; k++) m = std::max(m, std::fabs(real_form(K, n, k)));
-        double scale = 1.0;
-        if (m > 0.0) {
-            int e = 0;
-            const double f = std::frexp(m, &e);  // m = f 2^e, f in [0.5, 1)
-            scale = f == 0.5 ? m : std::ldexp(1.0, e);
-        }
-        mu[n] = float(scale);
-        for (int k = 0; k < kOzR; k++) {
-            double r = real_form(K, n, k) / scale;  // exact (power of two), |r| <= 1
-            for (int t = 0; t < kOzNS; t++) {
-                // r rounded to a multiple of u = 2^-8(t+1): (r + c) - c with c = 1.5 * 2^52 * u
-                // (|r| is far below 2^51 u, so the sum stays in c's binade; exact in FP64)
-                const double a = (r + magic[t]) - magic[t];
-                r -= a;
-                const int row = t * kOzR + n;
-                const size_t off = size_t(row >> 3) * kOzSbo + size_t(k >> 3) * kOzLbo + size_t(row & 7) * 16 +
-                                   size_t(k & 7) * 2;
-                const uint16_t bits = bf16_bits_exact(a);
-                std::memcpy(host_out + off, &bits, 2);
-            }
-        }
-    }
+    slice_real_form<kOzNS>(K, kOzD, reinterpret_cast<float*>(host_out + kOzMat), host_out, [](int t, int n) {
+        const int row = t * kOzR + n;
+        return size_t(row >> 3) * kOzSbo + size_t(row & 7) * 16;
+    });
 }
 
 // y = K v on every group of the 4 targets (ascending) of a double-float state.
@@ -1541,38 +1550,10 @@ size_t oz5_matrix_bytes() { return kOz5Mat + kOz5R * 4; }
 void prepare_oz5_matrix(const std::vector<cplx>& K, unsigned char* host_out) {
     QS_REQUIRE(K.size() == size_t(kOz5D) * kOz5D, "5-target tensor-core path takes 32 x 32 matrices");
     std::memset(host_out, 0, oz5_matrix_bytes());
-    float* mu = reinterpret_cast<float*>(host_out + kOz5Mat);
-    double magic[kOzNS];
-    for (int t = 0; t < kOzNS; t++) magic[t] = 1.5 * std::ldexp(1.0, 52 - 8 * (t + 1));
-    auto rf = [&](int n, int k) {
-        const cplx e = K[size_t(n >> 1) * kOz5D + size_t(k >> 1)];
-        if ((n & 1) == 0) return (k & 1) == 0 ? e.real() : -e.imag();
-        return (k & 1) == 0 ? e.imag() : e.real();
-    };
-    for (int n = 0; n < kOz5R; n++) {
-        double m = 0.0;
-        for (int k = 0; k < kOz5R; k++) m = std::max(m, std::fabs(rf(n, k)));
-        double scale = 1.0;
-        if (m > 0.0) {
-            int e = 0;
-            const double f = std::frexp(m, &e);
-            scale = f == 0.5 ? m : std::ldexp(1.0, e);
-        }
-        mu[n] = float(scale);
-        const int hv = n / kOz5D, nl = n % kOz5D;
-        for (int k = 0; k < kOz5R; k++) {
-            double r = rf(n, k) / scale;
-            for (int t = 0; t < kOzNS; t++) {
-                const double a = (r + magic[t]) - magic[t];
-                r -= a;
-                const int row = t * kOz5D + nl;
-                const size_t off = size_t(hv) * kOz5Half + size_t(row >> 3) * kOz5Sbo + size_t(k >> 3) * kOzLbo +
-                                   size_t(row & 7) * 16 + size_t(k & 7) * 2;
-                const uint16_t bits = bf16_bits_exact(a);
-                std::memcpy(host_out + off, &bits, 2);
-            }
-        }
-    }
+    slice_real_form<kOzNS>(K, kOz5D, reinterpret_cast<float*>(host_out + kOz5Mat), host_out, [](int t, int n) {
+        const int row = t * kOz5D + n % kOz5D;
+        return size_t(n / kOz5D) * kOz5Half + size_t(row >> 3) * kOz5Sbo + size_t(row & 7) * 16;
+    });
 }
 
 void launch_dense_oz5(void* psi, int n, const std::vector<int>& targets, const std::vector<int>& controls,
@@ -1626,38 +1607,11 @@ void prepare_bz_matrix(int q, const std::vector<cplx>& K, unsigned char* host_ou
     const size_t sbo = size_t(R / 8) * 128;
     QS_REQUIRE(K.size() == size_t(D) * D, "matrix size does not match the target count");
     std::memset(host_out, 0, bz_matrix_bytes(q));
-    float* mu = reinterpret_cast<float*>(host_out + size_t(kBzNS) * R * R * 2);
-    double magic[kBzNS];
-    for (int t = 0; t < kBzNS; t++) magic[t] = 1.5 * std::ldexp(1.0, 52 - 8 * (t + 1));
-    auto rf = [&](int n, int k) {
-        const cplx e = K[size_t(n >> 1) * D + size_t(k >> 1)];
-        if ((n & 1) == 0) return (k & 1) == 0 ? e.real() : -e.imag();
-        return (k & 1) == 0 ? e.imag() : e.real();
-    };
-    for (int n = 0; n < R; n++) {
-        double m = 0.0;
-        for (int k = 0; k < R; k++) m = std::max(m, std::fabs(rf(n, k)));
-        double scale = 1.0;
-        if (m > 0.0) {
-            int e = 0;
-            const double f = std::frexp(m, &e);
-            scale = f == 0.5 ? m : std::ldexp(1.0, e);
-        }
-        mu[n] = float(scale);
-        for (int k = 0; k < R; k++) {
-            double r = rf(n, k) / scale;
-            for (int t = 0; t < kBzNS; t++) {
-                const double a = (r + magic[t]) - magic[t];
-                r -= a;
-                // q = 5: [B_0; B_1; B_2]; q = 6: per output half h, [B_0h; B_1h; B_2h]
-                const int row = q == 5 ? t * R + n : (n / (R / 2)) * (kBzNS * (R / 2)) + t * (R / 2) + n % (R / 2);
-                const size_t off = size_t(row >> 3) * sbo + size_t(k >> 3) * kOzLbo + size_t(row & 7) * 16 +
-                                   size_t(k & 7) * 2;
-                const uint16_t bits = bf16_bits_exact(a);
-                std::memcpy(host_out + off, &bits, 2);
-            }
-        }
-    }
+    slice_real_form<kBzNS>(K, D, reinterpret_cast<float*>(host_out + size_t(kBzNS) * R * R * 2), host_out, [&](int t, int n) {
+        // q = 5: [B_0; B_1; B_2]; q = 6: per output half h, [B_0h; B_1h; B_2h]
+        const int row = q == 5 ? t * R + n : (n / (R / 2)) * (kBzNS * (R / 2)) + t * (R / 2) + n % (R / 2);
+        return size_t(row >> 3) * sbo + size_t(row & 7) * 16;
+    });
 }
 
 template <int Q>

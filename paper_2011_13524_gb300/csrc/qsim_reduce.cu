@@ -632,15 +632,20 @@ void ensure_scratch(qs_state* s, size_t part_doubles) {
     Scratch& sc = s->scratch;
     if (sc.part_cap < part_doubles) {
         if (sc.d_part) {
-            QS_TRY_CUDA(cudaStreamSynchronize(s->stream));
-            dev_free(sc.d_part);
+            if (s->pooled) {
+                dev_free_async(sc.d_part, s->stream);
+            } else {
+                QS_TRY_CUDA(cudaStreamSynchronize(s->stream));
+                dev_free(sc.d_part);
+            }
             sc.d_part = nullptr;
             sc.part_cap = 0;
         }
-        QS_TRY_CUDA(dev_malloc(&sc.d_part, part_doubles * sizeof(double)));
+        QS_TRY_CUDA(s->pooled ? dev_malloc_async(&sc.d_part, part_doubles * sizeof(double), s->stream)
+                              : dev_malloc(&sc.d_part, part_doubles * sizeof(double)));
         sc.part_cap = part_doubles;
     }
-    if (!sc.h_out) {
+    if (!sc.h_out && !s->pooled) {  // (a state of one call copies to pageable memory: no pinned allocation)
         QS_TRY_CUDA(host_malloc_pinned(&sc.h_out, 16 * sizeof(double)));
         sc.out_cap = 16;
     }
@@ -651,6 +656,11 @@ void finish2(qs_state* s, int nslots, double out[2]) {
     double* d_out = s->scratch.d_part + s->scratch.part_cap - 2;
     k_final2<<<1, kRedThreads, 0, s->stream>>>(s->scratch.d_part, nslots, d_out);
     QS_TRY_CUDA(cudaGetLastError());
+    if (s->pooled) {
+        QS_TRY_CUDA(cudaMemcpyAsync(out, d_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
+        QS_TRY_CUDA(cudaStreamSynchronize(s->stream));
+        return;
+    }
     QS_TRY_CUDA(cudaMemcpyAsync(s->scratch.h_out, d_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
     QS_TRY_CUDA(cudaStreamSynchronize(s->stream));
     out[0] = s->scratch.h_out[0];
