@@ -27,6 +27,7 @@
 // small. Per-thread sums are double-float and go to an FP64 accumulator once per tile, so the
 // result has the accuracy of an FP64 sum (about 2^-44 relative per tile).
 #include <algorithm>
+#include <cmath>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -706,6 +707,198 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_transition_tiled(const C* _
     }
 }
 
+// ---------------------------------------------------------------- X strings of one weight
+// A tile of 2^12 amplitudes of ket in shared memory and, per thread, its own 16 (tile-local index
+// tid + 256 k) in registers; w_y = sum_f ket_{y ^ f} by additions, then conj(bra_y) w_y once per
+// amplitude.
+// Every component is an integer F of 51 bits on one grid per tile, 2^-49 of the power of two below the
+// tile's largest component, held as F = 2^23 I + L: I sums exactly as a 32-bit integer (|I| <= 2^27, up
+// to 12 strings), L (0 <= L < 2^23) as a float, one integer addition per part and two strings (three
+// operands) and one packed FP32 addition per string. The sum becomes a double-float pair (24 bits and
+// a rest) for the product: its error is 2^-45 of the tile's largest component.
+// What bounds it: instruction issue, most of it per amplitude (reading, fixing and splitting, one complex
+// product), 2 to 3.3 per string, where the products of k_transition_tiled take 40 per string. The Ising
+// chain's 26 X terms at n = 26 (complex128): 0.59, 0.54 and 0.50 ms for 12, 9 and 5 strings, with the
+// diagonal terms' read (0.99 ms) 2.6 ms against 4.8 ms in tiled reads. Error of the chain's amplitude on
+// random states, rms: 2.3e-15 against 6.4e-15 at n = 12 (1.2e-15 / 2.4e-15 at n = 15). Cutting on an FP32
+// grid instead (20 bits and a rest) measured the same time and 2.0e-14. For expectations, whose pair
+// products take 12.5 per string, it gained 8 % and is not used.
+__device__ __forceinline__ uint32_t magnitude_bits(double2 v) {
+    return max(uint32_t(__double2hiint(v.x)) & 0x7FFFFFFFu, uint32_t(__double2hiint(v.y)) & 0x7FFFFFFFu);
+}
+__device__ __forceinline__ uint32_t magnitude_bits(float2 v) {
+    return max(__float_as_uint(v.x) & 0x7FFFFFFFu, __float_as_uint(v.y) & 0x7FFFFFFFu);
+}
+__device__ __forceinline__ int magnitude_exponent(uint32_t m, double2) { return int(m >> 20) - 1023; }
+__device__ __forceinline__ int magnitude_exponent(uint32_t m, float2) { return int(m >> 23) - 127; }
+__device__ __forceinline__ float4 split_pair(double2 v) { return to_tile(v); }
+__device__ __forceinline__ float4 split_pair(float2 v) { return make_float4(v.x, v.y, 0.f, 0.f); }
+
+// x = (2^23 I + L) 2^(e - 49) truncated, for |x| < 2^(e + 1); eb = e + 1023
+__device__ __forceinline__ void fix_mantissa(uint32_t sign, uint32_t ex, uint64_t man53, int eb, int& I, float& L) {
+    const int sh = min(eb + 3 - int(ex), 63);  // man53 2^(ex - 1075) in units of 2^(e - 49)
+    const long long s = static_cast<long long>(int(sign) >> 31);
+    const long long F = (static_cast<long long>(man53 >> sh) ^ s) - s;
+    const uint32_t lo = uint32_t(F), hi = uint32_t(uint64_t(F) >> 32);
+    I = int(__funnelshift_r(lo, hi, 23));
+    L = __fsub_rn(__uint_as_float((lo & 0x7FFFFFu) | 0x4B000000u), 8388608.f);
+}
+__device__ __forceinline__ void fix_point(double x, int eb, int& I, float& L) {
+    const uint32_t h = uint32_t(__double2hiint(x));
+    const uint32_t ex = (h >> 20) & 0x7FFu;
+    fix_mantissa(h, ex, (uint64_t((h & 0xFFFFFu) | 0x100000u) << 32) | uint32_t(__double2loint(x)), eb, I, L);
+}
+__device__ __forceinline__ void fix_point(float x, int eb, int& I, float& L) {
+    const uint32_t u = __float_as_uint(x), f = (u >> 23) & 0xFFu;
+    // (a subnormal keeps its bits without the implicit one)
+    const uint32_t man = (u & 0x7FFFFFu) | (f ? 0x800000u : 0u);
+    fix_mantissa(u, (f ? f : 1u) + 896u, uint64_t(man) << 29, eb, I, L);
+}
+
+// (2^23 I + L) 2^(e - 49) as a double-float pair, both parts of an amplitude side by side; su = 2^(e - 26)
+__device__ __forceinline__ void fixed_to_pair(int2 I, float2 L, float su, float2& h, float2& l) {
+    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 fa = __fadd2_rn(make_float2(__int_as_float((I.x >> 11) + 0x4B400000), __int_as_float((I.y >> 11) + 0x4B400000)),
+                                 make_float2(-12582912.f, -12582912.f));
+    const float2 fb = __fadd2_rn(make_float2(__int_as_float((I.x & 0x7FF) | 0x4B000000), __int_as_float((I.y & 0x7FF) | 0x4B000000)),
+                                 make_float2(-8388608.f, -8388608.f));
+    const float2 k = make_float2(2048.f, 2048.f);
+    const float2 w = __ffma2_rn(fa, k, fb);                       // RN(I)
+    const float2 t = __ffma2_rn(fa, make_float2(-2048.f, -2048.f), w);  // exact
+    const float2 rest = __ffma2_rn(t, m1, fb);                    // I - w, exact
+    const float2 low = __ffma2_rn(rest, make_float2(8388608.f, 8388608.f), L);  // units of 2^(e - 49)
+    const float sl = su * 1.1920928955078125e-07f;
+    h = __fmul2_rn(w, make_float2(su, su));
+    l = __fmul2_rn(low, make_float2(sl, sl));
+}
+
+// (s, c) += (ah + al) * (bh + bl) lane by lane
+__device__ __forceinline__ void acc_prod2(float2& s, float2& c, float2 ah, float2 al, float2 bh, float2 bl) {
+    const float2 m1 = make_float2(-1.f, -1.f);
+    const float2 p = __fmul2_rn(ah, bh);
+    float2 e = __ffma2_rn(ah, bh, make_float2(-p.x, -p.y));
+    e = __ffma2_rn(ah, bl, e);
+    e = __ffma2_rn(al, bh, e);
+    e = __ffma2_rn(al, bl, e);  // (the low parts of w are not centred: their products do not average out)
+    const float2 t = __fadd2_rn(s, p);
+    const float2 bp = __ffma2_rn(s, m1, t);
+    const float2 d = __fadd2_rn(__ffma2_rn(__ffma2_rn(bp, m1, t), m1, s), __ffma2_rn(bp, m1, p));
+    s = t;
+    c = __fadd2_rn(c, __fadd2_rn(d, e));
+}
+
+template <typename C>
+__global__ void __launch_bounds__(kTileThreads, 2) k_xsum(const C* __restrict__ ket, const C* __restrict__ bra,
+                                                          const __grid_constant__ XsumParams P, double* __restrict__ part) {
+    constexpr int K = kTileAmps / kTileThreads;
+    constexpr int kParts = 4;  // the thread's amplitudes are summed and multiplied K / kParts at a time
+    extern __shared__ __align__(16) unsigned char tsm[];
+    float4* tile = reinterpret_cast<float4*>(tsm);
+    __shared__ uint32_t smax[kTileThreads / 32];
+    __shared__ double sh[kTileThreads / 32];
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    uint64_t dthr = 0;
+#pragma unroll
+    for (int i = 0; i < 8; i++)
+        if ((tid >> i) & 1) dthr |= 1ull << P.tpos[i];
+    uint64_t rbase = deposit64(blockIdx.x, P.rest_mask);
+    const uint64_t step = deposit64(gridDim.x, P.rest_mask);
+    double accr = 0.0, acci = 0.0;
+    for (uint64_t r = blockIdx.x; r < P.n_tiles; r += gridDim.x) {
+        const uint64_t at = rbase | dthr;
+        rbase = ((rbase | ~P.rest_mask) + step) & P.rest_mask;
+        C v[K];
+        uint32_t m = 0;
+#pragma unroll
+        for (int k = 0; k < K; k++) v[k] = ket[at | P.dep_hi[k]];
+#pragma unroll
+        for (int k = 0; k < K; k++) m = max(m, magnitude_bits(v[k]));
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (lane == 0) smax[warp] = m;
+        __syncthreads();  // (and the previous tile's readers are done)
+#pragma unroll
+        for (int w = 0; w < kTileThreads / 32; w++) m = max(m, smax[w]);
+        const int e = max(magnitude_exponent(m, v[0]), -90);  // largest component below 2^(e + 1)
+        const float su = __uint_as_float(uint32_t(min(e, 115) - 26 + 127) << 23);
+        int2 I[K];
+        float2 L[K];
+#pragma unroll
+        for (int k = 0; k < K; k++) {
+            fix_point(v[k].x, e + 1023, I[k].x, L[k].x);
+            fix_point(v[k].y, e + 1023, I[k].y, L[k].y);
+            tile[tid + kTileThreads * k] =
+                make_float4(__int_as_float(I[k].x), __int_as_float(I[k].y), L[k].x, L[k].y);
+        }
+        __syncthreads();
+        float2 sr = make_float2(0.f, 0.f), cr = sr, si = sr, ci = sr;
+#pragma unroll
+        for (int hf = 0; hf < kParts; hf++) {
+            constexpr int kH = K / kParts;
+            C b[kH];
+#pragma unroll
+            for (int j = 0; j < kH; j++) b[j] = bra[at | P.dep_hi[hf * kH + j]];
+            int2 WI[kH];
+            float2 WL[kH];
+#pragma unroll
+            for (int j = 0; j < kH; j++) {
+                WI[j] = make_int2(0, 0);
+                WL[j] = make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                if ((P.item >> q) & 1u) {
+#pragma unroll
+                    for (int j = 0; j < kH; j++) {
+                        WI[j].x += I[(hf * kH + j) ^ (1 << q)].x;
+                        WI[j].y += I[(hf * kH + j) ^ (1 << q)].y;
+                        WL[j] = __fadd2_rn(WL[j], L[(hf * kH + j) ^ (1 << q)]);
+                    }
+                }
+            int g = 0;
+            for (; g + 1 < P.nf; g += 2) {
+                const uint32_t o = tid ^ P.f[g], p = tid ^ P.f[g + 1];
+#pragma unroll
+                for (int j = 0; j < kH; j++) {
+                    const float4 x = tile[o ^ uint32_t(kTileThreads * (hf * kH + j))];
+                    const float4 y = tile[p ^ uint32_t(kTileThreads * (hf * kH + j))];
+                    WI[j].x += __float_as_int(x.x) + __float_as_int(y.x);
+                    WI[j].y += __float_as_int(x.y) + __float_as_int(y.y);
+                    WL[j] = __fadd2_rn(WL[j], __fadd2_rn(make_float2(x.z, x.w), make_float2(y.z, y.w)));
+                }
+            }
+            if (g < P.nf) {
+                const uint32_t o = tid ^ P.f[g];
+#pragma unroll
+                for (int j = 0; j < kH; j++) {
+                    const float4 x = tile[o ^ uint32_t(kTileThreads * (hf * kH + j))];
+                    WI[j].x += __float_as_int(x.x);
+                    WI[j].y += __float_as_int(x.y);
+                    WL[j] = __fadd2_rn(WL[j], make_float2(x.z, x.w));
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < kH; j++) {
+                float2 wh, wl;
+                fixed_to_pair(WI[j], WL[j], su, wh, wl);
+                // conj(b) w = (b.re w.re + b.im w.im) + i (b.re w.im - b.im w.re)
+                const float4 y = split_pair(b[j]);
+                const float2 yh = make_float2(y.x, y.y), yl = make_float2(y.z, y.w);
+                acc_prod2(sr, cr, yh, yl, wh, wl);
+                acc_prod2(si, ci, yh, yl, make_float2(wh.y, wh.x), make_float2(wl.y, wl.x));
+            }
+        }
+        if (e > 115) sr.x = __uint_as_float(0x7FC00000u);  // not finite, or out of FP32's range
+        accr += (widen_float_int(sr.x) + widen_float_int(sr.y)) + widen_float_int(__fadd_rn(cr.x, cr.y));
+        acci += (widen_float_int(si.x) - widen_float_int(si.y)) + widen_float_int(__fsub_rn(ci.x, ci.y));
+    }
+    const double tr = block_sum<kTileThreads>(accr, sh);
+    const double ti = block_sum<kTileThreads>(acci, sh);
+    if (tid == 0) {
+        part[2 * blockIdx.x] = P.alpha * tr;
+        part[2 * blockIdx.x + 1] = P.alpha * ti;
+    }
+}
+
 // CTAs per SM of the tiled kernels at their shared-memory size (attribute raised once per device)
 template <typename C>
 int trans_blocks_per_sm() {
@@ -1075,6 +1268,116 @@ void launch_expect_pass(const TileParams& P, const void* psi, Arith ar, double* 
             break;
     }
     QS_TRY_CUDA(cudaGetLastError());
+}
+
+std::vector<PauliGroup> split_xsum(const std::vector<PauliGroup>& groups, int n, Arith ar,
+                                   std::vector<XsumParams>& passes) {
+    passes.clear();
+    if (n < kTileBits || ar == Arith::DF) return groups;
+    const uint64_t low = (1ull << kTileLowBits) - 1;
+    auto takes = [&](const PauliGroup& g) {
+        return g.xmask && g.coef.size() == 1 && g.zmask[0] == 0 && std::isfinite(g.coef[0]) &&
+               __builtin_popcountll(g.xmask & ~low) <= kTileBits - kTileLowBits;
+    };
+    std::map<double, int> weights;
+    for (const PauliGroup& g : groups)
+        if (takes(g)) weights[g.coef[0]]++;
+    double alpha = 0.0;
+    int most = 0;
+    for (const auto& w : weights)
+        if (w.second > most) {
+            alpha = w.first;
+            most = w.second;
+        }
+    if (most < kXsumMinGroups) return groups;
+    std::vector<PauliGroup> rest;
+    std::vector<uint64_t> flips;
+    for (const PauliGroup& g : groups) {
+        if (takes(g) && g.coef[0] == alpha) flips.push_back(g.xmask);
+        else rest.push_back(g);
+    }
+    std::sort(flips.begin(), flips.end());
+    struct Tile {
+        uint64_t T;
+        std::vector<uint64_t> f;
+    };
+    std::vector<Tile> tiles;  // as pack_tiles: the tile that grows least
+    for (uint64_t f : flips) {
+        int best = -1, best_growth = 1 << 30;
+        for (size_t t = 0; t < tiles.size(); t++) {
+            const uint64_t U = tiles[t].T | f;
+            if (tiles[t].f.size() >= size_t(kXsumMaxFlips) || __builtin_popcountll(U) > kTileBits) continue;
+            const int growth = __builtin_popcountll(U) - __builtin_popcountll(tiles[t].T);
+            if (growth < best_growth) {
+                best_growth = growth;
+                best = int(t);
+            }
+        }
+        if (best < 0) {
+            tiles.push_back(Tile{low, {}});
+            best = int(tiles.size()) - 1;
+        }
+        tiles[size_t(best)].T |= f;
+        tiles[size_t(best)].f.push_back(f);
+    }
+    const uint64_t full = n >= 64 ? ~0ull : ((1ull << n) - 1);
+    for (Tile& t : tiles) {
+        for (int q = 0; q < n && __builtin_popcountll(t.T) < kTileBits; q++) t.T |= 1ull << q;
+        XsumParams P;
+        int pos[kTileBits], np = 0;
+        for (int q = 0; q < n; q++)
+            if ((t.T >> q) & 1) pos[np++] = q;
+        for (int i = 0; i < kTileBits; i++) P.tpos[i] = uint8_t(pos[i]);
+        P.rest_mask = full & ~t.T;
+        P.n_tiles = 1ull << (n - kTileBits);
+        for (int k = 0; k < kTileAmps / kTileThreads; k++)
+            for (int i = 8; i < kTileBits; i++)
+                if (((k << 8) >> i) & 1) P.dep_hi[k] |= 1ull << pos[i];
+        P.alpha = alpha;
+        for (uint64_t f : t.f) {
+            const uint32_t l = compress_bits(f, pos, kTileBits);
+            if ((l & (l - 1)) == 0 && l >= 256u) P.item |= l >> 8;
+            else P.f[P.nf++] = l;
+        }
+        passes.push_back(P);
+    }
+    return rest;
+}
+
+namespace {
+// CTAs per SM of k_xsum (attribute raised once per device)
+template <typename C>
+int xsum_blocks_per_sm() {
+    static PerDevice setup;
+    static int b[kMaxDevices];
+    setup.once([](int dev) {
+        const size_t bytes = sizeof(float4) * kTileAmps;
+        QS_TRY_CUDA(cudaFuncSetAttribute(k_xsum<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
+        int nb = 0;
+        QS_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_xsum<C>, kTileThreads, bytes));
+        b[dev] = nb > 0 ? nb : 1;
+    });
+    return b[current_device()];
+}
+template <typename C>
+void launch_xsum_t(const XsumParams& P, const void* bra, const void* ket, double* part, unsigned grid, cudaStream_t st) {
+    const size_t bytes = sizeof(float4) * kTileAmps;
+    xsum_blocks_per_sm<C>();
+    k_xsum<C><<<grid, kTileThreads, bytes, st>>>(static_cast<const C*>(ket), static_cast<const C*>(bra), P, part);
+    QS_TRY_CUDA(cudaGetLastError());
+}
+}  // namespace
+
+unsigned xsum_grid(const XsumParams& P, Arith ar) {
+    const int per = ar == Arith::F32 ? xsum_blocks_per_sm<float2>() : xsum_blocks_per_sm<double2>();
+    return unsigned(std::max<uint64_t>(1, std::min<uint64_t>(P.n_tiles, uint64_t(per) * uint64_t(sm_count()))));
+}
+
+void launch_xsum(const XsumParams& P, const void* bra, const void* ket, Arith ar, double* part, unsigned grid,
+                 cudaStream_t st) {
+    QS_REQUIRE(ar != Arith::DF, "X-string sums read IEEE states");
+    if (ar == Arith::F32) launch_xsum_t<float2>(P, bra, ket, part, grid, st);
+    else launch_xsum_t<double2>(P, bra, ket, part, grid, st);
 }
 
 unsigned trans_pass_grid(const TileParams& P, Arith ar) {

@@ -336,6 +336,27 @@ unsigned expect_diag_grid(int n, Arith ar);
 void launch_expect_diag(const DiagObsParams& P, const void* psi, Arith ar, double* part, unsigned grid,
                         cudaStream_t st);
 ExpectPlan plan_expectation(const std::vector<PauliGroup>& groups, int n);
+// X strings of one weight (single-term groups without Z or Y) in a transition amplitude: sum_f <bra|X_f|ket> = <bra|w> with
+// w_y = sum_f ket_{y ^ f}, additions per string and one product per amplitude. One read per tile of
+// 12 qubits (0..2 and 9 others) that holds the flip masks.
+constexpr int kXsumMaxFlips = 12;
+struct XsumParams {
+    uint64_t rest_mask = 0, n_tiles = 0;
+    uint64_t dep_hi[kTileAmps / kTileThreads] = {};  // global offset of tile-local index 256 k
+    double alpha = 0.0;
+    uint8_t tpos[kTileBits] = {};                    // tile-local bit i = qubit tpos[i]
+    int32_t nf = 0;                                  // flips by shared memory, tile-local masks f[]
+    uint32_t item = 0;                               // bit b: the flip of tile-local bit 8 + b alone
+    uint32_t f[kXsumMaxFlips] = {};
+};
+// Takes such strings out of groups (the most frequent weight, when at least kXsumMinGroups strings of
+// a state of 12 qubits or more have it) and returns the rest.
+constexpr int kXsumMinGroups = 4;
+std::vector<PauliGroup> split_xsum(const std::vector<PauliGroup>& groups, int n, Arith ar, std::vector<XsumParams>& passes);
+unsigned xsum_grid(const XsumParams& P, Arith ar);
+// part[2 j], part[2 j + 1] = block j's partial of alpha <bra|w>
+void launch_xsum(const XsumParams& P, const void* bra, const void* ket, Arith ar, double* part, unsigned grid,
+                 cudaStream_t st);
 unsigned expect_pass_grid(const TileParams& P, Arith ar);
 // Transition amplitude <bra|O|ket>: tiles of 2^11 slots of both states (qubits 0..2 plus 8
 // others); flip groups with more than 8 bits above qubit 2 go to heavy.

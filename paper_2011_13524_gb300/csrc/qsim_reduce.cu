@@ -875,9 +875,15 @@ void reduce_transition(const qs_state* bra, const qs_pauli_obs* obs, const qs_st
         return;
     }
     const Arith ar = arith_of(s);
-    const ExpectPlan plan = plan_transition(groups, s->n);
-    std::vector<unsigned> grids;
+    std::vector<XsumParams> xsum;
+    const std::vector<PauliGroup> rest = split_xsum(groups, s->n, ar, xsum);
+    const ExpectPlan plan = rest.empty() ? ExpectPlan() : plan_transition(rest, s->n);
+    std::vector<unsigned> grids, xgrids;
     size_t slots_needed = 0;
+    for (const XsumParams& P : xsum) {
+        xgrids.push_back(xsum_grid(P, ar));
+        slots_needed += xgrids.back();
+    }
     for (const TileParams& P : plan.passes) {
         grids.push_back(trans_pass_grid(P, ar));
         slots_needed += grids.back();
@@ -886,6 +892,10 @@ void reduce_transition(const qs_state* bra, const qs_pauli_obs* obs, const qs_st
     slots_needed += size_t(gr) * plan.heavy.size();
     ensure_scratch(s, 2 * slots_needed + 2);
     size_t slots = 0;
+    for (size_t p = 0; p < xsum.size(); p++) {
+        launch_xsum(xsum[p], bra->data, ket->data, ar, s->scratch.d_part + 2 * slots, xgrids[p], s->stream);
+        slots += xgrids[p];
+    }
     for (size_t p = 0; p < plan.passes.size(); p++) {
         launch_transition_pass(plan.passes[p], bra->data, ket->data, ar, s->scratch.d_part + 2 * slots, grids[p],
                                s->stream);

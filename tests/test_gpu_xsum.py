@@ -1,0 +1,73 @@
+"""X strings of one weight (k_xsum) in transition amplitudes, beside the expectations of the same: against the oracle, and
+against the tiled reads (the same strings with weights that differ), on tile edges, several tiles,
+strings on register, lane and warp bits, with diagonal and other terms beside them."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def observable(n, strings):
+    coef, xm, zm = zip(*strings)
+    return W.PauliObservable(n, np.array(coef), np.array(xm, dtype=np.uint64), np.array(zm, dtype=np.uint64))
+
+
+def cases(n):
+    chain = [(1.0, 0, 3 << i) for i in range(n - 1)] + [(0.7, 1 << i, 0) for i in range(n)]
+    high = [(-0.3, 1 << i, 0) for i in range(n - 5, n)]
+    pairs = [(0.4, 3 << i, 0) for i in range(n - 1)] + [(0.4, 1 | (1 << (n - 1)), 0)]
+    mixed = chain + [(0.2, 3, 3), (0.5, 1, 2), (0.7, 7, 0), (-0.7, 5, 0), (1.5, 0, 0), (0.25, (1 << n) - 1, 5)]
+    few = [(1.0, 1, 0), (1.0, 2, 0), (1.0, 1 << (n - 1), 0)]  # fewer than a read of their own takes
+    return {"chain": chain, "high": high, "pairs": pairs, "mixed": mixed, "few": few}
+
+
+@pytest.mark.parametrize("dtype", ["c128", "c64"])
+@pytest.mark.parametrize("n", [11, 12, 13, 15])
+@pytest.mark.parametrize("case", ["chain", "high", "pairs", "mixed", "few"])
+def test_against_the_oracle(case, n, dtype):
+    import paper_2011_13524_gb300 as qs
+    obs = observable(n, cases(n)[case])
+    dt = qs.QS_C64 if dtype == "c64" else qs.QS_C128
+    a, b = qs.State(n, dt), qs.State(n, dt)
+    a.load(W.random_state_fast(n, 1))
+    b.load(W.random_state_fast(n, 2))
+    va, vb = a.get_vector().astype(np.complex128), b.get_vector().astype(np.complex128)
+    # the tiled reads' bound: 1e-13 of the weights (norm 1 to the storage's rounding)
+    tol = 1e-13 * float(np.abs(obs.coef).sum())
+    assert abs(a.expectation(obs)[0] - oracle.expectation(va, obs)[0]) < tol
+    t = oracle.transition_amplitude(va, vb, n, obs)
+    assert abs(a.transition_amplitude(obs, b) - t) < tol
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("dtype", ["c128", "c64"])
+def test_against_tiled_reads(dtype):
+    """Eight tiles and more per CTA; amplitudes over many magnitudes between tiles."""
+    import torch
+    import paper_2011_13524_gb300 as qs
+    n = 22
+    dt, tdt = (qs.QS_C64, torch.complex64) if dtype == "c64" else (qs.QS_C128, torch.complex128)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    states = []
+    for _ in range(2):
+        v = torch.randn(1 << n, dtype=tdt, device="cuda", generator=g)
+        v *= torch.exp2(-(torch.arange(1 << n, device="cuda") >> 14) % 31)
+        states.append(qs.State(n, dt, tensor=v / torch.linalg.vector_norm(v)))
+    a, b = states
+    same = observable(n, [(0.5, 1 << i, 0) for i in range(n)])
+    apart = observable(n, [(0.5 + 2.0 ** -20 * i, 1 << i, 0) for i in range(n)])
+    back = observable(n, [(-(2.0 ** -20) * i, 1 << i, 0) for i in range(1, n)])
+    tol = 1e-13 * n
+    assert abs(a.expectation(same)[0] - (a.expectation(apart)[0] + a.expectation(back)[0])) < tol
+    t = a.transition_amplitude(apart, b) + a.transition_amplitude(back, b)
+    assert abs(a.transition_amplitude(same, b) - t) < tol
+    zero = qs.State(n, dt)
+    assert a.transition_amplitude(same, a) == pytest.approx(a.expectation(same)[0], abs=tol)
+    assert abs(zero.expectation(same)[0]) < tol  # all tiles but one empty
+    for s in (a, b, zero):
+        s.close()
