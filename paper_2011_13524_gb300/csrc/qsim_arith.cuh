@@ -234,4 +234,61 @@ __device__ __forceinline__ double join_df_int(float hi, float lo) {
     return __longlong_as_double(w + static_cast<long long>(__float2int_rn(y)));
 }
 
+// an amplitude of a double-float kernel that reads and writes the IEEE layout itself
+__device__ __forceinline__ float4 df_of_ieee(float4 raw) {
+    const double2 d = *reinterpret_cast<const double2*>(&raw);
+    float4 r;
+    split_double_int(d.x, r.x, r.y);
+    split_double_int(d.y, r.z, r.w);
+    return r;
+}
+__device__ __forceinline__ float4 ieee_of_df(float4 v) {
+    const double2 d = make_double2(join_df_int(v.x, v.y), join_df_int(v.z, v.w));
+    return *reinterpret_cast<const float4*>(&d);
+}
+
+// c a + k b for a real c and a k that is real or imaginary (a Pauli rotation's factors): the sums of
+// first(c, a) and mac(k, b) without their products by zero
+template <typename R>
+__device__ __forceinline__ typename CT<R>::type rot_mix(typename CT<R>::type c, typename CT<R>::type k, bool imag,
+                                                        typename CT<R>::type a, typename CT<R>::type b) {
+    typename CT<R>::type r;
+    r.x = c.x * a.x;
+    r.y = c.x * a.y;
+    if constexpr (sizeof(R) == 4) {
+        r.x = imag ? fmaf(-k.y, b.y, r.x) : fmaf(k.x, b.x, r.x);
+        r.y = imag ? fmaf(k.y, b.x, r.y) : fmaf(k.x, b.y, r.y);
+    } else {
+        r.x = imag ? fma(-k.y, b.y, r.x) : fma(k.x, b.x, r.x);
+        r.y = imag ? fma(k.y, b.x, r.y) : fma(k.x, b.y, r.y);
+    }
+    return r;
+}
+template <typename P>
+struct RotMix;
+template <typename R>
+struct RotMix<NativeArith<R>> {
+    using C = typename CT<R>::type;
+    __device__ __forceinline__ static C mix(const C& c, const C& k, bool imag, const C& a, const C& b) {
+        return rot_mix<R>(c, k, imag, a, b);
+    }
+};
+template <>
+struct RotMix<DFArith> {
+    __device__ __forceinline__ static float4 mix(const float4& c, const float4& k, bool imag, const float4& a,
+                                                 const float4& b) {
+        DFArith::Acc s;
+        DFArith::dprod0(s.rs, s.rc, c.x, c.y, a.x, a.y);
+        DFArith::dprod0(s.is, s.ic, c.x, c.y, a.z, a.w);
+        if (imag) {
+            DFArith::dprod(s.rs, s.rc, -k.z, -k.w, b.z, b.w);
+            DFArith::dprod(s.is, s.ic, k.z, k.w, b.x, b.y);
+        } else {
+            DFArith::dprod(s.rs, s.rc, k.x, k.y, b.x, b.y);
+            DFArith::dprod(s.is, s.ic, k.x, k.y, b.z, b.w);
+        }
+        return DFArith::out(s);
+    }
+};
+
 }  // namespace qs

@@ -37,10 +37,28 @@ template <typename P, int M>
 struct DenseRegParams {
     IndexPlan ip;
     uint64_t offs[1 << M];
+    int32_t form;  // M = 1, FP64: 0 general, 1 real entries, 2 real diagonal and imaginary off-diagonal
     typename P::K K[(1 << M) * (1 << M)];
 };
 
-template <typename P, int M>
+// One-qubit FP64 gates are bound by the FP64 rate (GB300: 1/64 of FP32), eight multiply-adds per
+// amplitude in general; entries that are real (H, RY) or whose off-diagonal is imaginary (RX) need
+// four: 516 / 265 us at n = 25. The values are those of the general form, whose other products are zero.
+__device__ __forceinline__ void pair_form(const double2* K, int form, double2 a, double2 b, double2& ra, double2& rb) {
+    ra = make_double2(K[0].x * a.x, K[0].x * a.y);
+    if (form == 1) {
+        ra = make_double2(fma(K[1].x, b.x, ra.x), fma(K[1].x, b.y, ra.y));
+        rb = make_double2(K[2].x * a.x, K[2].x * a.y);
+    } else {
+        ra = make_double2(fma(-K[1].y, b.y, ra.x), fma(K[1].y, b.x, ra.y));
+        rb = make_double2(-K[2].y * a.y, K[2].y * a.x);
+    }
+    rb = make_double2(fma(K[3].x, b.x, rb.x), fma(K[3].x, b.y, rb.y));
+}
+
+// kSpecial: double-float, the state is read and written as IEEE complex128; FP64 and M = 1, a form other
+// than the general one.
+template <typename P, int M, bool kSpecial>
 __global__ void __launch_bounds__(kThreads) k_dense_reg(typename P::C* __restrict__ psi,
                                                         const __grid_constant__ DenseRegParams<P, M> Pm) {
     using C = typename P::C;
@@ -51,12 +69,25 @@ __global__ void __launch_bounds__(kThreads) k_dense_reg(typename P::C* __restric
         C v[D];
 #pragma unroll
         for (int w = 0; w < D; w++) v[w] = psi[x0 + Pm.offs[w]];
+        if constexpr (kSpecial && std::is_same<P, DFArith>::value) {
+#pragma unroll
+            for (int w = 0; w < D; w++) v[w] = df_of_ieee(v[w]);
+        }
+        if constexpr (kSpecial && std::is_same<P, NativeArith<double>>::value && M == 1) {
+            C ra, rb;
+            pair_form(Pm.K, Pm.form, v[0], v[1], ra, rb);
+            psi[x0 + Pm.offs[0]] = ra;
+            psi[x0 + Pm.offs[1]] = rb;
+            continue;
+        }
 #pragma unroll
         for (int z = 0; z < D; z++) {
             typename P::Acc a = P::first(Pm.K[z * D], v[0]);
 #pragma unroll
             for (int w = 1; w < D; w++) P::mac(a, Pm.K[z * D + w], v[w]);
-            psi[x0 + Pm.offs[z]] = P::out(a);
+            C o = P::out(a);
+            if constexpr (kSpecial && std::is_same<P, DFArith>::value) o = ieee_of_df(o);
+            psi[x0 + Pm.offs[z]] = o;
         }
     }
 }
@@ -71,6 +102,7 @@ __global__ void __launch_bounds__(kThreads) k_dense_reg(typename P::C* __restric
 struct DenseSmemParams {
     IndexPlan ip;
     uint64_t offs[64];
+    int32_t ieee;  // double-float: the state is read and written as IEEE complex128
 };
 
 template <typename P, int M, int R>
@@ -100,7 +132,12 @@ __global__ void __launch_bounds__(kThreads) k_dense_smem(typename P::C* __restri
         for (int e = threadIdx.x; e < D * G; e += kThreads) {
             const int w = e / G, gg = e % G;
             const uint64_t x0 = xs[gg];
-            if (x0 != ~0ull) tile[e] = psi[x0 + Pm.offs[w]];
+            if (x0 == ~0ull) continue;
+            C v = psi[x0 + Pm.offs[w]];
+            if constexpr (std::is_same<P, DFArith>::value) {
+                if (Pm.ieee) v = df_of_ieee(v);
+            }
+            tile[e] = v;
         }
         __syncthreads();
         const uint64_t x0 = xs[g];
@@ -115,7 +152,13 @@ __global__ void __launch_bounds__(kThreads) k_dense_smem(typename P::C* __restri
                 for (int r = 0; r < R; r++) P::mac(acc[r], Ks[(rc * R + r) * D + w], v);
             }
 #pragma unroll
-            for (int r = 0; r < R; r++) psi[x0 + Pm.offs[rc * R + r]] = P::out(acc[r]);
+            for (int r = 0; r < R; r++) {
+                C o = P::out(acc[r]);
+                if constexpr (std::is_same<P, DFArith>::value) {
+                    if (Pm.ieee) o = ieee_of_df(o);
+                }
+                psi[x0 + Pm.offs[rc * R + r]] = o;
+            }
         }
     }
 }
@@ -406,8 +449,12 @@ struct PauliRotParams {
     IndexPlan ip;
     uint64_t xmask, zmask;
     typename P::K c;      // cos(phi/2)
-    typename P::K kp, km;  // +- i^(1 + nY) sin(phi/2); diagonal case: cos +- i sin
+    typename P::K kp, km;  // +- i^(1 + nY) sin(phi/2), real or imaginary; diagonal case: cos +- i sin
+    int32_t imag;          // kp, km are imaginary
 };
+
+// Two products per real component (c is real, k real or imaginary): 494 -> 324 us at n = 25 in FP64,
+// which the FP64 rate bounds.
 
 template <typename P>
 __global__ void __launch_bounds__(kThreads) k_pauli_rot(typename P::C* __restrict__ psi,
@@ -422,11 +469,8 @@ __global__ void __launch_bounds__(kThreads) k_pauli_rot(typename P::C* __restric
         }
         const uint64_t y2 = y ^ Pm.xmask;
         const C a = psi[y], b = psi[y2];
-        typename P::Acc ra = P::first(Pm.c, a), rb = P::first(Pm.c, b);
-        P::mac(ra, parity64(y2 & Pm.zmask) ? Pm.km : Pm.kp, b);
-        P::mac(rb, parity64(y & Pm.zmask) ? Pm.km : Pm.kp, a);
-        psi[y] = P::out(ra);
-        psi[y2] = P::out(rb);
+        psi[y] = RotMix<P>::mix(Pm.c, parity64(y2 & Pm.zmask) ? Pm.km : Pm.kp, Pm.imag != 0, a, b);
+        psi[y2] = RotMix<P>::mix(Pm.c, parity64(y & Pm.zmask) ? Pm.km : Pm.kp, Pm.imag != 0, b, a);
     }
 }
 
@@ -504,13 +548,33 @@ void fill_offs(const Op& op, uint64_t* offs) {
 }
 
 template <typename P, int M>
-void launch_dense_reg(const Op& op, const IndexPlan& ip, void* psi, cudaStream_t st) {
+void launch_dense_reg(const Op& op, const IndexPlan& ip, void* psi, cudaStream_t st, bool ieee = false) {
+    using C = typename P::C;
     DenseRegParams<P, M> Pm;
     Pm.ip = ip;
+    Pm.form = 0;
+    if (M == 1 && op.data[0].imag() == 0.0 && op.data[3].imag() == 0.0) {
+        if (op.data[1].imag() == 0.0 && op.data[2].imag() == 0.0) Pm.form = 1;
+        else if (op.data[1].real() == 0.0 && op.data[2].real() == 0.0) Pm.form = 2;
+    }
     fill_offs<M>(op, Pm.offs);
     constexpr int D = 1 << M;
     for (int e = 0; e < D * D; e++) Pm.K[e] = P::host_k(op.data[e].real(), op.data[e].imag());
-    k_dense_reg<P, M><<<grid_for(ip.n_iter), kThreads, 0, st>>>(reinterpret_cast<typename P::C*>(psi), Pm);
+    C* p = reinterpret_cast<C*>(psi);
+    const unsigned grid = grid_for(ip.n_iter);
+    if constexpr (std::is_same<P, DFArith>::value) {
+        if (ieee) {
+            k_dense_reg<P, M, true><<<grid, kThreads, 0, st>>>(p, Pm);
+            return;
+        }
+    }
+    if constexpr (std::is_same<P, NativeArith<double>>::value && M == 1) {
+        if (Pm.form) {
+            k_dense_reg<P, M, true><<<grid, kThreads, 0, st>>>(p, Pm);
+            return;
+        }
+    }
+    k_dense_reg<P, M, false><<<grid, kThreads, 0, st>>>(p, Pm);
 }
 
 template <typename P, int M, int R>
@@ -530,9 +594,10 @@ void launch_dense_smem_r(const DenseSmemParams& Pm, void* psi, const void* dK, c
 }
 
 template <typename P, int M>
-void launch_dense_smem(const Op& op, const IndexPlan& ip, void* psi, const void* dK, cudaStream_t st) {
+void launch_dense_smem(const Op& op, const IndexPlan& ip, void* psi, const void* dK, cudaStream_t st, bool ieee) {
     DenseSmemParams Pm;
     Pm.ip = ip;
+    Pm.ieee = ieee ? 1 : 0;
     fill_offs<M>(op, Pm.offs);
     const Arith ar = std::is_same<P, DFArith>::value ? Arith::DF
                      : sizeof(typename P::C) == 8  ? Arith::F32
@@ -545,7 +610,7 @@ void launch_dense_smem(const Op& op, const IndexPlan& ip, void* psi, const void*
 }
 
 template <typename P>
-void launch_with(const Op& op, void* psi, int n, cudaStream_t st, void* stage, bool ieee_in) {
+void launch_with(const Op& op, void* psi, int n, cudaStream_t st, void* stage, bool ieee_in, bool ieee_io = false) {
     using C = typename P::C;
     using K = typename P::K;
     std::vector<int> fixed;
@@ -601,9 +666,9 @@ void launch_with(const Op& op, void* psi, int n, cudaStream_t st, void* stage, b
                 }
                 return launch_dense_oz5(psi, n, os.targets, os.controls, os.cvals, dK, st, ieee_in);
             }
-            if (m == 1) return launch_dense_reg<P, 1>(op, ip, psi, st);
-            if (m == 2) return launch_dense_reg<P, 2>(op, ip, psi, st);
-            if (m == 3) return launch_dense_reg<P, 3>(op, ip, psi, st);
+            if (m == 1) return launch_dense_reg<P, 1>(op, ip, psi, st, ieee_io);
+            if (m == 2) return launch_dense_reg<P, 2>(op, ip, psi, st, ieee_io);
+            if (m == 3) return launch_dense_reg<P, 3>(op, ip, psi, st, ieee_io);
             if (m == 4 && sizeof(C) == 8) return launch_dense_reg<P, 4>(op, ip, psi, st);
             // the shared-memory kernels read the matrix from device memory: either the
             // caller's copy (already in this policy's entry type) or the state's staging
@@ -618,9 +683,9 @@ void launch_with(const Op& op, void* psi, int n, cudaStream_t st, void* stage, b
                 QS_TRY_CUDA(cudaStreamSynchronize(st));  // hk is host memory that dies on return
                 dK = stage;
             }
-            if (m == 4) return launch_dense_smem<P, 4>(op, ip, psi, dK, st);
-            if (m == 5) return launch_dense_smem<P, 5>(op, ip, psi, dK, st);
-            if (m == 6) return launch_dense_smem<P, 6>(op, ip, psi, dK, st);
+            if (m == 4) return launch_dense_smem<P, 4>(op, ip, psi, dK, st, ieee_io);
+            if (m == 5) return launch_dense_smem<P, 5>(op, ip, psi, dK, st, ieee_io);
+            if (m == 6) return launch_dense_smem<P, 6>(op, ip, psi, dK, st, ieee_io);
             throw Error{QS_ERR_UNSUPPORTED, "dense gates act on at most 6 targets"};
         }
         case OpKind::Diag: {
@@ -667,6 +732,7 @@ void launch_with(const Op& op, void* psi, int n, cudaStream_t st, void* stage, b
             Pm.zmask = op.zmask;
             const double c = std::cos(op.angle / 2), sn = std::sin(op.angle / 2);
             Pm.c = P::host_k(c, 0.0);
+            Pm.imag = (1 + __builtin_popcountll(op.xmask & op.zmask)) & 1;
             if (op.xmask) {
                 // i^(1 + nY) sin
                 const int e = (1 + __builtin_popcountll(op.xmask & op.zmask)) & 3;
@@ -714,6 +780,17 @@ void launch_op_arith(const Op& op, void* psi, int n, Arith ar, cudaStream_t st, 
         case Arith::F64: launch_with<NativeArith<double>>(op, psi, n, st, stage, false); break;
         case Arith::DF: launch_with<DFArith>(op, psi, n, st, stage, ieee_in); break;
     }
+    QS_TRY_CUDA(cudaGetLastError());
+}
+
+bool takes_ieee_io(const Op& op) {
+    // (blocks on the tensor cores write the double-float layout)
+    return op.kind == OpKind::Dense && op.controls.empty() && !takes_ieee_in(op);
+}
+
+void launch_op_ieee(const Op& op, void* psi, int n, cudaStream_t st, void* stage) {
+    QS_REQUIRE(takes_ieee_io(op), "the op's double-float kernel does not read and write the IEEE layout");
+    launch_with<DFArith>(op, psi, n, st, stage, false, true);
     QS_TRY_CUDA(cudaGetLastError());
 }
 

@@ -185,6 +185,10 @@ void launch_op(const Op& op, void* psi, int n, qs_dtype dt, cudaStream_t st, voi
 // the double-float layout, the layout change done by the op's own kernel where it reads every
 // amplitude once (takes_ieee_in), else by a conversion pass before it
 void launch_op_arith(const Op& op, void* psi, int n, Arith ar, cudaStream_t st, void* stage, bool ieee_in = false);
+// Ops whose double-float kernel can read and write the IEEE layout itself, every amplitude once: a
+// single op costs one pass instead of three (a conversion on either side).
+bool takes_ieee_io(const Op& op);
+void launch_op_ieee(const Op& op, void* psi, int n, cudaStream_t st, void* stage);
 // Tile shape of the shared-memory dense kernel (4..6 targets on the CUDA cores): output rows per
 // thread, 4, 8 or 16, per device, arithmetic and width; 8 until the autotuner has timed them
 // (tune_dense_tile_rows) or a test has set one.

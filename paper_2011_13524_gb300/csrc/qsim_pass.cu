@@ -330,11 +330,9 @@ __global__ void __launch_bounds__(kPassThreads, 2) k_gate_pass(typename P::C* __
                                 s.put(l2, P::ipow(a, o.mode + 2 * par));
                                 s.put(l, P::ipow(b, o.mode + 2 * par2));
                             } else {  // entries cos, +- i^(1 + nY) sin
-                                typename P::Acc ra = P::first(k[0], a), rb = P::first(k[0], b);
-                                P::mac(ra, k[1 + par2], b);
-                                P::mac(rb, k[1 + par], a);
-                                s.put(l, P::out(ra));
-                                s.put(l2, P::out(rb));
+                                const bool imag = !(o.mode & 1);
+                                s.put(l, RotMix<P>::mix(k[0], k[1 + par2], imag, a, b));
+                                s.put(l2, RotMix<P>::mix(k[0], k[1 + par], imag, b, a));
                             }
                         }
                         break;
