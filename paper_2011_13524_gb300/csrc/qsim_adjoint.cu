@@ -44,139 +44,11 @@ struct GradAcc<NativeArith<float>> {
     __device__ double imag() const { return df_value(im); }
 };
 
-template <>
-struct GradAcc<DFArith> {
-    float s = 0.f, c = 0.f;  // imaginary part only: lx py - ly px
-    __device__ void add(float4 l, float4 p) {
-        DFArith::dprod(s, c, l.x, l.y, p.z, p.w);
-        DFArith::dprod(s, c, -l.z, -l.w, p.x, p.y);
-    }
-    __device__ double imag() const { return double(s) + double(c); }
-};
-
 // the imaginary part of an FP32-pair gradient accumulator as its unevaluated pair (s, c)
-__device__ __forceinline__ void acc_pair(const GradAcc<DFArith>& g, float& s, float& c) {
-    s = g.s;
-    c = g.c;
-}
 __device__ __forceinline__ void acc_pair(const GradAcc<NativeArith<float>>& g, float& s, float& c) {
     s = g.im.hi;
     c = g.im.lo;
 }
-
-// Block sums of NR gradient partials, to part[r * gridDim.x + blockIdx.x]. FP32-pair
-// accumulators are summed as FP32 pairs (TwoSum) across each warp and then across the eight warp
-// sums, and converted to FP64 once per block: on GB300 FP64 warp stages (or a conversion in every
-// lane) cost microseconds per launch. FP64 accumulators keep FP64 sums. One barrier for all NR
-// sums; the order is fixed, so results are reproducible.
-__device__ __forceinline__ void pair_sum_down(float& s, float& c, int o) {
-    const float os = __shfl_down_sync(0xffffffffu, s, o), oc = __shfl_down_sync(0xffffffffu, c, o);
-    float h, e;
-    DFArith::two_sum(s, os, h, e);
-    s = h;
-    c = __fadd_rn(c, __fadd_rn(oc, e));
-}
-template <typename P, int NR>
-__device__ __forceinline__ void grad_block_sums(const GradAcc<P> (&g)[NR], double* part) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    constexpr int W = kAdjThreads / 32;
-    if constexpr (std::is_same<P, NativeArith<double>>::value) {
-        __shared__ double sh[NR][W];
-#pragma unroll
-        for (int r = 0; r < NR; r++) {
-            double v = g[r].imag();
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) sh[r][wid] = v;
-        }
-        __syncthreads();
-        if (wid == 0) {
-#pragma unroll
-            for (int r = 0; r < NR; r++) {
-                double v = lane < W ? sh[r][lane] : 0.0;
-#pragma unroll
-                for (int o = W / 2; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-                if (lane == 0) part[size_t(r) * gridDim.x + blockIdx.x] = v;
-            }
-        }
-    } else {
-        __shared__ float2 sh[NR][W];
-#pragma unroll
-        for (int r = 0; r < NR; r++) {
-            float s, c;
-            acc_pair(g[r], s, c);
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) pair_sum_down(s, c, o);
-            if (lane == 0) sh[r][wid] = make_float2(s, c);
-        }
-        __syncthreads();
-        if (wid == 0) {
-#pragma unroll
-            for (int r = 0; r < NR; r++) {
-                const float2 v = lane < W ? sh[r][lane] : make_float2(0.f, 0.f);
-                float s = v.x, c = v.y;
-#pragma unroll
-                for (int o = W / 2; o > 0; o >>= 1) pair_sum_down(s, c, o);
-                if (lane == 0) part[size_t(r) * gridDim.x + blockIdx.x] = double(s) + double(c);
-            }
-        }
-    }
-}
-
-template <typename P>
-struct AdjRotParams {
-    IndexPlan ip;            // pivot bit = the rotation's qubit
-    uint64_t bit;            // 1 << qubit
-    typename P::K U[4];      // R^+ as a 2x2 matrix, row-major
-    int32_t axis;            // 1 = X, 2 = Y, 3 = Z
-};
-
-template <typename P>
-__global__ void __launch_bounds__(kAdjThreads) k_adj_rot(typename P::C* __restrict__ psi, typename P::C* __restrict__ lam,
-                                                          const __grid_constant__ AdjRotParams<P> A, double* part) {
-    using C = typename P::C;
-    GradAcc<P> g;
-    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-    for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < A.ip.n_iter; i += stride) {
-        const uint64_t i0 = expand(i, A.ip), i1 = i0 | A.bit;
-        const C a = psi[i0], b = psi[i1], la = lam[i0], lb = lam[i1];
-        // (P psi) on the pair: X -> (b, a); Y -> (-i b, i a); Z -> (a, -b)
-        if (A.axis == 1) {
-            g.add(la, b);
-            g.add(lb, a);
-        } else if (A.axis == 2) {
-            g.add(la, P::ipow(b, 3));
-            g.add(lb, P::ipow(a, 1));
-        } else {
-            g.add(la, a);
-            g.add(lb, P::ipow(b, 2));
-        }
-        typename P::Acc r0 = P::zero(), r1 = P::zero(), s0 = P::zero(), s1 = P::zero();
-        P::mac(r0, A.U[0], a); P::mac(r0, A.U[1], b);
-        P::mac(r1, A.U[2], a); P::mac(r1, A.U[3], b);
-        P::mac(s0, A.U[0], la); P::mac(s0, A.U[1], lb);
-        P::mac(s1, A.U[2], la); P::mac(s1, A.U[3], lb);
-        psi[i0] = P::out(r0);
-        psi[i1] = P::out(r1);
-        lam[i0] = P::out(s0);
-        lam[i1] = P::out(s1);
-    }
-    const GradAcc<P> ga[1] = {g};
-    grad_block_sums<P, 1>(ga, part);
-}
-
-// NR consecutive reverse steps (2 to 4) for rotations on distinct qubits q_0 (the latest in the
-// circuit), q_1, ...: each group of 2^NR amplitudes (bits q_0..q_{NR-1}) gets, rotation by
-// rotation in that order, the gradient partial of rotation r and the un-apply of R_r, all in
-// registers. (The rotations commute, so each gradient is the same whichever others are already
-// un-applied.) Partials of rotation r go to part[r grid .. (r + 1) grid).
-template <typename P, int NR>
-struct AdjRotNParams {
-    IndexPlan ip;            // the NR bits inserted
-    uint64_t bit[NR];        // 1 << q_r
-    typename P::K U[NR][4];  // R_r^+
-    int32_t axis[NR];
-};
 
 template <typename P>
 __device__ __forceinline__ void rot_step(typename P::C& a, typename P::C& b, typename P::C& la, typename P::C& lb,
@@ -202,102 +74,242 @@ __device__ __forceinline__ void rot_step(typename P::C& a, typename P::C& b, typ
     lb = P::out(s1);
 }
 
-// The double-float update of a pair by R^+ for X or Y axes, whose entries are real multiples of
-// 1 and i (X: [[c, -i s], [-i s, c]]; Y: [[c, -s], [s, c]]): every output component is a sum of
-// two real products, formed as one double-float dot product (the general 2 x 2 complex form
-// costs twice the products, half of them by zero). Z axes keep the general form.
-__device__ __forceinline__ void df_dot_re(float ah, float al, float bh, float bl, float ch, float cl, float dh,
-                                          float dl, float& h, float& l) {
-    float s, c;
-    DFArith::dprod0(s, c, ah, al, bh, bl);
-    DFArith::dprod(s, c, ch, cl, dh, dl);
-    DFArith::two_sum(s, c, h, l);
-}
-__device__ __forceinline__ void df_rot_pair(float4& a, float4& b, int axis, float ch, float cl, float sh, float sl) {
-    float4 ra, rb;
-    if (axis == 1) {  // a' = c a - i s b, b' = -i s a + c b
-        df_dot_re(ch, cl, a.x, a.y, sh, sl, b.z, b.w, ra.x, ra.y);
-        df_dot_re(ch, cl, a.z, a.w, -sh, -sl, b.x, b.y, ra.z, ra.w);
-        df_dot_re(sh, sl, a.z, a.w, ch, cl, b.x, b.y, rb.x, rb.y);
-        df_dot_re(-sh, -sl, a.x, a.y, ch, cl, b.z, b.w, rb.z, rb.w);
-    } else {  // a' = c a - s b, b' = s a + c b
-        df_dot_re(ch, cl, a.x, a.y, -sh, -sl, b.x, b.y, ra.x, ra.y);
-        df_dot_re(ch, cl, a.z, a.w, -sh, -sl, b.z, b.w, ra.z, ra.w);
-        df_dot_re(sh, sl, a.x, a.y, ch, cl, b.x, b.y, rb.x, rb.y);
-        df_dot_re(sh, sl, a.z, a.w, ch, cl, b.z, b.w, rb.z, rb.w);
+// One thread's partial of a rotation as 8 bytes, and sums of such: FP32 pairs, or an FP64 value for
+// the FP64 policy. (On GB300 FP64 warp stages, or a conversion in every lane, cost microseconds per
+// launch: FP32 pairs stay pairs until one FP64 conversion per block.)
+template <typename P>
+struct GradSlot {
+    using T = float2;
+    __device__ __forceinline__ static T zero() { return make_float2(0.f, 0.f); }
+    __device__ __forceinline__ static T of(const GradAcc<P>& g) {
+        T t;
+        acc_pair(g, t.x, t.y);
+        return t;
     }
-    a = ra;
-    b = rb;
-}
+    __device__ __forceinline__ static T add(T a, T b) {
+        float h, e;
+        DFArith::two_sum(a.x, b.x, h, e);
+        return make_float2(h, __fadd_rn(a.y, __fadd_rn(b.y, e)));
+    }
+    __device__ __forceinline__ static T down(T a, int o) {
+        return make_float2(__shfl_down_sync(0xffffffffu, a.x, o), __shfl_down_sync(0xffffffffu, a.y, o));
+    }
+    __device__ __forceinline__ static double value(T a) { return double(a.x) + double(a.y); }
+};
 template <>
-__device__ __forceinline__ void rot_step<DFArith>(float4& a, float4& b, float4& la, float4& lb, int axis,
-                                                  const float4* U, GradAcc<DFArith>& g) {
-    if (axis == 3) {  // general form
-        g.add(la, a);
-        g.add(lb, DFArith::ipow(b, 2));
-        DFArith::Acc r0 = DFArith::first(U[0], a), r1 = DFArith::first(U[2], a), s0 = DFArith::first(U[0], la),
-                     s1 = DFArith::first(U[2], la);
-        DFArith::mac(r0, U[1], b);
-        DFArith::mac(r1, U[3], b);
-        DFArith::mac(s0, U[1], lb);
-        DFArith::mac(s1, U[3], lb);
-        a = DFArith::out(r0);
-        b = DFArith::out(r1);
-        la = DFArith::out(s0);
-        lb = DFArith::out(s1);
-        return;
+struct GradSlot<NativeArith<double>> {
+    using T = double;
+    __device__ __forceinline__ static T zero() { return 0.0; }
+    __device__ __forceinline__ static T of(const GradAcc<NativeArith<double>>& g) { return g.imag(); }
+    __device__ __forceinline__ static T add(T a, T b) { return a + b; }
+    __device__ __forceinline__ static T down(T a, int o) { return __shfl_down_sync(0xffffffffu, a, o); }
+    __device__ __forceinline__ static double value(T a) { return a; }
+};
+
+// One rotation's reverse step on a pair of a tile: the gradient partial, then R^+ on both buffers.
+template <typename P>
+struct TileRot {
+    using C = typename P::C;
+    using Acc = GradAcc<P>;
+    __device__ __forceinline__ static C order(const C& v) { return v; }  // global <-> tile element
+    __device__ __forceinline__ static void step(C& a, C& b, C& la, C& lb, int axis, const typename P::K* U, Acc& g) {
+        rot_step<P>(a, b, la, lb, axis, U, g);
     }
-    if (axis == 1) {
-        g.add(la, b);
-        g.add(lb, a);
-    } else {
-        g.add(la, DFArith::ipow(b, 3));
-        g.add(lb, DFArith::ipow(a, 1));
+    __device__ __forceinline__ static typename GradSlot<P>::T slot(const Acc& g) { return GradSlot<P>::of(g); }
+};
+// Double-float: tile elements {re_hi, im_hi, re_lo, im_lo}, real and imaginary parts as packed pairs. The
+// entries of R^+ are real multiples of 1 and i (X: [[c, -i s], [-i s, c]]; Y: [[c, -s], [s, c]]), so every
+// component is a sum of two real products.
+template <>
+struct TileRot<DFArith> {
+    using C = float4;
+    struct Acc {
+        float2 s = make_float2(0.f, 0.f), c = make_float2(0.f, 0.f);
+    };
+    __device__ __forceinline__ static C order(const C& v) { return make_float4(v.x, v.z, v.y, v.w); }
+    __device__ __forceinline__ static Pair2 pair(const C& v) { return Pair2{make_float2(v.x, v.y), make_float2(v.z, v.w)}; }
+    __device__ __forceinline__ static Pair2 neg(const Pair2& v) {
+        return Pair2{make_float2(-v.h.x, -v.h.y), make_float2(-v.l.x, -v.l.y)};
     }
-    // c = Re U[0]; s = -Im U[1] (X) or -Re U[1] (Y)
-    const float ch = U[0].x, cl = U[0].y;
-    const float sh = axis == 1 ? -U[1].z : -U[1].x, sl = axis == 1 ? -U[1].w : -U[1].y;
-    df_rot_pair(a, b, axis, ch, cl, sh, sl);
-    df_rot_pair(la, lb, axis, ch, cl, sh, sl);
+    __device__ __forceinline__ static Pair2 conj_swap(const Pair2& v) {  // (im, -re)
+        return Pair2{make_float2(v.h.y, -v.h.x), make_float2(v.l.y, -v.l.x)};
+    }
+    // (df_dot2 gives {re_hi, re_lo, im_hi, im_lo})
+    __device__ __forceinline__ static C dot(float2 xh, float2 xl, const Pair2& a, float2 yh, float2 yl, const Pair2& b) {
+        return order(df_dot2(xh, xl, a, yh, yl, b));
+    }
+    __device__ __forceinline__ static void update(C& a, C& b, int axis, float ch, float cl, float sh, float sl) {
+        const Pair2 va = pair(a), vb = pair(b);
+        const float2 c2 = make_float2(ch, ch), c2l = make_float2(cl, cl);
+        if (axis == 1) {  // a' = c a - i s b, b' = -i s a + c b
+            const float2 s2 = make_float2(sh, -sh), s2l = make_float2(sl, -sl);
+            a = dot(c2, c2l, va, s2, s2l, swapped(vb));
+            b = dot(s2, s2l, swapped(va), c2, c2l, vb);
+        } else {  // a' = c a - s b, b' = s a + c b
+            const float2 s2 = make_float2(sh, sh), s2l = make_float2(sl, sl);
+            const float2 m2 = make_float2(-sh, -sh), m2l = make_float2(-sl, -sl);
+            a = dot(c2, c2l, va, m2, m2l, vb);
+            b = dot(s2, s2l, va, c2, c2l, vb);
+        }
+    }
+    __device__ __forceinline__ static void grad(Acc& g, const Pair2& l, const Pair2& p) {
+        dprod2(g.s, g.c, l.h, l.l, p.h, p.l, false);
+    }
+    __device__ __forceinline__ static void step(C& a, C& b, C& la, C& lb, int axis, const float4* U, Acc& g) {
+        const Pair2 va = pair(a), vb = pair(b), wa = pair(la), wb = pair(lb);
+        if (axis == 1) {  // Im conj(la) b + Im conj(lb) a
+            grad(g, wa, conj_swap(vb));
+            grad(g, wb, conj_swap(va));
+        } else {  // Y psi = (-i b, i a): Re conj(lb) a - Re conj(la) b
+            grad(g, wb, va);
+            grad(g, neg(wa), vb);
+        }
+        // c = Re U[0]; s = -Im U[1] (X) or -Re U[1] (Y)
+        const float ch = U[0].x, cl = U[0].y;
+        const float sh = axis == 1 ? -U[1].z : -U[1].x, sl = axis == 1 ? -U[1].w : -U[1].y;
+        update(a, b, axis, ch, cl, sh, sl);
+        update(la, lb, axis, ch, cl, sh, sl);
+    }
+    __device__ __forceinline__ static float2 slot(const Acc& g) {
+        float h, e;
+        DFArith::two_sum(g.s.x, g.s.y, h, e);
+        return make_float2(h, __fadd_rn(e, __fadd_rn(g.c.x, g.c.y)));
+    }
+};
+
+// Consecutive reverse steps for rotations on distinct qubits q_0 (the latest in the circuit), q_1, ...
+// in one pass: a tile of psi and of lambda (2^t amplitudes each, t <= kAdjTileBits local qubits that
+// hold every q_r) stays in shared memory while, two rotations at a time, each thread takes the gradient
+// partials of a group of four amplitudes and un-applies both rotations in registers. (The rotations
+// commute, so each gradient is the same whichever others are already un-applied.) Partials of rotation r
+// go to part[r grid .. (r + 1) grid).
+// What bounds it: double-float arithmetic (about 110 FP32 operations per amplitude and rotation, on packed
+// pairs) and, per pass, about 20 us of reads, writes and a second wave that is two thirds full (1024
+// tiles on 608 CTA slots at n = 20). A layer of 20 RY rotations at n = 20: ten passes of two rotations
+// 150 us, three passes here 137 us with scalar double-float updates and 124 us with packed pairs (46 us
+// for eight rotations). Four CTAs per SM (64 registers, 150 bytes spilled) and three (85) differ by less
+// than the runs.
+constexpr int kAdjTileBits = 10;
+constexpr int kAdjMaxRot = 10;
+template <typename P>
+struct AdjTileParams {
+    uint64_t n_tiles;
+    uint64_t dep_hi[1 << (kAdjTileBits - 8)];  // address bits of local bits 8..t-1
+    int32_t t, nr;
+    uint8_t lq[kAdjTileBits];                  // local bit -> qubit, ascending
+    uint8_t bit[kAdjMaxRot];                   // local bit of rotation r
+    uint8_t axis[kAdjMaxRot];
+    typename P::K U[kAdjMaxRot][4];            // R_r^+
+};
+
+__device__ __forceinline__ uint32_t adj_insert(uint32_t j, int p) {
+    const uint32_t lo = j & ((1u << p) - 1u);
+    return ((j ^ lo) << 1) | lo;
 }
 
-// Four CTAs per SM (64 registers; a few bytes spill): 8.37 -> 8.05 ms for the n = 20 HEA gradient.
-template <typename P, int NR>
-__global__ void __launch_bounds__(kAdjThreads, 4) k_adj_rotn(typename P::C* __restrict__ psi, typename P::C* __restrict__ lam,
-                                                           const __grid_constant__ AdjRotNParams<P, NR> A, double* part) {
+template <typename P>
+__global__ void __launch_bounds__(kAdjThreads, 4) k_adj_tile(typename P::C* __restrict__ psi, typename P::C* __restrict__ lam,
+                                                             const __grid_constant__ AdjTileParams<P> A, double* part) {
     using C = typename P::C;
-    constexpr int E = 1 << NR;
-    GradAcc<P> g[NR];
-    const uint64_t stride = uint64_t(gridDim.x) * blockDim.x;
-    for (uint64_t i = uint64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < A.ip.n_iter; i += stride) {
-        const uint64_t i0 = expand(i, A.ip);
-        uint64_t ix[E];
-#pragma unroll
-        for (int e = 0; e < E; e++) {
-            uint64_t x = i0;
-#pragma unroll
-            for (int r = 0; r < NR; r++)
-                if ((e >> r) & 1) x |= A.bit[r];
-            ix[e] = x;
+    using R = TileRot<P>;
+    using S = GradSlot<P>;
+    using T = typename S::T;
+    extern __shared__ __align__(16) unsigned char adj_smem[];
+    const uint32_t tid = threadIdx.x, N = 1u << A.t;
+    C* sp = reinterpret_cast<C*>(adj_smem);
+    C* sl = sp + N;
+    T* acc = reinterpret_cast<T*>(sl + N);  // [rotation][thread]
+    for (int r = 0; r < A.nr; r++) acc[r * kAdjThreads + tid] = S::zero();
+    uint64_t off = 0;
+#pragma unroll 1
+    for (int b = 0; b < A.t && b < 8; b++)
+        if ((tid >> b) & 1u) off |= 1ull << A.lq[b];
+    for (uint64_t tile = blockIdx.x; tile < A.n_tiles; tile += gridDim.x) {
+        uint64_t base = tile;
+#pragma unroll 1
+        for (int b = 0; b < A.t; b++) {
+            const uint64_t lo = base & ((1ull << A.lq[b]) - 1ull);
+            base = ((base ^ lo) << 1) | lo;
         }
-        C v[E], l[E];
+        C* gp = psi + (base | off);
+        C* gl = lam + (base | off);
+        constexpr int kU = (1 << kAdjTileBits) / kAdjThreads;
+        {
+            C v[kU], u[kU];
 #pragma unroll
-        for (int e = 0; e < E; e++) {
-            v[e] = psi[ix[e]];
-            l[e] = lam[ix[e]];
+            for (int k = 0; k < kU; k++)
+                if (tid + k * kAdjThreads < N) {
+                    v[k] = gp[A.dep_hi[k]];
+                    u[k] = gl[A.dep_hi[k]];
+                }
+#pragma unroll
+            for (int k = 0; k < kU; k++)
+                if (tid + k * kAdjThreads < N) {
+                    sp[tid + k * kAdjThreads] = R::order(v[k]);
+                    sl[tid + k * kAdjThreads] = R::order(u[k]);
+                }
+        }
+        __syncthreads();
+        for (int r = 0; r < A.nr; r += 2) {
+            if (r + 1 < A.nr) {
+                const int b0 = A.bit[r], b1 = A.bit[r + 1];
+                const int blo = min(b0, b1), bhi = max(b0, b1);
+                if (tid < N / 4) {  // N / 4 <= kAdjThreads
+                    const uint32_t l = adj_insert(adj_insert(tid, blo), bhi);
+                    const uint32_t m0 = 1u << b0, m1 = 1u << b1;
+                    C v[4] = {sp[l], sp[l | m0], sp[l | m1], sp[l | m0 | m1]};
+                    C u[4] = {sl[l], sl[l | m0], sl[l | m1], sl[l | m0 | m1]};
+                    typename R::Acc g0, g1;
+                    R::step(v[0], v[1], u[0], u[1], A.axis[r], A.U[r], g0);
+                    R::step(v[2], v[3], u[2], u[3], A.axis[r], A.U[r], g0);
+                    R::step(v[0], v[2], u[0], u[2], A.axis[r + 1], A.U[r + 1], g1);
+                    R::step(v[1], v[3], u[1], u[3], A.axis[r + 1], A.U[r + 1], g1);
+                    sp[l] = v[0];
+                    sp[l | m0] = v[1];
+                    sp[l | m1] = v[2];
+                    sp[l | m0 | m1] = v[3];
+                    sl[l] = u[0];
+                    sl[l | m0] = u[1];
+                    sl[l | m1] = u[2];
+                    sl[l | m0 | m1] = u[3];
+                    T* a = acc + r * kAdjThreads + tid;
+                    a[0] = S::add(a[0], R::slot(g0));
+                    a[kAdjThreads] = S::add(a[kAdjThreads], R::slot(g1));
+                }
+            } else {
+                const uint32_t m0 = 1u << A.bit[r];
+                typename R::Acc g;
+                for (uint32_t j = tid; j < N / 2; j += kAdjThreads) {
+                    const uint32_t l = adj_insert(j, A.bit[r]);
+                    C a = sp[l], b = sp[l | m0], la = sl[l], lb = sl[l | m0];
+                    R::step(a, b, la, lb, A.axis[r], A.U[r], g);
+                    sp[l] = a;
+                    sp[l | m0] = b;
+                    sl[l] = la;
+                    sl[l | m0] = lb;
+                }
+                T* a = acc + r * kAdjThreads + tid;
+                a[0] = S::add(a[0], R::slot(g));
+            }
+            __syncthreads();
         }
 #pragma unroll
-        for (int r = 0; r < NR; r++)
-#pragma unroll
-            for (int e = 0; e < E; e++)
-                if (!((e >> r) & 1)) rot_step<P>(v[e], v[e | (1 << r)], l[e], l[e | (1 << r)], A.axis[r], A.U[r], g[r]);
-#pragma unroll
-        for (int e = 0; e < E; e++) {
-            psi[ix[e]] = v[e];
-            lam[ix[e]] = l[e];
-        }
+        for (int k = 0; k < kU; k++)
+            if (tid + k * kAdjThreads < N) {
+                gp[A.dep_hi[k]] = R::order(sp[tid + k * kAdjThreads]);
+                gl[A.dep_hi[k]] = R::order(sl[tid + k * kAdjThreads]);
+            }
     }
-    grad_block_sums<P, NR>(g, part);
+    __syncthreads();
+    // rotation r's sum over the block by warp r mod 8, in a fixed order
+    const uint32_t lane = tid & 31u;
+    for (int r = int(tid >> 5); r < A.nr; r += kAdjThreads / 32) {
+        T v = acc[r * kAdjThreads + lane];
+        for (int k = 1; k < kAdjThreads / 32; k++) v = S::add(v, acc[r * kAdjThreads + lane + 32 * k]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v = S::add(v, S::down(v, o));
+        if (lane == 0) part[size_t(r) * gridDim.x + blockIdx.x] = S::value(v);
+    }
 }
 
 // out[s] = sum of part[s * nb .. s * nb + nb) in a fixed order, one block per slot
@@ -506,48 +518,47 @@ void rot_dagger(int axis, double theta, cplx (&U)[4]) {
     else { U[0] = cplx(c, -s); U[1] = 0.0; U[2] = 0.0; U[3] = cplx(c, s); }
 }
 
-template <typename P, int NR>
-void launch_rotn(void* psi, void* lam, int n, const int* qubit, const int* axis, const double* theta, double* part,
+// qubits 0 and 1 always lie in the tile: runs of 64 bytes (double-float)
+uint64_t adj_low(int n) { return (1ull << std::min(n, 2)) - 1; }
+
+template <typename P>
+void launch_tile(void* psi, void* lam, int n, int nr, const int* qubit, const int* axis, const double* theta, double* part,
                  unsigned grid, cudaStream_t st) {
-    AdjRotNParams<P, NR> A;
-    A.ip = make_index_plan(n, std::vector<int>(qubit, qubit + NR), 0);
-    for (int r = 0; r < NR; r++) {
-        A.bit[r] = 1ull << qubit[r];
-        A.axis[r] = axis[r];
+    AdjTileParams<P> A;
+    const int t = std::min(n, kAdjTileBits);
+    uint64_t local = adj_low(n);
+    for (int r = 0; r < nr; r++) local |= 1ull << qubit[r];
+    for (int q = 0; q < n && __builtin_popcountll(local) < t; q++) local |= 1ull << q;
+    QS_REQUIRE(__builtin_popcountll(local) == t, "rotations of a pass on too many qubits");
+    int loc_of[64], k = 0;
+    for (int q = 0; q < n; q++)
+        if ((local >> q) & 1) {
+            loc_of[q] = k;
+            A.lq[k++] = uint8_t(q);
+        }
+    A.t = t;
+    A.nr = nr;
+    A.n_tiles = 1ull << (n - t);
+    for (int h = 0; h < (1 << (kAdjTileBits - 8)); h++) {
+        A.dep_hi[h] = 0;
+        for (int b = 8; b < t; b++)
+            if ((h >> (b - 8)) & 1) A.dep_hi[h] |= 1ull << A.lq[b];
+    }
+    for (int r = 0; r < nr; r++) {
+        A.bit[r] = uint8_t(loc_of[qubit[r]]);
+        A.axis[r] = uint8_t(axis[r]);
         cplx U[4];
         rot_dagger(axis[r], theta[r], U);
         for (int e = 0; e < 4; e++) A.U[r][e] = P::host_k(U[e].real(), U[e].imag());
     }
-    k_adj_rotn<P, NR><<<grid, kAdjThreads, 0, st>>>(reinterpret_cast<typename P::C*>(psi),
-                                                    reinterpret_cast<typename P::C*>(lam), A, part);
-}
-
-// Two rotations per pass: three or four (8 or 16 amplitudes of psi and lambda per thread) were
-// measured slower in every arithmetic at n = 20 (the registers cut the resident warps), so only
-// NR = 2 is instantiated.
-template <typename P>
-void launch_rotn_any(int nr, void* psi, void* lam, int n, const int* qubit, const int* axis, const double* theta,
-                     double* part, unsigned grid, cudaStream_t st) {
-    QS_REQUIRE(nr == 2, "two rotations per pass");
-    launch_rotn<P, 2>(psi, lam, n, qubit, axis, theta, part, grid, st);
-}
-
-template <typename P>
-void launch_rot(void* psi, void* lam, int n, int qubit, int axis, double theta, double* part, unsigned grid,
-                cudaStream_t st) {
-    AdjRotParams<P> A;
-    A.ip = make_index_plan(n, {qubit}, 0);
-    A.bit = 1ull << qubit;
-    A.axis = axis;
-    // R^+ = cos(theta/2) I - i sin(theta/2) P
-    const double c = std::cos(theta / 2), s = std::sin(theta / 2);
-    cplx U[4];
-    if (axis == 1) { U[0] = c; U[1] = cplx(0, -s); U[2] = cplx(0, -s); U[3] = c; }
-    else if (axis == 2) { U[0] = c; U[1] = -s; U[2] = s; U[3] = c; }
-    else { U[0] = cplx(c, -s); U[1] = 0.0; U[2] = 0.0; U[3] = cplx(c, s); }
-    for (int e = 0; e < 4; e++) A.U[e] = P::host_k(U[e].real(), U[e].imag());
-    k_adj_rot<P><<<grid, kAdjThreads, 0, st>>>(reinterpret_cast<typename P::C*>(psi),
-                                               reinterpret_cast<typename P::C*>(lam), A, part);
+    const size_t smem = 2 * (sizeof(typename P::C) << t) + sizeof(typename GradSlot<P>::T) * kAdjThreads * size_t(nr);
+    static PerDevice setup;
+    setup.once([](int) {
+        constexpr size_t most = 2 * (sizeof(typename P::C) << kAdjTileBits) + 8 * kAdjThreads * kAdjMaxRot;
+        QS_TRY_CUDA(cudaFuncSetAttribute(k_adj_tile<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(most)));
+    });
+    k_adj_tile<P><<<grid, kAdjThreads, smem, st>>>(reinterpret_cast<typename P::C*>(psi),
+                                                   reinterpret_cast<typename P::C*>(lam), A, part);
 }
 
 }  // namespace
@@ -560,26 +571,18 @@ unsigned adj_grid(int n) {
     return unsigned(want);
 }
 
-void launch_adjoint_rotation(void* psi, void* lam, int n, Arith ar, int qubit, int axis, double theta, double* part,
-                             unsigned grid, cudaStream_t st) {
-    switch (ar) {
-        case Arith::F32: launch_rot<NativeArith<float>>(psi, lam, n, qubit, axis, theta, part, grid, st); break;
-        case Arith::F64: launch_rot<NativeArith<double>>(psi, lam, n, qubit, axis, theta, part, grid, st); break;
-        case Arith::DF: launch_rot<DFArith>(psi, lam, n, qubit, axis, theta, part, grid, st); break;
-    }
-    QS_TRY_CUDA(cudaGetLastError());
+bool adjoint_rotations_fit(uint64_t qubits, int n) {
+    return __builtin_popcountll(qubits) <= kAdjMaxRot &&
+           __builtin_popcountll(qubits | adj_low(n)) <= std::min(n, kAdjTileBits);
 }
-
-int adjoint_max_rotations(Arith) { return 2; }
 
 void launch_adjoint_rotations(void* psi, void* lam, int n, Arith ar, int nr, const int* qubit, const int* axis,
                               const double* theta, double* part, unsigned grid, cudaStream_t st) {
-    QS_REQUIRE(nr >= 2 && nr <= adjoint_max_rotations(ar), "rotations per pass out of range");
-    QS_REQUIRE(n >= nr, "fewer qubits than rotations");
+    QS_REQUIRE(nr >= 1 && nr <= kAdjMaxRot, "rotations per pass out of range");
     switch (ar) {
-        case Arith::F32: launch_rotn_any<NativeArith<float>>(nr, psi, lam, n, qubit, axis, theta, part, grid, st); break;
-        case Arith::F64: launch_rotn_any<NativeArith<double>>(nr, psi, lam, n, qubit, axis, theta, part, grid, st); break;
-        case Arith::DF: launch_rotn_any<DFArith>(nr, psi, lam, n, qubit, axis, theta, part, grid, st); break;
+        case Arith::F32: launch_tile<NativeArith<float>>(psi, lam, n, nr, qubit, axis, theta, part, grid, st); break;
+        case Arith::F64: launch_tile<NativeArith<double>>(psi, lam, n, nr, qubit, axis, theta, part, grid, st); break;
+        case Arith::DF: launch_tile<DFArith>(psi, lam, n, nr, qubit, axis, theta, part, grid, st); break;
     }
     QS_TRY_CUDA(cudaGetLastError());
 }

@@ -1347,9 +1347,9 @@ qs_status qs_adjoint_grad(const qs_circuit* c, const double* theta, const qs_pau
         return g.param_index >= 0 && g.mc == 0 && (g.named == QS_NAMED_RX || g.named == QS_NAMED_RY);
     };
     struct Step {
-        int kind = 0;               // 0 rotation, 1 diagonal run, 2 other gate, 3 rotations sharing a pass
-        int gate = -1;              // kinds 0, 2
-        std::vector<int> rots;      // kind 3: the rotations, latest first (slots slot0, slot0 + 1, ...)
+        int kind = 0;               // 0 rotations sharing a pass, 1 diagonal run, 2 other gate
+        int gate = -1;              // kinds 0 (its first), 2
+        std::vector<int> rots;      // kind 0: the rotations, latest first (slots slot0, slot0 + 1, ...)
         int slot0 = 0;              // first gradient slot
         std::shared_ptr<AdjDiagParams> diag;  // kind 1 (a few KB: held once, not copied with the step)
         size_t tab_byte = 0;        // kind 1: offset of its tables in the upload
@@ -1536,32 +1536,24 @@ qs_status qs_adjoint_grad(const qs_circuit* c, const double* theta, const qs_pau
                 }
                 flush();
             }
-            // up to adjoint_max_rotations consecutive rotation steps on distinct qubits share one pass
+            // consecutive rotation steps on distinct qubits share a pass as far as its tile holds them
             // (their slots are adjacent)
             {
-                const int maxr = std::min(adjoint_max_rotations(ar), c->n);
                 std::vector<Step> merged;
                 for (size_t i = 0; i < steps.size();) {
-                    if (steps[i].kind != 0 || maxr < 2) {
+                    if (steps[i].kind != 0) {
                         merged.push_back(steps[i++]);
                         continue;
                     }
-                    size_t j = i;
+                    Step m = steps[i];
                     uint64_t used = 0;
-                    while (j < steps.size() && int(j - i) < maxr && steps[j].kind == 0 &&
-                           !((used >> c->gates[steps[j].gate].targets[0]) & 1)) {
-                        used |= 1ull << c->gates[steps[j].gate].targets[0];
-                        j++;
+                    for (; i < steps.size() && steps[i].kind == 0; i++) {
+                        const uint64_t q = 1ull << c->gates[steps[i].gate].targets[0];
+                        if ((used & q) || (used && !adjoint_rotations_fit(used | q, c->n))) break;
+                        used |= q;
+                        m.rots.push_back(steps[i].gate);
                     }
-                    if (j - i >= 2) {
-                        Step m = steps[i];
-                        m.kind = 3;
-                        for (size_t t = i; t < j; t++) m.rots.push_back(steps[t].gate);
-                        merged.push_back(m);
-                    } else {
-                        merged.push_back(steps[i]);
-                    }
-                    i = j > i + 1 ? j : i + 1;
+                    merged.push_back(m);
                 }
                 steps.swap(merged);
             }
@@ -1615,10 +1607,10 @@ qs_status qs_adjoint_grad(const qs_circuit* c, const double* theta, const qs_pau
                 continue;
             }
             const qs_gate& g = c->gates[stp.gate];
-            if (stp.kind == 3) {
+            if (stp.kind == 0) {
                 const int nr = int(stp.rots.size());
-                int q[4], ax[4];
-                double th[4];
+                int q[kAdjMaxRotations], ax[kAdjMaxRotations];
+                double th[kAdjMaxRotations];
                 for (int r = 0; r < nr; r++) {
                     const qs_gate& gr = c->gates[stp.rots[r]];
                     q[r] = gr.targets[0];
@@ -1627,14 +1619,6 @@ qs_status qs_adjoint_grad(const qs_circuit* c, const double* theta, const qs_pau
                     slot_param[stp.slot0 + r] = gr.param_index;
                 }
                 launch_adjoint_rotations(psi->data, lam->data, c->n, ar, nr, q, ax, th, d_part + size_t(stp.slot0) * nb, nb, st);
-                continue;
-            }
-            if (stp.kind == 0) {
-                const int axis = g.named == QS_NAMED_RX ? 1 : 2;
-                const double th = theta ? theta[g.param_index] : g.params[0];
-                launch_adjoint_rotation(psi->data, lam->data, c->n, ar, g.targets[0], axis, th,
-                                        d_part + size_t(stp.slot0) * nb, nb, st);
-                slot_param[stp.slot0] = g.param_index;
                 continue;
             }
             Op op = op_of_gate(g, c->n, theta);

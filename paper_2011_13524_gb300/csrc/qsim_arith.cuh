@@ -291,4 +291,37 @@ struct RotMix<DFArith> {
     }
 };
 
+// Real and imaginary parts side by side in packed FP32 pairs (each lane rounds as the scalar
+// instruction would): the sums of DFArith::mac with half the
+// instructions.
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
+struct Pair2 {
+    float2 h, l;  // (re_hi, im_hi), (re_lo, im_lo)
+};
+__device__ __forceinline__ void dprod2(float2& s, float2& c, float2 ah, float2 al, float2 bh, float2 bl, bool first) {
+    const float2 p = __fmul2_rn(ah, bh);
+    float2 e = __ffma2_rn(ah, bh, make_float2(-p.x, -p.y));
+    e = __ffma2_rn(ah, bl, e);
+    e = __ffma2_rn(al, bh, e);
+    if (first) {
+        s = p;
+        c = e;
+        return;
+    }
+    const float2 t = __fadd2_rn(s, p);
+    const float2 bp = sub2(t, s);
+    const float2 d = __fadd2_rn(sub2(s, sub2(t, bp)), sub2(p, bp));
+    s = t;
+    c = __fadd2_rn(c, __fadd2_rn(d, e));
+}
+__device__ __forceinline__ float4 df_dot2(float2 xh, float2 xl, const Pair2& a, float2 yh, float2 yl, const Pair2& b) {
+    float2 s, c;
+    dprod2(s, c, xh, xl, a.h, a.l, true);
+    dprod2(s, c, yh, yl, b.h, b.l, false);
+    const float2 h = __fadd2_rn(s, c), bp = sub2(h, s);
+    const float2 l = __fadd2_rn(sub2(s, sub2(h, bp)), sub2(c, bp));
+    return make_float4(h.x, l.x, h.y, l.y);
+}
+__device__ __forceinline__ Pair2 swapped(const Pair2& v) { return Pair2{make_float2(v.h.y, v.h.x), make_float2(v.l.y, v.l.x)}; }
+
 }  // namespace qs

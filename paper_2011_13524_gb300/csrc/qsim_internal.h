@@ -376,15 +376,14 @@ void launch_expect_pass(const TileParams& P, const void* psi, Arith ar, double* 
 void launch_apply_observable(const std::vector<PauliGroup>& groups, const void* psi, void* lam, int n,
                              Arith ar, cudaStream_t st);
 
-// Fused adjoint step for an uncontrolled rotation exp(i theta P/2), P = X/Y/Z (axis 1/2/3) on
-// `qubit`: per-block partials of Im <lam|P|psi> into part[0..grid), then psi, lam <- R^+ psi, R^+ lam.
+// Fused adjoint steps for uncontrolled rotations exp(i theta P/2), P = X/Y/Z (axis 1/2/3): per-block
+// partials of Im <lam|P|psi>, then psi, lam <- R^+ psi, R^+ lam.
 unsigned adj_grid(int n);
-void launch_adjoint_rotation(void* psi, void* lam, int n, Arith ar, int qubit, int axis, double theta, double* part,
-                             unsigned grid, cudaStream_t st);
-// nr consecutive rotation steps (2..adjoint_max_rotations(ar), which is 2) on distinct qubits
-// (qubit[0] first, the latest in the circuit), one pass: partials of rotation r into
-// part[r grid .. (r + 1) grid).
-int adjoint_max_rotations(Arith ar);
+// Consecutive rotation steps on distinct qubits (qubit[0] first, the latest in the circuit) in one pass:
+// partials of rotation r into part[r grid .. (r + 1) grid). adjoint_rotations_fit: whether rotations on
+// these qubits share a pass (at most 10, one alone always).
+constexpr int kAdjMaxRotations = 10;
+bool adjoint_rotations_fit(uint64_t qubits, int n);
 void launch_adjoint_rotations(void* psi, void* lam, int n, Arith ar, int nr, const int* qubit, const int* axis,
                               const double* theta, double* part, unsigned grid, cudaStream_t st);
 // Reverse step for a run of diagonal gates on psi and lam (both multiplied by the run's inverse),

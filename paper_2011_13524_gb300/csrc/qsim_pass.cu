@@ -77,29 +77,7 @@ __device__ __forceinline__ void pass_pair(const typename P::K* K, int, typename 
     a = P::out(r0);
     b = P::out(r1);
 }
-// Real and imaginary parts side by side in packed FP32 pairs (each lane rounds as the scalar
-// instruction would), for the general complex update: the sums of DFArith::mac with half the
-// instructions, 92 + 8 register swaps for a pair instead of 172.
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
-struct Pair2 {
-    float2 h, l;  // (re_hi, im_hi), (re_lo, im_lo)
-};
-__device__ __forceinline__ void dprod2(float2& s, float2& c, float2 ah, float2 al, float2 bh, float2 bl, bool first) {
-    const float2 p = __fmul2_rn(ah, bh);
-    float2 e = __ffma2_rn(ah, bh, make_float2(-p.x, -p.y));
-    e = __ffma2_rn(ah, bl, e);
-    e = __ffma2_rn(al, bh, e);
-    if (first) {
-        s = p;
-        c = e;
-        return;
-    }
-    const float2 t = __fadd2_rn(s, p);
-    const float2 bp = sub2(t, s);
-    const float2 d = __fadd2_rn(sub2(s, sub2(t, bp)), sub2(p, bp));
-    s = t;
-    c = __fadd2_rn(c, __fadd2_rn(d, e));
-}
+// The general complex update on packed pairs: 92 + 8 register swaps for a pair instead of 172 instructions.
 __device__ __forceinline__ float4 df_mul_add2(const float4& k0, const float4& k1, const Pair2& a, const Pair2& as,
                                               const Pair2& b, const Pair2& bs) {
     float2 s, c;
@@ -111,20 +89,11 @@ __device__ __forceinline__ float4 df_mul_add2(const float4& k0, const float4& k1
     const float2 l = __fadd2_rn(sub2(s, sub2(h, bp)), sub2(c, bp));
     return make_float4(h.x, l.x, h.y, l.y);
 }
-__device__ __forceinline__ float4 df_dot2(float2 xh, float2 xl, const Pair2& a, float2 yh, float2 yl, const Pair2& b) {
-    float2 s, c;
-    dprod2(s, c, xh, xl, a.h, a.l, true);
-    dprod2(s, c, yh, yl, b.h, b.l, false);
-    const float2 h = __fadd2_rn(s, c), bp = sub2(h, s);
-    const float2 l = __fadd2_rn(sub2(s, sub2(h, bp)), sub2(c, bp));
-    return make_float4(h.x, l.x, h.y, l.y);
-}
 template <>
 __device__ __forceinline__ void pass_pair<DFArith>(const float4* K, int mode, float4& a, float4& b) {
     const Pair2 va{make_float2(a.x, a.z), make_float2(a.y, a.w)}, vb{make_float2(b.x, b.z), make_float2(b.y, b.w)};
     auto dup = [](float f) { return make_float2(f, f); };
     auto mp = [](float f) { return make_float2(-f, f); };
-    auto swapped = [](const Pair2& v) { return Pair2{make_float2(v.h.y, v.h.x), make_float2(v.l.y, v.l.x)}; };
     if (mode == 0) {
         const Pair2 wa = swapped(va), wb = swapped(vb);
         a = df_mul_add2(K[0], K[1], va, wa, vb, wb);

@@ -653,7 +653,8 @@ void ensure_scratch(qs_state* s, size_t part_doubles) {
 
 // final reduce of nslots partials into d_part[out_off..], copy 2 doubles to host, sync
 void finish2(qs_state* s, int nslots, double out[2]) {
-    double* d_out = s->scratch.d_part + s->scratch.part_cap - 2;
+    // (straight into the pinned landing area, which the device can address, where there is one)
+    double* d_out = s->pooled ? s->scratch.d_part + s->scratch.part_cap - 2 : s->scratch.h_out;
     k_final2<<<1, kRedThreads, 0, s->stream>>>(s->scratch.d_part, nslots, d_out);
     QS_TRY_CUDA(cudaGetLastError());
     if (s->pooled) {
@@ -661,7 +662,6 @@ void finish2(qs_state* s, int nslots, double out[2]) {
         QS_TRY_CUDA(cudaStreamSynchronize(s->stream));
         return;
     }
-    QS_TRY_CUDA(cudaMemcpyAsync(s->scratch.h_out, d_out, 2 * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
     QS_TRY_CUDA(cudaStreamSynchronize(s->stream));
     out[0] = s->scratch.h_out[0];
     out[1] = s->scratch.h_out[1];
