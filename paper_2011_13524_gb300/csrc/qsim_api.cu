@@ -197,8 +197,9 @@ void apply_single(qs_state* s, const Op& op) {
 // less than a full pass as launches of their own (one controlled phase, say) is launched gate by
 // gate from the size on where traffic counts more than launches.
 constexpr int kPassTrafficQubits = 18;
-void run_ops(qs_state* s, const std::vector<Op>& ops) {
-    const bool df_run = use_df(s) && !s->df;
+// `fp64`: in IEEE doubles also where double-float is set.
+void run_ops(qs_state* s, const std::vector<Op>& ops, bool fp64 = false) {
+    const bool df_run = use_df(s) && !s->df && !fp64;
     const Arith ar = df_run ? Arith::DF : arith_of(s);
     const std::vector<GatePass> passes = schedule_passes(ops, s->n, ar);
     if (passes.empty()) {  // a double-float run rounds the state to that format whatever its gates
@@ -1306,6 +1307,18 @@ qs_status qs_apply_observable_rotation(qs_state* s, const qs_pauli_obs* H, doubl
     API_END
 }
 
+// A gradient's forward pass in complex128 goes gate by gate in FP64 (several gates per pass,
+// qsim_pass.cu) up to this size, and its result is rounded to double-float once, for the reverse sweep.
+// There the host's work for a fused plan (the partition of a new circuit, every block's matrix and
+// slices) takes longer than all the kernels. Ansatz of 10 layers, first / later calls of a circuit,
+// fused against passes: n = 8 1784 / 846 against 1029 / 524 us, n = 12 2376 / 1116 against 1495 / 769,
+// n = 16 3676 / 1213 against 1943 / 1007; 40 layers at n = 16 9519 / 3562 against 7107 / 3365. At
+// n = 17 and 10 layers later calls are equal (1300 against 1266) and beyond it the blocks win. The
+// gradient's error against 64 bits falls (n = 14, 8 layers, rms: 1.5e-14 to 0.9e-14); passes in
+// double-float took 866 us at n = 16 but raised it to 2.1e-14. complex64 keeps its blocks: in it the
+// order of the roundings shows.
+constexpr int kForwardPassQubits = 16;
+
 qs_status qs_adjoint_grad(const qs_circuit* c, const double* theta, const qs_pauli_obs* H, qs_dtype dt, void* stream,
                           double* energy, double* grad) {
     API_BEGIN
@@ -1336,7 +1349,6 @@ qs_status qs_adjoint_grad(const qs_circuit* c, const double* theta, const qs_pau
         lam->df = 1;
     }
     const Arith ar = arith_of(psi);
-    launch_set_basis_arith(psi->data, c->n, ar, 0, st);
     // The reverse sweep as steps: single-qubit X/Y rotations use the fused reverse step
     // (gradient partials + un-apply in one pass); maximal runs of diagonal gates (CZ, phases,
     // RZ and Z-string rotations, diagonal gates) take one pass for the whole run; other gates
@@ -1575,7 +1587,21 @@ qs_status qs_adjoint_grad(const qs_circuit* c, const double* theta, const qs_pau
                    : ar == Arith::F32 && tensor_c64x_enabled() ? 6
                    : ar == Arith::F32                           ? 4
                                                                 : 2;
-    apply_plan(psi, plan_fusion(c, kf, theta));
+    if (ar != Arith::F32 && c->n <= kForwardPassQubits) {
+        std::vector<Op> ops;
+        ops.reserve(size_t(c->n_gates));
+        for (int i = 0; i < c->n_gates; i++) ops.push_back(op_of_gate(c->gates[i], c->n, theta));
+        psi->df = 0;
+        launch_set_basis_arith(psi->data, c->n, Arith::F64, 0, st);
+        run_ops(psi, ops, true);
+        if (ar == Arith::DF) {
+            launch_to_df(psi->data, c->n, st);
+            psi->df = 1;
+        }
+    } else {
+        launch_set_basis_arith(psi->data, c->n, ar, 0, st);
+        apply_plan(psi, plan_fusion(c, kf, theta));
+    }
     // lambda = H psi ; E = Re <psi|lambda>
     launch_apply_observable(groups, psi->data, lam->data, c->n, ar, st);
     double e2[2];
