@@ -410,13 +410,15 @@ LayoutFold layout_fold(const std::vector<Op>& ops, const std::vector<int>& runs)
     return f;
 }
 
-void apply_plan_impl(qs_state* s, const FusionPlan& p, float* block_ms) {
+// `started` (optional): set once the block matrices are on the device, before the first launch
+void apply_plan_impl(qs_state* s, const FusionPlan& p, float* block_ms, bool* started = nullptr) {
     QS_REQUIRE(p.n == s->n, "plan and state have different qubit counts");
     std::vector<Op> ops;
     ops.reserve(p.blocks.size());
     for (size_t b = 0; b < p.blocks.size(); b++) ops.push_back(block_op(p, b));
     const bool df_run = use_df(s);
     WideMats wm = upload_wide(s, df_run ? Arith::DF : arith_of(s), ops);
+    if (started) *started = true;
     std::vector<cudaEvent_t> ev;
     try {
         const std::vector<int> runs = diag_runs(ops);
@@ -492,11 +494,19 @@ void trotter_by_terms(qs_state* s, const qs_pauli_obs* H, double angle, int n_sl
 // Two slices at n = 26 (complex128): 35.5 ms by terms, 4.4 ms in blocks. From states that no longer
 // fit the 129 MB L2 on; the Ising chain, one slice, by terms / in blocks (planned afresh): 0.92 / 1.04
 // ms at n = 22, 2.15 / 1.35 at n = 23, 4.26 / 1.71 at n = 24 in complex128, 0.99 / 0.95 at n = 23 and
-// 2.35 / 1.19 at n = 24 in complex64 (about 0.7 ms of it host planning and block matrices).
+// 2.35 / 1.19 at n = 24 in complex64 (about 0.7 ms of it host planning and block matrices). The blocks'
+// matrices are copied to the device and waited for, which a stream capture does not allow: there the
+// terms keep their passes, which are launches alone.
 constexpr double kTrotterFuseBytes = 128.0 * (1 << 20);
 constexpr int kTrotterPlanGates = 256;  // gates per plan (slices repeat it): bounds the planning time
 bool trotter_fused(const qs_state* s, const qs_pauli_obs* H, double angle) {
     if (std::ldexp(double(amp_bytes(s->dt)), s->n) < kTrotterFuseBytes) return false;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s->stream, &capture) != cudaSuccess) {
+        cudaGetLastError();  // (the launches report it)
+        return false;
+    }
+    if (capture != cudaStreamCaptureStatusNone) return false;
     for (int k = 0; k < H->n_terms; k++)
         if (!std::isfinite(angle * H->coef[k])) return false;  // no block matrix holds it
     return s->dt == QS_C64 ? tensor_c64x_enabled() : use_df(s) && tensor_c128_enabled();
@@ -543,13 +553,26 @@ void trotter_by_blocks(qs_state* s, const qs_pauli_obs* H, double angle, int n_s
         c.gates = all.data();
         return plan_fusion(&c, 5);
     };
+    // without memory for a plan's block matrices its terms keep their passes, which need none
+    auto apply = [&](const FusionPlan& plan, const std::vector<qs_gate>& gates, int repeat) {
+        bool started = false;
+        try {
+            apply_plan_impl(s, plan, nullptr, &started);
+        } catch (const Error& e) {
+            if (e.code != QS_ERR_OOM || started) throw;
+            std::vector<Op> ops;
+            for (int r = 0; r < repeat; r++)
+                for (const qs_gate& g : gates) ops.push_back(op_of_gate(g, s->n, nullptr));
+            run_ops(s, ops);
+        }
+    };
     if (pieces.size() == 1 && pieces[0].long_term < 0) {  // whole slices, several per plan
         const int per = std::max(1, std::min(n_slices, kTrotterPlanGates / int(pieces[0].gates.size())));
         const FusionPlan plan = plan_of(pieces[0].gates, per);
         const int rest = n_slices % per;
         DFScope df(s, use_df(s) && n_slices > per);  // one plan folds the layout changes into its passes
-        for (int r = 0; r + per <= n_slices; r += per) apply_plan(s, plan);
-        if (rest) apply_plan(s, plan_of(pieces[0].gates, rest));
+        for (int r = 0; r + per <= n_slices; r += per) apply(plan, pieces[0].gates, per);
+        if (rest) apply(plan_of(pieces[0].gates, rest), pieces[0].gates, rest);
         return;
     }
     std::vector<FusionPlan> plans(pieces.size());
@@ -559,7 +582,7 @@ void trotter_by_blocks(qs_state* s, const qs_pauli_obs* H, double angle, int n_s
     for (int r = 0; r < n_slices; r++)
         for (size_t i = 0; i < pieces.size(); i++) {
             if (pieces[i].long_term < 0)
-                apply_plan(s, plans[i]);
+                apply(plans[i], pieces[i].gates, 1);
             else
                 launch_op_arith(trotter_op(H, pieces[i].long_term, angle, n_slices), s->data, s->n, arith_of(s),
                                 s->stream, stage_of(s));
