@@ -1,11 +1,12 @@
-// Fused reverse step of the adjoint gradient for a single-qubit rotation
+// Fused reverse steps of the adjoint gradient: for single-qubit rotations (below) and for runs of
+// diagonal gates (second half of the file). A rotation is
 // R_P(theta) = exp(+i theta P / 2), P in {X, Y, Z} (the paper's gate table sign).
 //
 // At gate j of the reverse sweep psi holds psi_j (the state after the gate) and lambda holds
 // lambda_j = U_{j+1}^+ ... U_G^+ H psi_G. Then dE/dtheta_j = -Im <lambda_j|P|psi_j>; afterwards
-// both buffers are multiplied by R_P(theta)^+. One pass over the qubit's amplitude pairs does
-// both: each pair contributes conj(lambda) * (P psi) to the block's partial sum, then the 2x2
-// adjoint is applied to the pair in psi and in lambda. Per-block partials land in their own
+// both buffers are multiplied by R_P(theta)^+. Both are done pair by pair: each contributes
+// conj(lambda) * (P psi) to the block's partial sum, then the 2x2 adjoint is applied to the pair in
+// psi and in lambda; several rotations share a pass over the state. Per-block partials land in their own
 // slots (deterministic); one final kernel reduces every gate's slots.
 #include <algorithm>
 
@@ -419,6 +420,24 @@ __device__ __forceinline__ float2 kone<float2>() { return make_float2(1.f, 0.f);
 template <>
 __device__ __forceinline__ double2 kone<double2>() { return make_double2(1.0, 0.0); }
 
+// f and sign times factor F at x
+template <typename K>
+__device__ __forceinline__ void adj_diag_factor(const AdjDiagFactor& F, uint64_t x, const K* stab, K& f, int& sign) {
+    if ((x & F.cond_mask) != F.cond_val) return;
+    sign ^= parity64(x & F.zmask);
+    if (F.pair_shift) sign ^= parity64(x & (x >> F.pair_shift) & F.pair_mask);
+    if (F.sign_only) {
+        sign ^= 1;
+    } else if (F.tab_off >= 0) {
+        uint32_t li = 0;
+        for (int b = 0; b < F.nrun; b++) {
+            const uint32_t c = F.run[b];
+            li |= (uint32_t(x >> (c & 0xFFu)) & ((1u << ((c >> 8) & 0xFFu)) - 1u)) << (c >> 16);
+        }
+        f = kmul(f, stab[F.tab_off + int(li)]);
+    }
+}
+
 constexpr int kDiagKA = 4;  // amplitudes per thread between two gradient flushes
 
 // Thread t of T = grid x 256 threads takes the amplitudes x = j T + t, kDiagKA values of j at a
@@ -426,6 +445,10 @@ constexpr int kDiagKA = 4;  // amplitudes per thread between two gradient flushe
 // (Walsh-Hadamard across the lanes), and lane g takes the coefficient at its gradient term's Z
 // bits among the lane bits, with the sign of the rest of the term's Z bits: every term of the
 // run from one transform, so the per-amplitude cost does not grow with the number of gradients.
+// Factors on the bits of t alone (below log2 T) are multiplied once per thread, not per amplitude.
+// What bounds it: instruction issue. A layer's RZ gates and CZ ladder, every factor per amplitude / the
+// low ones per thread: complex128 135 / 86 us at n = 22, complex64 27.5 / 20.4 us at n = 20 (two or four
+// amplitudes per thread up to n = 20: 38 us before there in complex128, a whole 20-layer gradient 5.21 / 5.04 ms).
 template <typename P>
 __global__ void __launch_bounds__(kAdjThreads) k_adj_diag(typename P::C* __restrict__ psi, typename P::C* __restrict__ lam,
                                                            const typename P::K* __restrict__ tab,
@@ -445,6 +468,10 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_diag(typename P::C* __restr
     const uint64_t gz = lane < A.ng ? A.gz[lane] : 0;
     R gsum;  // lane g: this warp's sum for gradient term g
     const uint64_t t0 = t - uint64_t(lane);  // the warp's first thread
+    K f_low = kone<K>();
+    int sign_low = 0;
+#pragma unroll 1
+    for (int k = 0; k < A.nlow; k++) adj_diag_factor(A.f[k], t, stab, f_low, sign_low);
     for (uint64_t j0 = 0; j0 < J; j0 += kDiagKA) {
         R acc[kDiagKA];
 #pragma unroll
@@ -453,25 +480,10 @@ __global__ void __launch_bounds__(kAdjThreads) k_adj_diag(typename P::C* __restr
             if (j0 + j >= J || x >= A.n_amp) continue;
             C p = psi[x], l = lam[x];
             if (A.ng) acc[j] = im_conj_prod(l, p, R());
-            K f = kone<K>();
-            int sign = 0;
+            K f = f_low;
+            int sign = sign_low;
 #pragma unroll 1
-            for (int k = 0; k < A.nf; k++) {
-                const AdjDiagFactor& F = A.f[k];
-                if ((x & F.cond_mask) != F.cond_val) continue;
-                sign ^= parity64(x & F.zmask);
-                if (F.pair_shift) sign ^= parity64(x & (x >> F.pair_shift) & F.pair_mask);
-                if (F.sign_only) {
-                    sign ^= 1;
-                } else if (F.tab_off >= 0) {
-                    uint32_t li = 0;
-                    for (int b = 0; b < F.nrun; b++) {
-                        const uint32_t c = F.run[b];
-                        li |= (uint32_t(x >> (c & 0xFFu)) & ((1u << ((c >> 8) & 0xFFu)) - 1u)) << (c >> 16);
-                    }
-                    f = kmul(f, stab[F.tab_off + int(li)]);
-                }
-            }
+            for (int k = A.nlow; k < A.nf; k++) adj_diag_factor(A.f[k], x, stab, f, sign);
             p = P::out(P::first(f, p));
             l = P::out(P::first(f, l));
             if (sign) {
@@ -587,8 +599,23 @@ void launch_adjoint_rotations(void* psi, void* lam, int n, Arith ar, int nr, con
     QS_TRY_CUDA(cudaGetLastError());
 }
 
-void launch_adjoint_diag(void* psi, void* lam, int n, Arith ar, const void* tab, const AdjDiagParams& A, double* part,
+void launch_adjoint_diag(void* psi, void* lam, int n, Arith ar, const void* tab, const AdjDiagParams& run, double* part,
                          unsigned grid, cudaStream_t st) {
+    AdjDiagParams A = run;
+    const uint64_t T = uint64_t(grid) * kAdjThreads;
+    auto low = [&](const AdjDiagFactor& f) {
+        uint64_t bits = f.cond_mask | f.zmask | f.pair_mask | (f.pair_mask << f.pair_shift);
+        for (int j = 0; j < f.nq; j++) bits |= 1ull << f.q[j];
+        return bits < T;
+    };
+    // (signs commute exactly; in complex64 the tables keep their order, another one would change the
+    // product's last bit)
+    AdjDiagFactor* const end = A.f + A.nf;
+    if (ar == Arith::F32)
+        std::stable_partition(A.f, end, [](const AdjDiagFactor& f) { return f.tab_off >= 0; });
+    else
+        std::stable_partition(A.f, end, low);
+    A.nlow = int(std::find_if_not(A.f, end, low) - A.f);
     const size_t smem = adj_diag_smem(A.ntab, ar);
     switch (ar) {
         case Arith::F32:

@@ -408,7 +408,8 @@ struct AdjDiagFactor {
 };
 struct AdjDiagParams {
     uint64_t n_amp = 0;
-    int32_t nf = 0, ng = 0, ntab = 0, pad = 0;
+    int32_t nf = 0, ng = 0, ntab = 0;
+    int32_t nlow = 0;  // (set by the launch) leading factors that are one value for all of a thread's amplitudes
     AdjDiagFactor f[kAdjDiagMaxF];
     uint64_t gz[kAdjDiagMaxG];
 };
