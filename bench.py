@@ -521,16 +521,15 @@ def measure_extras(args, qs, torch, circuit):
     del stc
     torch.cuda.empty_cache()
     # Pauli rotation of an n-qubit X/Y/Z string (one pass over amplitude pairs), and one Trotter
-    # slice of the transverse-field Ising chain (2n - 1 Pauli rotations), complex128 double-float
+    # slice of the transverse-field Ising chain (2n - 1 Pauli rotations, fused into blocks), complex128
     stp = qs.State(n, qs.QS_C128)
     xm = sum(1 << q for q in range(n) if q % 3 != 2)
     zm = sum(1 << q for q in range(n) if q % 3 != 0)
     ms = timed(lambda: stp.apply_pauli_rotation(xm, zm, 0.3), reps=3)
-    out["pauli_rotation_call_n30_ms"] = ms  # one public call: includes the double-float layout passes
+    out["pauli_rotation_call_n30_ms"] = ms  # one public call (FP64 arithmetic)
     tf = W.tfim_observable(n, 1.0)
     ms = timed(lambda: stp.apply_observable_rotation(tf, 0.1, 1))
     out["tfim_trotter_slice_n30_ms"] = ms
-    out["pauli_rotation_in_trotter_n30_gbps"] = tf.n_terms * 2 * 16 * 2.0 ** n / (ms / 1e3) / 1e9
     del stp
     torch.cuda.empty_cache()
     # analysis calls at n = 30 complex128: transition amplitude of the TFIM observable between two

@@ -447,8 +447,8 @@ constexpr int kDiagKA = 4;  // amplitudes per thread between two gradient flushe
 // run from one transform, so the per-amplitude cost does not grow with the number of gradients.
 // Factors on the bits of t alone (below log2 T) are multiplied once per thread, not per amplitude.
 // What bounds it: instruction issue. A layer's RZ gates and CZ ladder, every factor per amplitude / the
-// low ones per thread: complex128 135 / 86 us at n = 22, complex64 27.5 / 20.4 us at n = 20 (two or four
-// amplitudes per thread up to n = 20: 38 us before there in complex128, a whole 20-layer gradient 5.21 / 5.04 ms).
+// low ones per thread: complex128 38.4 / 28.2 us at n = 20 (926 / 635 instructions per amplitude) and
+// 135 / 86 us at n = 22, complex64 27.5 / 20.4 us at n = 20.
 template <typename P>
 __global__ void __launch_bounds__(kAdjThreads) k_adj_diag(typename P::C* __restrict__ psi, typename P::C* __restrict__ lam,
                                                            const typename P::K* __restrict__ tab,

@@ -6,8 +6,9 @@
 // warps and chunks; the energy is a compensated (double-float) sum.
 //
 // Layout of the work:
-//  * One CTA of 1024 threads per SM claims circuits through an atomic counter, longest first
-//    (the host sorts by estimated cost); nothing waits on another CTA.
+//  * One CTA of 512 threads per SM claims work through atomic counters, longest first (the host
+//    sorts by estimated cost): chunks of the circuits wider than 13 qubits level by level, with a
+//    bounded grid barrier between levels, whole narrower circuits on groups of 1..16 warps.
 //  * A circuit's gates are split on the host into passes. Each pass owns a window of at most
 //    13 "local" qubits and holds gates acting only inside it; a gate joins the earliest pass
 //    after every pass that touched its qubits and that still has room, so the passes applied in
