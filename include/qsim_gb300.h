@@ -400,7 +400,8 @@ qs_status qs_debug_set_tile_rows(qs_dtype dt, int m, int rows);
 qs_status qs_debug_set_wait_limit(long long polls);
 qs_status qs_debug_set_fault(int what);
 /* Every device and pinned-host allocation of the library is counted. qs_debug_fail_alloc makes
- * the allocation after `after` more successful ones fail as if memory had run out (-1: none), so
+ * the allocation after `after` more successful ones fail as if memory had run out (-1: none; the CUDA
+ * runtime is asked for more than any device has, so that its own error state is a real failure's), so
  * that the failing call returns QS_ERR_OOM; *held (optional) receives the number of allocations
  * the library holds now, to check that a failed call freed everything it had allocated. */
 qs_status qs_debug_fail_alloc(long long after, long long* held);

@@ -282,13 +282,25 @@ Op op_of_gate(const qs_gate& g, int n, const double* theta) {
 namespace {
 std::atomic<long long> g_alloc_held{0};
 std::atomic<long long> g_alloc_fail_after{-1};
-// true when this allocation is the one the test hook makes fail
+// true when this allocation is the one the test hook makes fail: a request that no device can meet
+// leaves the runtime as a real failure does (its last error set)
 bool injected_failure() {
     long long k = g_alloc_fail_after.load();
     while (k >= 0) {
-        if (g_alloc_fail_after.compare_exchange_weak(k, k - 1)) return k == 0;
+        if (!g_alloc_fail_after.compare_exchange_weak(k, k - 1)) continue;
+        if (k == 0) {
+            void* none = nullptr;
+            if (cudaMalloc(&none, size_t(1) << 60) == cudaSuccess) cudaFree(none);
+        }
+        return k == 0;
     }
     return false;
+}
+// The caller gets the error. It does not stay the thread's last error, which the check after the
+// next launch would take for that launch's.
+cudaError_t failed(cudaError_t e) {
+    cudaGetLastError();
+    return e;
 }
 }  // namespace
 
@@ -325,18 +337,19 @@ void trim_pools() {
 }
 
 cudaError_t dev_malloc_raw(void** p, size_t bytes) {
-    if (injected_failure()) return cudaErrorMemoryAllocation;
+    if (injected_failure()) return failed(cudaErrorMemoryAllocation);
     cudaError_t e = cudaMalloc(p, bytes);
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         trim_pools();
         e = cudaMalloc(p, bytes);
     }
-    if (e == cudaSuccess) g_alloc_held++;
+    if (e != cudaSuccess) return failed(e);
+    g_alloc_held++;
     return e;
 }
 cudaError_t dev_malloc_async_raw(void** p, size_t bytes, cudaStream_t st) {
-    if (injected_failure()) return cudaErrorMemoryAllocation;
+    if (injected_failure()) return failed(cudaErrorMemoryAllocation);
     const cudaMemPool_t pool = device_pool();
     cudaError_t e = pool ? cudaMallocFromPoolAsync(p, bytes, pool, st) : cudaMallocAsync(p, bytes, st);
     if (e == cudaErrorMemoryAllocation) {
@@ -344,13 +357,15 @@ cudaError_t dev_malloc_async_raw(void** p, size_t bytes, cudaStream_t st) {
         trim_pools();
         e = cudaMallocAsync(p, bytes, st);
     }
-    if (e == cudaSuccess) g_alloc_held++;
+    if (e != cudaSuccess) return failed(e);
+    g_alloc_held++;
     return e;
 }
 cudaError_t host_malloc_pinned_raw(void** p, size_t bytes) {
-    if (injected_failure()) return cudaErrorMemoryAllocation;
+    if (injected_failure()) return failed(cudaErrorMemoryAllocation);
     const cudaError_t e = cudaMallocHost(p, bytes);
-    if (e == cudaSuccess) g_alloc_held++;
+    if (e != cudaSuccess) return failed(e);
+    g_alloc_held++;
     return e;
 }
 cudaError_t dev_free(void* p) {

@@ -210,3 +210,23 @@ def test_allocation_failures_adjoint_and_batch(hooks):
         torch.cuda.synchronize()
 
     assert sweep_allocation_failures(qs, op_batch, cleanup_batch) >= 5
+
+
+def test_a_failed_allocation_leaves_no_error_behind(hooks):
+    """The error of an allocation that failed is the failing call's alone: the caller's next launches, the
+    same state's and another one's, do not report it again."""
+    import torch
+    qs = hooks
+    a, b = qs.State(6, qs.QS_C128), qs.State(6, qs.QS_C128)
+    obs = W.tfim_observable(6, 1.0)
+    ref = b.expectation(obs)[0]
+    qs.check(qs.lib().qs_debug_fail_alloc(0, None))
+    with pytest.raises(qs.QsError) as e:
+        a.expectation(obs)  # allocates its scratch
+    assert e.value.code == qs.QS_ERR_OOM
+    a.apply_gate(W.Gate("X", (0,)))
+    a.apply_gate(W.Gate("X", (0,)))
+    torch.zeros(4, device="cuda").sum().item()
+    assert abs(a.expectation(obs)[0] - ref) < 1e-13
+    a.close()
+    b.close()
