@@ -887,7 +887,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_xsum(const C* __restrict__ 
                 acc_prod2(si, ci, yh, yl, make_float2(wh.y, wh.x), make_float2(wl.y, wl.x));
             }
         }
-        if (e > 115) sr.x = __uint_as_float(0x7FC00000u);  // not finite, or out of FP32's range
+        if (e > 115) sr.x = si.x = __uint_as_float(0x7FC00000u);  // not finite, or out of FP32's range
         accr += (widen_float_int(sr.x) + widen_float_int(sr.y)) + widen_float_int(__fadd_rn(cr.x, cr.y));
         acci += (widen_float_int(si.x) - widen_float_int(si.y)) + widen_float_int(__fsub_rn(ci.x, ci.y));
     }

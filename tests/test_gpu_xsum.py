@@ -71,3 +71,23 @@ def test_against_tiled_reads(dtype):
     assert abs(zero.expectation(same)[0]) < tol  # all tiles but one empty
     for s in (a, b, zero):
         s.close()
+
+
+@pytest.mark.parametrize("dtype", ["c128", "c64"])
+@pytest.mark.parametrize("part", [1.0, 1j])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_not_finite(bad, part, dtype):
+    """One amplitude of the ket that is not finite: neither part of the sum is a number to go on with."""
+    import paper_2011_13524_gb300 as qs
+    n = 14
+    dt = qs.QS_C64 if dtype == "c64" else qs.QS_C128
+    obs = observable(n, [(0.5, 1 << i, 0) for i in range(n)])
+    a, b = qs.State(n, dt), qs.State(n, dt)
+    v = W.random_state_fast(n, 2)
+    v[5000] = complex(bad, 0.25) if part == 1.0 else complex(0.25, bad)
+    a.load(W.random_state_fast(n, 1))
+    b.load(v)
+    t = a.transition_amplitude(obs, b)
+    assert not np.isfinite(t.real) and not np.isfinite(t.imag)
+    a.close()
+    b.close()
