@@ -322,7 +322,8 @@ qs_status qs_expectation_noalloc(const void* dev_psi, int n, qs_dtype dt, void* 
 /* out = <a|b> (Sec. 4.2.2 inner_product) as (re, im); same n and dtype; synchronises. */
 qs_status qs_inner_product(const qs_state* a, const qs_state* b, double out[2]);
 /* Transition amplitude of an observable (Sec. 4.5): out = <bra|H|ket> = sum_k coef_k
- * <bra|P_k|ket> as (re, im), FP64 sums. Both states must have the same n and dtype. */
+ * <bra|P_k|ket> as (re, im), in double-float sums and products (complex128 components cut at 2^-46 of
+ * themselves) with FP64 sums over tiles. Both states must have the same n and dtype. */
 qs_status qs_transition_amplitude(const qs_state* bra, const qs_pauli_obs* H, const qs_state* ket, double out[2]);
 /* Marginal probability (Sec. 4.2.2): measured_value[q] for every qubit q is 0, 1 or 2
  * (2 = any value); out = sum of |psi_x|^2 over the x that match (not divided by the norm).

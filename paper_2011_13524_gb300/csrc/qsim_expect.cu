@@ -711,92 +711,62 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_transition_tiled(const C* _
 // A tile of 2^12 amplitudes of ket in shared memory and, per thread, its own 16 (tile-local index
 // tid + 256 k) in registers; w_y = sum_f ket_{y ^ f} by additions, then conj(bra_y) w_y once per
 // amplitude.
-// Every component is an integer F of 51 bits on one grid per tile, 2^-49 of the power of two below the
-// tile's largest component, held as F = 2^23 I + L: I sums exactly as a 32-bit integer (|I| <= 2^27, up
-// to 12 strings), L (0 <= L < 2^23) as a float, one integer addition per part and two strings (three
-// operands) and one packed FP32 addition per string. The sum becomes a double-float pair (24 bits and
-// a rest) for the product: its error is 2^-45 of the tile's largest component.
-// What bounds it: instruction issue, most of it per amplitude (reading, fixing and splitting, one complex
-// product), 2 to 3.3 per string, where the products of k_transition_tiled take 40 per string. The Ising
-// chain's 26 X terms at n = 26 (complex128): 0.59, 0.54 and 0.50 ms for 12, 9 and 5 strings, with the
-// diagonal terms' read (0.99 ms) 2.6 ms against 4.8 ms in tiled reads. Error of the chain's amplitude on
-// random states, rms: 2.3e-15 against 6.4e-15 at n = 12 (1.2e-15 / 2.4e-15 at n = 15). Cutting on an FP32
-// grid instead (20 bits and a rest) measured the same time and 2.0e-14. For expectations, whose pair
-// products take 12.5 per string, it gained 8 % and is not used.
-__device__ __forceinline__ uint32_t magnitude_bits(double2 v) {
-    return max(uint32_t(__double2hiint(v.x)) & 0x7FFFFFFFu, uint32_t(__double2hiint(v.y)) & 0x7FFFFFFFu);
-}
-__device__ __forceinline__ uint32_t magnitude_bits(float2 v) {
-    return max(__float_as_uint(v.x) & 0x7FFFFFFFu, __float_as_uint(v.y) & 0x7FFFFFFFu);
-}
-__device__ __forceinline__ int magnitude_exponent(uint32_t m, double2) { return int(m >> 20) - 1023; }
-__device__ __forceinline__ int magnitude_exponent(uint32_t m, float2) { return int(m >> 23) - 127; }
-__device__ __forceinline__ float4 split_pair(double2 v) { return to_tile(v); }
-__device__ __forceinline__ float4 split_pair(float2 v) { return make_float4(v.x, v.y, 0.f, 0.f); }
+// The sums are floating: a component enters as k_transition_tiled holds it (24 bits and a rest of 23,
+// complex64 as it is), each addition is a TwoSum whose error joins the rests, eight packed FP32
+// instructions per string and amplitude (seven in complex64) where the products take 40. Whatever else
+// the tile holds, w_y keeps 2^-45 of the components it is the sum of.
+// What bounds it: the FP32 pipe. Norms, inner product and the Ising chain's amplitude at n = 26
+// (complex128): 5.94 ms with the X terms in tiled reads, 4.25 ms here, about 2.0 of them for 26 strings.
+// Error of the amplitude on random states, rms: 2.3e-15 against 6.4e-15 at n = 12 (1.2e-15 / 2.4e-15 at
+// n = 15; complex64 2.2e-15 / 5.3e-15 and 1.0e-15 / 2.3e-15). Sums on one fixed-point grid per tile took 0.35
+// ms less, but a component's error was then 2^-49 of the tile's largest: beside an amplitude of 1, one of
+// 2^-40 was 20 % off.
+__device__ __forceinline__ float2 tile_hi(float4 v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 tile_lo(float4 v) { return make_float2(v.z, v.w); }
+__device__ __forceinline__ float2 tile_hi(float2 v) { return v; }
+__device__ __forceinline__ float2 tile_lo(float2) { return make_float2(0.f, 0.f); }
 
-// x = (2^23 I + L) 2^(e - 49) truncated, for |x| < 2^(e + 1); eb = e + 1023
-__device__ __forceinline__ void fix_mantissa(uint32_t sign, uint32_t ex, uint64_t man53, int eb, int& I, float& L) {
-    const int sh = min(eb + 3 - int(ex), 63);  // man53 2^(ex - 1075) in units of 2^(e - 49)
-    const long long s = static_cast<long long>(int(sign) >> 31);
-    const long long F = (static_cast<long long>(man53 >> sh) ^ s) - s;
-    const uint32_t lo = uint32_t(F), hi = uint32_t(uint64_t(F) >> 32);
-    I = int(__funnelshift_r(lo, hi, 23));
-    L = __fsub_rn(__uint_as_float((lo & 0x7FFFFFu) | 0x4B000000u), 8388608.f);
-}
-__device__ __forceinline__ void fix_point(double x, int eb, int& I, float& L) {
-    const uint32_t h = uint32_t(__double2hiint(x));
-    const uint32_t ex = (h >> 20) & 0x7FFu;
-    fix_mantissa(h, ex, (uint64_t((h & 0xFFFFFu) | 0x100000u) << 32) | uint32_t(__double2loint(x)), eb, I, L);
-}
-__device__ __forceinline__ void fix_point(float x, int eb, int& I, float& L) {
-    const uint32_t u = __float_as_uint(x), f = (u >> 23) & 0xFFu;
-    // (a subnormal keeps its bits without the implicit one)
-    const uint32_t man = (u & 0x7FFFFFu) | (f ? 0x800000u : 0u);
-    fix_mantissa(u, (f ? f : 1u) + 896u, uint64_t(man) << 29, eb, I, L);
-}
-
-// (2^23 I + L) 2^(e - 49) as a double-float pair, both parts of an amplitude side by side; su = 2^(e - 26)
-__device__ __forceinline__ void fixed_to_pair(int2 I, float2 L, float su, float2& h, float2& l) {
+// h + e = a + b exactly, lane by lane
+__device__ __forceinline__ float2 two_sum_pair(float2 a, float2 b, float2& e) {
     const float2 m1 = make_float2(-1.f, -1.f);
-    const float2 fa = __fadd2_rn(make_float2(__int_as_float((I.x >> 11) + 0x4B400000), __int_as_float((I.y >> 11) + 0x4B400000)),
-                                 make_float2(-12582912.f, -12582912.f));
-    const float2 fb = __fadd2_rn(make_float2(__int_as_float((I.x & 0x7FF) | 0x4B000000), __int_as_float((I.y & 0x7FF) | 0x4B000000)),
-                                 make_float2(-8388608.f, -8388608.f));
-    const float2 k = make_float2(2048.f, 2048.f);
-    const float2 w = __ffma2_rn(fa, k, fb);                       // RN(I)
-    const float2 t = __ffma2_rn(fa, make_float2(-2048.f, -2048.f), w);  // exact
-    const float2 rest = __ffma2_rn(t, m1, fb);                    // I - w, exact
-    const float2 low = __ffma2_rn(rest, make_float2(8388608.f, 8388608.f), L);  // units of 2^(e - 49)
-    const float sl = su * 1.1920928955078125e-07f;
-    h = __fmul2_rn(w, make_float2(su, su));
-    l = __fmul2_rn(low, make_float2(sl, sl));
+    const float2 h = __fadd2_rn(a, b);
+    const float2 bp = __ffma2_rn(a, m1, h);
+    e = __fadd2_rn(__ffma2_rn(__ffma2_rn(bp, m1, h), m1, a), __ffma2_rn(bp, m1, b));
+    return h;
+}
+// (s, c) += x
+__device__ __forceinline__ void acc_sum2(float2& s, float2& c, float4 x) {
+    float2 e;
+    s = two_sum_pair(s, tile_hi(x), e);
+    c = __fadd2_rn(c, __fadd2_rn(tile_lo(x), e));
+}
+__device__ __forceinline__ void acc_sum2(float2& s, float2& c, float2 x) {
+    float2 e;
+    s = two_sum_pair(s, x, e);
+    c = __fadd2_rn(c, e);
 }
 
 // (s, c) += (ah + al) * (bh + bl) lane by lane
 __device__ __forceinline__ void acc_prod2(float2& s, float2& c, float2 ah, float2 al, float2 bh, float2 bl) {
-    const float2 m1 = make_float2(-1.f, -1.f);
     const float2 p = __fmul2_rn(ah, bh);
-    float2 e = __ffma2_rn(ah, bh, make_float2(-p.x, -p.y));
+    float2 e = __ffma2_rn(ah, bh, make_float2(-p.x, -p.y)), d;
     e = __ffma2_rn(ah, bl, e);
     e = __ffma2_rn(al, bh, e);
-    e = __ffma2_rn(al, bl, e);  // (the low parts of w are not centred: their products do not average out)
-    const float2 t = __fadd2_rn(s, p);
-    const float2 bp = __ffma2_rn(s, m1, t);
-    const float2 d = __fadd2_rn(__ffma2_rn(__ffma2_rn(bp, m1, t), m1, s), __ffma2_rn(bp, m1, p));
-    s = t;
+    e = __ffma2_rn(al, bl, e);  // (the rests of w are not centred: their products do not average out)
+    s = two_sum_pair(s, p, d);
     c = __fadd2_rn(c, __fadd2_rn(d, e));
 }
 
 template <typename C>
 __global__ void __launch_bounds__(kTileThreads, 2) k_xsum(const C* __restrict__ ket, const C* __restrict__ bra,
                                                           const __grid_constant__ XsumParams P, double* __restrict__ part) {
+    using T = decltype(to_tile(C()));
     constexpr int K = kTileAmps / kTileThreads;
     constexpr int kParts = 4;  // the thread's amplitudes are summed and multiplied K / kParts at a time
     extern __shared__ __align__(16) unsigned char tsm[];
-    float4* tile = reinterpret_cast<float4*>(tsm);
-    __shared__ uint32_t smax[kTileThreads / 32];
+    T* tile = reinterpret_cast<T*>(tsm);
     __shared__ double sh[kTileThreads / 32];
-    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
+    const uint32_t tid = threadIdx.x;
     uint64_t dthr = 0;
 #pragma unroll
     for (int i = 0; i < 8; i++)
@@ -808,26 +778,14 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_xsum(const C* __restrict__ 
         const uint64_t at = rbase | dthr;
         rbase = ((rbase | ~P.rest_mask) + step) & P.rest_mask;
         C v[K];
-        uint32_t m = 0;
+        T own[K];
 #pragma unroll
         for (int k = 0; k < K; k++) v[k] = ket[at | P.dep_hi[k]];
-#pragma unroll
-        for (int k = 0; k < K; k++) m = max(m, magnitude_bits(v[k]));
-        m = __reduce_max_sync(0xffffffffu, m);
-        if (lane == 0) smax[warp] = m;
-        __syncthreads();  // (and the previous tile's readers are done)
-#pragma unroll
-        for (int w = 0; w < kTileThreads / 32; w++) m = max(m, smax[w]);
-        const int e = max(magnitude_exponent(m, v[0]), -90);  // largest component below 2^(e + 1)
-        const float su = __uint_as_float(uint32_t(min(e, 115) - 26 + 127) << 23);
-        int2 I[K];
-        float2 L[K];
+        __syncthreads();  // the previous tile's readers are done
 #pragma unroll
         for (int k = 0; k < K; k++) {
-            fix_point(v[k].x, e + 1023, I[k].x, L[k].x);
-            fix_point(v[k].y, e + 1023, I[k].y, L[k].y);
-            tile[tid + kTileThreads * k] =
-                make_float4(__int_as_float(I[k].x), __int_as_float(I[k].y), L[k].x, L[k].y);
+            own[k] = to_tile(v[k]);
+            tile[tid + kTileThreads * k] = own[k];
         }
         __syncthreads();
         float2 sr = make_float2(0.f, 0.f), cr = sr, si = sr, ci = sr;
@@ -837,57 +795,30 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_xsum(const C* __restrict__ 
             C b[kH];
 #pragma unroll
             for (int j = 0; j < kH; j++) b[j] = bra[at | P.dep_hi[hf * kH + j]];
-            int2 WI[kH];
-            float2 WL[kH];
+            float2 ws[kH], wc[kH];
 #pragma unroll
-            for (int j = 0; j < kH; j++) {
-                WI[j] = make_int2(0, 0);
-                WL[j] = make_float2(0.f, 0.f);
-            }
+            for (int j = 0; j < kH; j++) ws[j] = wc[j] = make_float2(0.f, 0.f);
 #pragma unroll
             for (int q = 0; q < 4; q++)
                 if ((P.item >> q) & 1u) {
 #pragma unroll
-                    for (int j = 0; j < kH; j++) {
-                        WI[j].x += I[(hf * kH + j) ^ (1 << q)].x;
-                        WI[j].y += I[(hf * kH + j) ^ (1 << q)].y;
-                        WL[j] = __fadd2_rn(WL[j], L[(hf * kH + j) ^ (1 << q)]);
-                    }
+                    for (int j = 0; j < kH; j++) acc_sum2(ws[j], wc[j], own[(hf * kH + j) ^ (1 << q)]);
                 }
-            int g = 0;
-            for (; g + 1 < P.nf; g += 2) {
-                const uint32_t o = tid ^ P.f[g], p = tid ^ P.f[g + 1];
-#pragma unroll
-                for (int j = 0; j < kH; j++) {
-                    const float4 x = tile[o ^ uint32_t(kTileThreads * (hf * kH + j))];
-                    const float4 y = tile[p ^ uint32_t(kTileThreads * (hf * kH + j))];
-                    WI[j].x += __float_as_int(x.x) + __float_as_int(y.x);
-                    WI[j].y += __float_as_int(x.y) + __float_as_int(y.y);
-                    WL[j] = __fadd2_rn(WL[j], __fadd2_rn(make_float2(x.z, x.w), make_float2(y.z, y.w)));
-                }
-            }
-            if (g < P.nf) {
+            for (int g = 0; g < P.nf; g++) {
                 const uint32_t o = tid ^ P.f[g];
 #pragma unroll
-                for (int j = 0; j < kH; j++) {
-                    const float4 x = tile[o ^ uint32_t(kTileThreads * (hf * kH + j))];
-                    WI[j].x += __float_as_int(x.x);
-                    WI[j].y += __float_as_int(x.y);
-                    WL[j] = __fadd2_rn(WL[j], make_float2(x.z, x.w));
-                }
+                for (int j = 0; j < kH; j++) acc_sum2(ws[j], wc[j], tile[o ^ uint32_t(kTileThreads * (hf * kH + j))]);
             }
 #pragma unroll
             for (int j = 0; j < kH; j++) {
-                float2 wh, wl;
-                fixed_to_pair(WI[j], WL[j], su, wh, wl);
+                float2 wl;
+                const float2 wh = two_sum_pair(ws[j], wc[j], wl);
                 // conj(b) w = (b.re w.re + b.im w.im) + i (b.re w.im - b.im w.re)
-                const float4 y = split_pair(b[j]);
-                const float2 yh = make_float2(y.x, y.y), yl = make_float2(y.z, y.w);
-                acc_prod2(sr, cr, yh, yl, wh, wl);
-                acc_prod2(si, ci, yh, yl, make_float2(wh.y, wh.x), make_float2(wl.y, wl.x));
+                const T y = to_tile(b[j]);
+                acc_prod2(sr, cr, tile_hi(y), tile_lo(y), wh, wl);
+                acc_prod2(si, ci, tile_hi(y), tile_lo(y), make_float2(wh.y, wh.x), make_float2(wl.y, wl.x));
             }
         }
-        if (e > 115) sr.x = si.x = __uint_as_float(0x7FC00000u);  // not finite, or out of FP32's range
         accr += (widen_float_int(sr.x) + widen_float_int(sr.y)) + widen_float_int(__fadd_rn(cr.x, cr.y));
         acci += (widen_float_int(si.x) - widen_float_int(si.y)) + widen_float_int(__fsub_rn(ci.x, ci.y));
     }
@@ -1345,13 +1276,17 @@ std::vector<PauliGroup> split_xsum(const std::vector<PauliGroup>& groups, int n,
 }
 
 namespace {
+template <typename C>
+constexpr size_t xsum_tile_bytes() {
+    return 2 * sizeof(float) * kTileAmps * (sizeof(C) / 8);
+}
 // CTAs per SM of k_xsum (attribute raised once per device)
 template <typename C>
 int xsum_blocks_per_sm() {
     static PerDevice setup;
     static int b[kMaxDevices];
     setup.once([](int dev) {
-        const size_t bytes = sizeof(float4) * kTileAmps;
+        const size_t bytes = xsum_tile_bytes<C>();
         QS_TRY_CUDA(cudaFuncSetAttribute(k_xsum<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)));
         int nb = 0;
         QS_TRY_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_xsum<C>, kTileThreads, bytes));
@@ -1361,7 +1296,7 @@ int xsum_blocks_per_sm() {
 }
 template <typename C>
 void launch_xsum_t(const XsumParams& P, const void* bra, const void* ket, double* part, unsigned grid, cudaStream_t st) {
-    const size_t bytes = sizeof(float4) * kTileAmps;
+    const size_t bytes = xsum_tile_bytes<C>();
     xsum_blocks_per_sm<C>();
     k_xsum<C><<<grid, kTileThreads, bytes, st>>>(static_cast<const C*>(ket), static_cast<const C*>(bra), P, part);
     QS_TRY_CUDA(cudaGetLastError());

@@ -91,3 +91,38 @@ def test_not_finite(bad, part, dtype):
     assert not np.isfinite(t.real) and not np.isfinite(t.imag)
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("dtype", ["c128", "c64"])
+@pytest.mark.parametrize("orders", [10, 40, 90])
+def test_small_components_beside_large_ones(orders, dtype):
+    """Ket amplitudes over many binary orders within one tile, read out one by one: each sum keeps its own
+    accuracy. The bound: components cut at 2^-46 of themselves (complex64: exact), at most 13 of them summed
+    with an error of 2^-47 of their magnitudes per addition, one product."""
+    import paper_2011_13524_gb300 as qs
+    n = 14
+    dt = qs.QS_C64 if dtype == "c64" else qs.QS_C128
+    obs = observable(n, [(1.0, 1 << i, 0) for i in range(n)])
+    a, b = qs.State(n, dt), qs.State(n, dt)
+    order = (np.arange(1 << n) * 2654435761 >> 7) % (orders + 1)
+    b.load(W.random_state_fast(n, 3) * 2.0 ** (7.0 - order))
+    ket = b.get_vector().astype(np.clongdouble)
+    for y in (0, 1, 255, 256, 4095, 4096, 9999, (1 << n) - 1):
+        near = ket[[y ^ (1 << i) for i in range(n)]]
+        bra = np.zeros(1 << n, dtype=np.complex128)
+        bra[y] = 1.0
+        a.load(bra)
+        err = abs(np.clongdouble(a.transition_amplitude(obs, b)) - near.sum())
+        assert err < 2.0 ** -42 * np.abs(near).sum()
+    # a small answer beside amplitudes of 1 that it does not read
+    small = W.random_state_fast(n, 4) * 2.0 ** -orders
+    small[[4095, (1 << n) - 1]] = 1.0
+    b.load(small)
+    ket = b.get_vector().astype(np.clongdouble)
+    near = ket[[1 << i for i in range(n)]]
+    bra = np.zeros(1 << n, dtype=np.complex128)
+    bra[0] = 1.0
+    a.load(bra)
+    assert abs(np.clongdouble(a.transition_amplitude(obs, b)) - near.sum()) < 2.0 ** -42 * np.abs(near).sum()
+    a.close()
+    b.close()
