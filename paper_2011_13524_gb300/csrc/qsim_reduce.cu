@@ -12,6 +12,7 @@
 // (y, y ^ f) once, with A = conj(psi_{y^f}) psi_y:
 //   <psi|P|psi> restricted to the pair = i^{#Y} (s(y) A + s(y^f) conj(A)).
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -864,19 +865,13 @@ void reduce_pauli_transition(qs_state* lam, const qs_state* psi, uint64_t xmask,
     finish2(lam, int(g), out);
 }
 
-void reduce_transition(const qs_state* bra, const qs_pauli_obs* obs, const qs_state* ket, double out[2]) {
+namespace {
+// <bra|O|ket> of the X strings `xsum` and the groups `rest`
+void transition_sum(const qs_state* bra, const std::vector<XsumParams>& xsum, const std::vector<PauliGroup>& rest,
+                    const qs_state* ket, double out[2]) {
     qs_state* s = const_cast<qs_state*>(bra);
-    const std::vector<PauliGroup> groups = group_observable(obs, s->n);
     const uint64_t N = 1ull << s->n;
-    QS_REQUIRE(arith_of(bra) == arith_of(ket), "states in different layouts");
-    if (ket->stream != s->stream) QS_TRY_CUDA(cudaStreamSynchronize(ket->stream));
-    if (groups.empty()) {
-        out[0] = out[1] = 0.0;
-        return;
-    }
     const Arith ar = arith_of(s);
-    std::vector<XsumParams> xsum;
-    const std::vector<PauliGroup> rest = split_xsum(groups, s->n, ar, xsum);
     const ExpectPlan plan = rest.empty() ? ExpectPlan() : plan_transition(rest, s->n);
     std::vector<unsigned> grids, xgrids;
     size_t slots_needed = 0;
@@ -921,6 +916,24 @@ void reduce_transition(const qs_state* bra, const qs_pauli_obs* obs, const qs_st
         slots += gr;
     }
     finish2(s, int(slots), out);
+}
+}  // namespace
+
+void reduce_transition(const qs_state* bra, const qs_pauli_obs* obs, const qs_state* ket, double out[2]) {
+    const qs_state* s = bra;
+    const std::vector<PauliGroup> groups = group_observable(obs, s->n);
+    QS_REQUIRE(arith_of(bra) == arith_of(ket), "states in different layouts");
+    if (ket->stream != s->stream) QS_TRY_CUDA(cudaStreamSynchronize(ket->stream));
+    if (groups.empty()) {
+        out[0] = out[1] = 0.0;
+        return;
+    }
+    std::vector<XsumParams> xsum;
+    const std::vector<PauliGroup> rest = split_xsum(groups, s->n, arith_of(s), xsum);
+    transition_sum(bra, xsum, rest, ket, out);
+    // ket components summed before their product with bra can leave FP32's range (from 2^124 on) where
+    // the products do not: a result that is not finite is the tiled reads' to give
+    if (!xsum.empty() && !(std::isfinite(out[0]) && std::isfinite(out[1]))) transition_sum(bra, {}, groups, ket, out);
 }
 
 void reduce_marginal(const qs_state* st, const int32_t* measured, double* out) {

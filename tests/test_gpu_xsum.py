@@ -126,3 +126,20 @@ def test_small_components_beside_large_ones(orders, dtype):
     assert abs(np.clongdouble(a.transition_amplitude(obs, b)) - near.sum()) < 2.0 ** -42 * np.abs(near).sum()
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("dtype", ["c128", "c64"])
+def test_sums_beyond_the_range(dtype):
+    """Ket components whose sums, not whose products with the bra, leave FP32's range."""
+    import paper_2011_13524_gb300 as qs
+    n = 14
+    dt = qs.QS_C64 if dtype == "c64" else qs.QS_C128
+    obs = observable(n, [(1.0, 1 << i, 0) for i in range(n)])
+    a, b = qs.State(n, dt), qs.State(n, dt)
+    a.load(W.random_state_fast(n, 1) * 1e-25)
+    b.load(np.full(1 << n, 3e38 - 2.5e38j))
+    va, vb = a.get_vector().astype(np.complex128), b.get_vector().astype(np.complex128)
+    t = a.transition_amplitude(obs, b)
+    assert abs(t - oracle.transition_amplitude(va, vb, n, obs)) < 1e-13 * n * float(np.sum(np.abs(va)) * np.abs(vb[0]))
+    a.close()
+    b.close()
