@@ -291,8 +291,9 @@ qs_status qs_dense_tile_rows(qs_dtype dt, int m, int* rows, int* tuned);
  * read of the state evaluates every group whose mask lies in a tile of 12 qubits (qubits 0..2
  * plus up to 9 others), in double-float arithmetic with FP64-class accuracy for complex128 and
  * exact products for complex64; groups with more than 9 X/Y positions above qubit 2 take one
- * read each, and so does a read's only group if it is a single term (in FP64 for complex128, exact
- * products and sums for complex64). Synchronises. */
+ * read each, and so does a read's only group if it is a single term (in FP64 for complex128; for
+ * complex64 exact products in FP32 pairs and compensated sums, in FP64 where a product leaves the range
+ * that FP32 pairs hold). Synchronises. */
 qs_status qs_expectation(const qs_state* s, const qs_pauli_obs* obs, double out[2]);
 /* Host only (no GPU needed): how qs_expectation reads an n-qubit state for obs. *n_passes = the
  * tiled reads; tile_masks (optional, cap entries) receives each read's tile qubits as a bit mask;

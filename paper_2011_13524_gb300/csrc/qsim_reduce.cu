@@ -129,9 +129,11 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_group(const C* __restric
 //    seven per pair and term).
 //  * complex64: products exact in FP32 pairs, summed with two levels of compensation (TwoSum of the
 //    sums and of their errors: nothing above 2^-70 of a thread's sum is dropped), both components of a
-//    pair side by side in packed instructions; one FP64 conversion per thread.
-// 24 random strings, whole call, one launch per group / here: complex64 1.62 / 0.33 ms at n = 23 (284 us
-// of kernel, L2 reads and packed FP32 arithmetic about equal) and 67.8 / 12.9 ms at n = 28, complex128
+//    pair side by side in packed instructions; one FP64 conversion per thread. A pair with a product
+//    below 2^-100 (its rounding error can fall under FP32's range) or from 2^80 on goes to an FP64 sum
+//    instead, as the group kernel forms it.
+// 24 random strings, whole call, one launch per group / here: complex64 1.62 / 0.35 ms at n = 23 (300 us
+// of kernel, 15 of them for the range; L2 reads and packed FP32 arithmetic about equal) and 67.8 / 12.9 ms at n = 28, complex128
 // 0.75 / 0.36 ms at n = 22 and 50.9 / 25.4 ms at n = 28.
 constexpr int kMaxSingles = 64;
 struct SingleTerm {
@@ -154,12 +156,30 @@ __device__ __forceinline__ float2 two_sum2(float2 a, float2 b, float2& e) {
 }
 struct SingleAccF {  // complex64
     float2 s = make_float2(0.f, 0.f), c = make_float2(0.f, 0.f), d = make_float2(0.f, 0.f);
-    __device__ __forceinline__ void add(float2 a, float2 b, bool imag, int neg) {
+    double wide = 0.0;
+    // at least kRange for a product outside [2^-100, 2^80), zero included (the shift drops the sign)
+    static constexpr uint32_t kRange = 180u << 24;
+    __device__ __forceinline__ static uint32_t range(float p) { return 2u * __float_as_uint(p) - (27u << 24); }
+    // the factors of a pair's two products
+    __device__ __forceinline__ static float2 factor(float2 a, bool imag, int neg) {
         const uint32_t sg = uint32_t(neg) << 31;
-        float2 u = imag ? make_float2(a.y, -a.x) : a;
-        u.x = __uint_as_float(__float_as_uint(u.x) ^ sg);
-        u.y = __uint_as_float(__float_as_uint(u.y) ^ sg);
-        const float2 p = __fmul2_rn(u, b);
+        const float2 u = imag ? make_float2(a.y, -a.x) : a;
+        return make_float2(__uint_as_float(__float_as_uint(u.x) ^ sg), __uint_as_float(__float_as_uint(u.y) ^ sg));
+    }
+    __device__ __forceinline__ static bool in_range(float2 a, float2 b, bool imag, int neg) {
+        const float2 p = __fmul2_rn(factor(a, imag, neg), b);
+        return max(range(p.x), range(p.y)) < kRange;
+    }
+    template <bool kInRange>
+    __device__ __forceinline__ void add(float2 a, float2 b, bool imag, int neg) {
+        const float2 u = factor(a, imag, neg), p = __fmul2_rn(u, b);
+        if constexpr (!kInRange) {  // (a product that a factor makes zero is exact)
+            if ((range(p.x) >= kRange && u.x != 0.f && b.x != 0.f) || (range(p.y) >= kRange && u.y != 0.f && b.y != 0.f)) {
+                wide = fma(double(u.x), double(b.x), wide);
+                wide = fma(double(u.y), double(b.y), wide);
+                return;
+            }
+        }
         float2 e, e2;
         s = two_sum2(s, p, e);
         e = __fadd2_rn(e, __ffma2_rn(u, b, make_float2(-p.x, -p.y)));
@@ -167,11 +187,13 @@ struct SingleAccF {  // complex64
         d = __fadd2_rn(d, e2);
     }
     __device__ double value() const {
-        return (double(s.x) + double(s.y)) + ((double(c.x) + double(c.y)) + (double(d.x) + double(d.y)));
+        return ((double(s.x) + double(s.y)) + ((double(c.x) + double(c.y)) + (double(d.x) + double(d.y)))) + wide;
     }
 };
 struct SingleAccD {  // complex128
     double s = 0.0, c = 0.0;
+    __device__ __forceinline__ static bool in_range(double2, double2, bool, int) { return true; }
+    template <bool>
     __device__ __forceinline__ void add(double2 a, double2 b, bool imag, int neg) {
         const long long sg = static_cast<long long>(uint64_t(neg) << 63);
         const double ux = imag ? a.y : a.x, uy = imag ? -a.x : a.y;
@@ -202,10 +224,20 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_singles(const C* __restr
             b[u] = psi[y ^ T.f];
             neg[u] = parity64(y & T.z);
         }
+        bool fast = i0 + (kU - 1) * stride < P.pairs;  // (one branch for the four: their sums interleave)
+        if (fast) {
 #pragma unroll
-        for (int u = 0; u < kU; u++) {
-            if (i0 + u * stride >= P.pairs) break;
-            acc.add(a[u], b[u], imag, neg[u]);
+            for (int u = 0; u < kU; u++) fast &= Acc::in_range(a[u], b[u], imag, neg[u]);
+        }
+        if (fast) {
+#pragma unroll
+            for (int u = 0; u < kU; u++) acc.template add<true>(a[u], b[u], imag, neg[u]);
+        } else {
+#pragma unroll
+            for (int u = 0; u < kU; u++) {
+                if (i0 + u * stride >= P.pairs) break;
+                acc.template add<false>(a[u], b[u], imag, neg[u]);
+            }
         }
     }
     __shared__ double sh[kRedThreads / 32];

@@ -57,3 +57,42 @@ def test_singles_hold_wide_magnitudes():
         ref = oracle.expectation(vec, obs)[0]
         assert abs(st.expectation(obs)[0] - ref) < 1e-15 * float((np.abs(vec) ** 2).sum())
     st.close()
+
+
+@pytest.mark.parametrize("scale", [2.0 ** -80, 2.0 ** 70])
+@pytest.mark.parametrize("n", [4, 14])
+def test_singles_of_scaled_complex64_states(n, scale):
+    """Amplitudes whose products leave FP32's range: the sums are those of FP64 products, as in a group of
+    its own, to 1e-14 of the summed magnitudes (FP64 on both sides)."""
+    import paper_2011_13524_gb300 as qs
+    full = (1 << n) - 1
+    st = qs.State(n, qs.QS_C64)
+    st.load(W.random_state_fast(n, 11) * scale)
+    vec = st.get_vector().astype(np.complex128)
+    for x, z in [(full, 0), (full, 5), (full, full), (1, 2)]:
+        obs = W.PauliObservable(n, np.array([0.75]), np.array([x], dtype=np.uint64), np.array([z], dtype=np.uint64))
+        size = float((np.abs(vec) * np.abs(vec[np.arange(1 << n) ^ x])).sum())
+        assert abs(st.expectation(obs)[0] - oracle.expectation(vec, obs)[0]) < 1e-14 * size
+    st.close()
+
+
+def test_singles_of_small_pairs_beside_large_ones():
+    """A string that joins amplitudes of 2^-70 only, beside one of 1, in complex64; and an amplitude that is
+    not finite."""
+    import paper_2011_13524_gb300 as qs
+    n = 14
+    full = (1 << n) - 1
+    v = W.random_state_fast(n, 12) * 2.0 ** -70
+    v[1000] = 1.0
+    v[1000 ^ full] = 0.0
+    st = qs.State(n, qs.QS_C64)
+    st.load(v)
+    vec = st.get_vector().astype(np.complex128)
+    obs = W.PauliObservable(n, np.array([1.0]), np.array([full], dtype=np.uint64), np.array([3], dtype=np.uint64))
+    size = float((np.abs(vec) * np.abs(vec[::-1])).sum())
+    assert abs(st.expectation(obs)[0] - oracle.expectation(vec, obs)[0]) < 1e-14 * size
+    for bad in (np.nan, np.inf):
+        v[77] = bad
+        st.load(v)
+        assert not np.isfinite(st.expectation(obs)[0])
+    st.close()
