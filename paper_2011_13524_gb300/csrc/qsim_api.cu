@@ -193,10 +193,12 @@ void apply_single(qs_state* s, const Op& op) {
     launch_op(op, s->data, s->n, s->dt, s->stream, stage_of(s));
 }
 
-// Ops applied gate by gate, several per pass over the state (qsim_pass.cu). A pass whose gates move
-// less than a full pass as launches of their own (one controlled phase, say) is launched gate by
-// gate from the size on where traffic counts more than launches.
-constexpr int kPassTrafficQubits = 18;
+// Ops applied gate by gate, several per pass over the state (qsim_pass.cu), or each as its own launch where
+// the pass's gates cost less so: a pass of one gate always does (a Pauli rotation at n = 26 0.57 ms as a
+// tile, 0.36 as a launch in complex128, 0.25 / 0.19 in complex64), others from kPassCostQubits on by
+// the costs of their kinds. Below, launches count more than traffic. A double-float run's first and last
+// passes also save a conversion pass as tiles, kConversionCost.
+constexpr double kConversionCost = 0.9;
 // `fp64`: in IEEE doubles also where double-float is set.
 void run_ops(qs_state* s, const std::vector<Op>& ops, bool fp64 = false) {
     const bool df_run = use_df(s) && !s->df && !fp64;
@@ -206,14 +208,20 @@ void run_ops(qs_state* s, const std::vector<Op>& ops, bool fp64 = false) {
         DFScope df(s, df_run);
         return;
     }
-    auto single = [&](const GatePass& p) { return !p.local || (p.share < 1.0 && s->n >= kPassTrafficQubits); };
+    auto single = [&](size_t i) {
+        const GatePass& p = passes[i];
+        if (!p.local) return true;
+        const int converts = df_run ? int(i == 0) + int(i + 1 == passes.size()) : 0;
+        if (s->n < kPassCostQubits) return p.ops.size() == 1 && !converts;
+        return p.alone < p.tile - kConversionCost * converts;
+    };
     // a double-float run changes the layout in its first and last passes where those are tile passes
-    const bool in = df_run && !single(passes.front()), out = df_run && !single(passes.back());
+    const bool in = df_run && !single(0), out = df_run && !single(passes.size() - 1);
     DFScope df(s, df_run, in);
     for (size_t i = 0; i < passes.size(); i++) {
         const GatePass& p = passes[i];
         const bool last = i + 1 == passes.size();
-        if (single(p)) {
+        if (single(i)) {
             for (size_t k : p.ops) launch_op_arith(ops[k], s->data, s->n, ar, s->stream, stage_of(s));
         } else {
             launch_gate_pass(p, ops, s->data, s->n, ar, in && i == 0, out && last, s->stream);

@@ -228,8 +228,10 @@ struct GatePass {
     std::vector<size_t> ops;  // indices into the run's ops
     uint64_t local = 0;       // the tile's qubits
     size_t data = 0;          // matrix entries
-    double share = 0.0;       // traffic of the ops as single launches, in full passes
+    double alone = 0.0;       // estimated cost of the ops as launches of their own, and
+    double tile = 0.0;        // as this pass, in light full passes over the state (measured from 20 qubits on)
 };
+constexpr int kPassCostQubits = 20;
 int gate_pass_bits(int n, Arith ar);
 std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith ar);
 // ieee_in / ieee_out (double-float): psi holds / is left in IEEE complex128

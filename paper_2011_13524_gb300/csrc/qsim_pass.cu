@@ -350,11 +350,51 @@ bool is_identity(const Op& op) {
     return (op.kind == OpKind::Phase && op.phase == cplx(1.0, 0.0)) ||
            (op.kind == OpKind::Pauli && op.xmask == 0 && op.zmask == 0);
 }
-// share of a full pass's traffic that the op costs as a launch of its own
-double op_share(const Op& op) {
-    double f = std::ldexp(1.0, -int(op.controls.size()));
-    if (op.kind == OpKind::Swap) f *= 0.5;
-    return f;
+// What an op costs as a launch of its own and inside a tile pass, which adds kPassBase for the staging,
+// in full passes of the lightest kind (an X gate's launch: 356 us at n = 26, 90 at n = 24, 21 at n = 22
+// in complex128, 175 / 48 / 12 us in complex64). From runs of 1, 2, 3, 4 and 8 gates of a kind on low qubits,
+// as launches and as one pass, at n = 20, 22, 24 and 26; the figures lean to the launches where the sizes
+// differ. One launch each / one pass, microseconds for 8 gates at n = 26 (F64 at n = 24): double-float
+// U3 2849 / 2239, RY 2855 / 1386, dense pair 3207 / 3794, RZ 2737 / 2862, rotation 2880 / 1716, CZ 1202 /
+// 1035, X 2749 / 1184; complex64 U3 1336 / 516, dense pair 1501 / 873, RZ 1448 / 1467, CZ 765 / 589; F64
+// U3 2098 / 1882, RZ 1051 / 1201, rotation 1432 / 1541. A tile pass gains nothing per diagonal factor (index
+// and parity work per amplitude and gate) and, in double-float, nothing per dense pair (arithmetic).
+enum OpClass { kOpD1, kOpD1Half, kOpD2, kOpSign, kOpFactor, kOpSwap, kOpFlip, kOpRot, kOpClasses };
+struct ClassCost {
+    double alone, inside;
+};
+constexpr ClassCost kClassCost[3][kOpClasses] = {  // by Arith
+    {{1.0, 0.45}, {1.0, 0.45}, {1.3, 0.75}, {1.1, 0.38}, {1.05, 1.1}, {1.9, 0.35}, {1.05, 0.45}, {1.05, 0.5}},    // F32
+    {{2.9, 2.55}, {1.5, 1.4}, {5.8, 5.0}, {1.0, 0.2}, {1.45, 1.5}, {1.6, 0.25}, {1.0, 0.3}, {2.0, 2.1}},         // F64
+    {{1.0, 0.72}, {1.0, 0.45}, {1.15, 1.25}, {1.2, 0.28}, {1.0, 1.0}, {1.4, 0.25}, {0.95, 0.38}, {1.05, 0.55}},  // DF
+};
+static_assert(int(Arith::F32) == 0 && int(Arith::F64) == 1 && int(Arith::DF) == 2, "order of kClassCost");
+constexpr double kPassBase[3] = {0.95, 1.1, 1.1};
+OpClass op_class(const Op& op) {
+    switch (op.kind) {
+        case OpKind::Dense: {
+            if (op.targets.size() > 1) return kOpD2;
+            const auto& d = op.data;
+            const bool re = d[0].imag() == 0.0 && d[3].imag() == 0.0;
+            const bool half = re && ((d[1].imag() == 0.0 && d[2].imag() == 0.0) || (d[1].real() == 0.0 && d[2].real() == 0.0));
+            return half ? kOpD1Half : kOpD1;
+        }
+        case OpKind::Swap: return kOpSwap;
+        case OpKind::Diag: return kOpFactor;
+        case OpKind::Phase: return op.phase.real() == 0.0 || op.phase.imag() == 0.0 ? kOpSign : kOpFactor;
+        case OpKind::Pauli: return op.xmask ? kOpFlip : kOpSign;
+        default: return op.xmask ? kOpRot : kOpFactor;
+    }
+}
+ClassCost op_pass_cost(const Op& op, Arith ar) {
+    ClassCost c = kClassCost[int(ar)][op_class(op)];
+    // a launch touches the share of the state that its controls select; on the lowest qubits it still
+    // moves most of the lines
+    for (int q : op.controls) c.alone *= ar == Arith::F32 ? (q < 4 ? 0.9 : 0.55) : (q < 3 ? 0.8 : 0.5);
+    if (op.kind == OpKind::Swap) c.alone *= 0.5;
+    // a launch reads a long string's amplitudes further apart (X or Y on 13 qubits: 1.2 to 1.6)
+    if (op.kind == OpKind::PauliRot && op.xmask) c.alone += 0.03 * (__builtin_popcountll(op.xmask) - 2);
+    return c;
 }
 constexpr int kPassOps = 128, kPassData = 640;      // a pass's limits (16.5 KB of parameters)
 constexpr int kPassOpsS = 24, kPassDataS = 96;      // the small form's (3.2 KB)
@@ -544,7 +584,7 @@ std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith a
         }
         uint64_t L = low, bx = 0, bd = 0;
         size_t data = 0;
-        double share = 0.0;
+        p.tile = kPassBase[int(ar)];
         keep.clear();
         bool ended = false;
         for (size_t i : rem) {
@@ -554,7 +594,9 @@ std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith a
                 data + e <= size_t(kPassData) && __builtin_popcountll(L | q[i].x) <= t && fits_alone(op, q[i])) {
                 L |= q[i].x;
                 data += e;
-                share += op_share(op);
+                const ClassCost cost = op_pass_cost(op, ar);
+                p.alone += cost.alone;
+                p.tile += cost.inside;
                 p.ops.push_back(i);
             } else {
                 bx |= q[i].x;
@@ -566,7 +608,6 @@ std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith a
         for (int b = 0; b < n && __builtin_popcountll(L) < t; b++) L |= 1ull << b;
         p.local = L;
         p.data = data;
-        p.share = share;
         out.push_back(std::move(p));
         rem.swap(keep);
     }

@@ -92,3 +92,44 @@ def test_long_runs_and_many_slices():
     st.apply_observable_rotation(obs, 0.9, 150)  # 1350 rotations
     assert float(np.max(np.abs(st.get_vector() - oracle.observable_rotation(psi, 9, obs, 0.9, 150)))) < 2e-12
     st.close()
+
+
+@pytest.mark.parametrize("arith", ["df", "f64", "c64"])
+@pytest.mark.parametrize("n", [19, 20])
+def test_launches_between_passes(n, arith):
+    """Runs of one kind, of one gate to more than a tile pays for, on either side of the size from which a
+    pass may be launched gate by gate: as tiles, as launches, and both in one run."""
+    import torch
+    import paper_2011_13524_gb300 as qs
+    dt, tdt = (qs.QS_C64, torch.complex64) if arith == "c64" else (qs.QS_C128, torch.complex128)
+    rng = W.SplitMix64(n)
+    qubits = [(0, n - 1), (n // 2, 1), (n - 1, 3), (2, n - 2)]
+    apart = W.Gate("DENSE", (0, n // 2, n - 1), matrix=W.random_unitary(8, rng))  # in no tile
+    kinds = {
+        "u3": lambda a, b: W.Gate("U3", (a,), params=(0.3 + a, 0.2, 0.7)),
+        "ry": lambda a, b: W.Gate("RY", (a,), (b,), (1,), params=(0.3 + a,)),
+        "dense": lambda a, b: W.Gate("DENSE", (a, b), matrix=W.random_unitary(4, rng)),
+        "cz": lambda a, b: W.Gate("CZ", (a, b)),
+        "rz": lambda a, b: W.Gate("RZ", (a,), params=(0.7,)),
+        "diag": lambda a, b: W.Gate("DIAG", (a, b), matrix=np.exp(1j * np.arange(4))),
+        "swap": lambda a, b: W.Gate("SWAP", (a, b)),
+        "y": lambda a, b: W.Gate("Y", (a,)),
+        "rot": lambda a, b: W.Gate("PAULIROT", (a, b), pauli=(1, 2), params=(0.4,)),
+    }
+    gates = []
+    for make in kinds.values():
+        for count in (1, 2, 12):
+            gates += [make(*qubits[i % 4]) for i in range(count)] + [apart]
+    c = W.Circuit(n, gates)
+    v = random_tensor(n, tdt, n)
+    a, b = qs.State(n, dt, tensor=v.clone()), qs.State(n, dt, tensor=v)
+    a.set_arith(math=qs.QS_MATH_FP64 if arith == "f64" else qs.QS_MATH_DF)
+    b.set_arith(math=qs.QS_MATH_FP64)
+    a.run(c, 0)
+    for g in gates:
+        b.apply_gate(g)
+    a.synchronize()
+    b.synchronize()
+    assert float((a.tensor - b.tensor).abs().max()) < TOL[arith]
+    a.close()
+    b.close()
