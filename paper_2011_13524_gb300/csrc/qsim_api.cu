@@ -486,11 +486,11 @@ void trotter_by_terms(qs_state* s, const qs_pauli_obs* H, double angle, int n_sl
     std::vector<Op> ops;
     for (int k = 0; k < H->n_terms; k++) ops.push_back(trotter_op(H, k, angle, n_slices));
     // slices in batches of a bounded number of ops
-    const int per = int(std::max<size_t>(1, 1024 / std::max<size_t>(1, ops.size())));
+    const int64_t per = std::max<int64_t>(1, 1024 / int64_t(ops.size()));
     DFScope df(s, use_df(s) && n_slices > per);
-    for (int r = 0; r < n_slices; r += per) {
+    for (int64_t r = 0; r < n_slices; r += per) {
         std::vector<Op> some;
-        for (int j = r; j < std::min(n_slices, r + per); j++) some.insert(some.end(), ops.begin(), ops.end());
+        for (int64_t j = r; j < std::min<int64_t>(n_slices, r + per); j++) some.insert(some.end(), ops.begin(), ops.end());
         run_ops(s, some);
     }
 }
@@ -579,7 +579,7 @@ void trotter_by_blocks(qs_state* s, const qs_pauli_obs* H, double angle, int n_s
         const FusionPlan plan = plan_of(pieces[0].gates, per);
         const int rest = n_slices % per;
         DFScope df(s, use_df(s) && n_slices > per);  // one plan folds the layout changes into its passes
-        for (int r = 0; r + per <= n_slices; r += per) apply(plan, pieces[0].gates, per);
+        for (int64_t r = 0; r + per <= n_slices; r += per) apply(plan, pieces[0].gates, per);
         if (rest) apply(plan_of(pieces[0].gates, rest), pieces[0].gates, rest);
         return;
     }
@@ -1331,10 +1331,13 @@ qs_status qs_apply_observable_rotation(qs_state* s, const qs_pauli_obs* H, doubl
     const uint64_t all = s->n >= 64 ? ~0ull : ((1ull << s->n) - 1);
     for (int k = 0; k < H->n_terms; k++)
         QS_REQUIRE(((H->x_mask[k] | H->z_mask[k]) & ~all) == 0, "Pauli mask names a qubit outside the state");
-    if (trotter_fused(s, H, angle))
+    if (H->n_terms == 0) {  // (a double-float call rounds the state to that format whatever its terms)
+        DFScope df(s, use_df(s));
+    } else if (trotter_fused(s, H, angle)) {
         trotter_by_blocks(s, H, angle, n_slices);
-    else
+    } else {
         trotter_by_terms(s, H, angle, n_slices);
+    }
     API_END
 }
 

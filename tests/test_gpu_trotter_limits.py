@@ -58,3 +58,18 @@ def test_no_memory_for_blocks(slices):
     assert float((a.tensor - b.tensor).abs().max()) < TOL
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("n", [5, N])
+def test_no_terms_many_slices(n):
+    """Without terms a call has nothing to loop over, whatever its slices."""
+    import numpy as np
+    import torch
+    import paper_2011_13524_gb300 as qs
+    st = qs.State(n, qs.QS_C128)
+    ref = st.tensor.clone()
+    none = W.PauliObservable(n, np.array([]), np.array([], dtype=np.uint64), np.array([], dtype=np.uint64))
+    st.apply_observable_rotation(none, 0.4, 2 ** 31 - 1)
+    st.synchronize()
+    assert torch.equal(st.tensor, ref)
+    st.close()
