@@ -482,9 +482,7 @@ Op trotter_op(const qs_pauli_obs* H, int k, double angle, int n_slices) {
 }
 
 // term by term, several per pass over the state
-void trotter_by_terms(qs_state* s, const qs_pauli_obs* H, double angle, int n_slices) {
-    std::vector<Op> ops;
-    for (int k = 0; k < H->n_terms; k++) ops.push_back(trotter_op(H, k, angle, n_slices));
+void trotter_by_terms(qs_state* s, const std::vector<Op>& ops, int n_slices) {
     // slices in batches of a bounded number of ops
     const int64_t per = std::max<int64_t>(1, 1024 / int64_t(ops.size()));
     DFScope df(s, use_df(s) && n_slices > per);
@@ -496,17 +494,18 @@ void trotter_by_terms(qs_state* s, const qs_pauli_obs* H, double angle, int n_sl
 }
 
 // Where a pass over the state costs more than preparing a block on the host, the terms of up to 6
-// qubits are fused like the gates of a circuit (5-qubit blocks, on the tensor cores): a slice of a
-// 26-qubit Ising chain has 51 terms, and two slices are 9 blocks instead of 102 passes. Terms longer
-// than 6 qubits keep a pass of their own between the blocks of the terms before and after them.
-// Two slices at n = 26 (complex128): 35.5 ms by terms, 4.4 ms in blocks. From states that no longer
+// qubits are fused like the gates of a circuit (5-qubit blocks, on the tensor cores) if that costs less than
+// their passes: a slice of a 26-qubit Ising chain has 51 terms, and two slices are 9 blocks instead of
+// 102 launches. Terms longer than 6 qubits, and runs of terms that share too few qubits for blocks, go by
+// terms, in the order of the slice.
+// Two slices of the chain at n = 26 (complex128): 35.5 ms by launches, 4.4 ms in blocks. From states that no longer
 // fit the 129 MB L2 on; the Ising chain, one slice, by terms / in blocks (planned afresh): 0.92 / 1.04
 // ms at n = 22, 2.15 / 1.35 at n = 23, 4.26 / 1.71 at n = 24 in complex128, 0.99 / 0.95 at n = 23 and
 // 2.35 / 1.19 at n = 24 in complex64 (about 0.7 ms of it host planning and block matrices). The blocks'
 // matrices are copied to the device and waited for, which a stream capture does not allow: there the
 // terms keep their passes, which are launches alone.
 constexpr double kTrotterFuseBytes = 128.0 * (1 << 20);
-constexpr int kTrotterPlanGates = 256;  // gates per plan (slices repeat it): bounds the planning time
+constexpr int kTrotterPlanGates = 256;  // gates per plan, of one slice or several: bounds the planning time
 bool trotter_fused(const qs_state* s, const qs_pauli_obs* H, double angle) {
     if (std::ldexp(double(amp_bytes(s->dt)), s->n) < kTrotterFuseBytes) return false;
     cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
@@ -520,21 +519,95 @@ bool trotter_fused(const qs_state* s, const qs_pauli_obs* H, double angle) {
     return s->dt == QS_C64 ? tensor_c64x_enabled() : use_df(s) && tensor_c128_enabled();
 }
 
+// A plan's blocks in the unit of scheduled_cost: launches by width (n = 24 and 26), and the host's time for
+// a wide block's matrix and its upload, 30 us (60 for 6 targets) against the 3 TB/s of state that such a
+// launch reads. The partition alone decides, no matrix is made for it. One slice, by terms / in blocks
+// wherever they fit / now: 100 random pairs on 26 qubits (complex128) 22.7 / 11.6 / 11.6 ms, 100 strings of
+// four 25.9 / 38.5 / 26.0, all hoppings of range 8 (Jordan-Wigner strings, 176 terms) 34.3 / 165.8 / 34.3, where
+// 6-target blocks run on the CUDA cores.
+double blocks_cost(const qs_state* s, const std::vector<BlockShape>& blocks, const std::vector<Op>& terms, Arith ar) {
+    static constexpr double wide[2][7] = {{0, 1.0, 1.15, 2.5, 1.4, 1.5, 19.0}, {0, 0.95, 1.0, 1.0, 1.8, 1.25, 1.7}};
+    const double unit_us = std::ldexp(double(amp_bytes(s->dt)), s->n) / 3e6;
+    double t = 0.0;
+    for (const BlockShape& b : blocks) {
+        if (b.gates.size() == 1)
+            t += scheduled_cost({terms[size_t(b.gates[0]) % terms.size()]}, s->n, ar);
+        else
+            t += wide[ar == Arith::F32 ? 1 : 0][b.width] + (b.width < 4 ? 0.0 : b.width < 6 ? 30.0 : 60.0) / unit_us;
+    }
+    return t;
+}
+
+// one slice as parts in order: fused runs of terms, and terms by passes
+struct TrotterPart {
+    std::vector<Op> ops;
+    FusionPlan plan;
+    bool fused = false;
+};
+
 void trotter_by_blocks(qs_state* s, const qs_pauli_obs* H, double angle, int n_slices) {
-    // a slice as pieces: runs of terms that fit a gate, and single long terms
-    struct Piece {
-        std::vector<qs_gate> gates;
-        int long_term = -1;
+    const Arith ar = use_df(s) ? Arith::DF : arith_of(s);
+    std::vector<qs_gate> repeated;
+    auto circuit_of = [&](const std::vector<qs_gate>& gates, int repeat) {
+        repeated.clear();
+        for (int r = 0; r < repeat; r++) repeated.insert(repeated.end(), gates.begin(), gates.end());
+        qs_circuit c;
+        std::memset(&c, 0, sizeof(c));
+        c.n = s->n;
+        c.n_gates = int(repeated.size());
+        c.gates = repeated.data();
+        return c;
     };
-    std::vector<Piece> pieces;
+    auto plan_of = [&](const std::vector<qs_gate>& gates, int repeat) {
+        const qs_circuit c = circuit_of(gates, repeat);
+        return plan_fusion(&c, 5);
+    };
+    // without memory for a plan's block matrices its terms keep their passes, which need none
+    auto apply = [&](const FusionPlan& plan, const std::vector<Op>& ops, int repeat) {
+        bool started = false;
+        try {
+            apply_plan_impl(s, plan, nullptr, &started);
+        } catch (const Error& e) {
+            if (e.code != QS_ERR_OOM || started) throw;
+            std::vector<Op> all;
+            for (int r = 0; r < repeat; r++) all.insert(all.end(), ops.begin(), ops.end());
+            run_ops(s, all);
+        }
+    };
+    std::vector<TrotterPart> parts;
+    std::vector<qs_gate> run;  // terms that fit a gate, not yet in a part
+    std::vector<Op> run_terms;
+    auto flush = [&](bool whole) {
+        if (run.empty()) return;
+        TrotterPart p;
+        // a slice that is one run repeats in its plan
+        const int repeat = whole ? std::max(1, std::min(n_slices, kTrotterPlanGates / int(run.size()))) : 1;
+        if (run.size() > 1) {
+            const qs_circuit c = circuit_of(run, repeat);
+            p.fused = blocks_cost(s, plan_shapes(&c, 5), run_terms, ar) < repeat * scheduled_cost(run_terms, s->n, ar);
+        }
+        if (p.fused) p.plan = plan_of(run, repeat);
+        if (p.fused && whole) {
+            const int rest = n_slices % repeat;
+            DFScope df(s, use_df(s) && n_slices > repeat);  // one plan folds the layout changes into its passes
+            for (int64_t r = 0; r + repeat <= n_slices; r += repeat) apply(p.plan, run_terms, repeat);
+            if (rest) apply(plan_of(run, rest), run_terms, rest);
+            return;
+        }
+        if (p.fused || parts.empty() || parts.back().fused) parts.push_back(std::move(p));
+        parts.back().ops.insert(parts.back().ops.end(), run_terms.begin(), run_terms.end());
+        run.clear();
+        run_terms.clear();
+    };
     for (int k = 0; k < H->n_terms; k++) {
         const uint64_t sup = H->x_mask[k] | H->z_mask[k];
         if (__builtin_popcountll(sup) > QS_MAX_TARGETS) {
-            pieces.emplace_back();
-            pieces.back().long_term = k;
+            flush(false);
+            if (parts.empty() || parts.back().fused) parts.emplace_back();
+            parts.back().ops.push_back(trotter_op(H, k, angle, n_slices));
             continue;
         }
-        if (pieces.empty() || pieces.back().long_term >= 0) pieces.emplace_back();
+        if (run.size() == size_t(kTrotterPlanGates)) flush(false);
         qs_gate g;
         std::memset(&g, 0, sizeof(g));
         g.kind = QS_GATE_NAMED;
@@ -548,52 +621,18 @@ void trotter_by_blocks(qs_state* s, const qs_pauli_obs* H, double angle, int n_s
             g.pauli[g.m++] = x ? 1 + z : 3;
         }
         if (g.m == 0) g.m = 1;  // identity term: a phase, written as exp(i a I / 2) on qubit 0
-        pieces.back().gates.push_back(g);
+        run.push_back(g);
+        run_terms.push_back(trotter_op(H, k, angle, n_slices));
     }
-    if (pieces.empty()) return;
-    auto plan_of = [&](const std::vector<qs_gate>& gates, int repeat) {
-        std::vector<qs_gate> all;
-        for (int r = 0; r < repeat; r++) all.insert(all.end(), gates.begin(), gates.end());
-        qs_circuit c;
-        std::memset(&c, 0, sizeof(c));
-        c.n = s->n;
-        c.n_gates = int(all.size());
-        c.gates = all.data();
-        return plan_fusion(&c, 5);
-    };
-    // without memory for a plan's block matrices its terms keep their passes, which need none
-    auto apply = [&](const FusionPlan& plan, const std::vector<qs_gate>& gates, int repeat) {
-        bool started = false;
-        try {
-            apply_plan_impl(s, plan, nullptr, &started);
-        } catch (const Error& e) {
-            if (e.code != QS_ERR_OOM || started) throw;
-            std::vector<Op> ops;
-            for (int r = 0; r < repeat; r++)
-                for (const qs_gate& g : gates) ops.push_back(op_of_gate(g, s->n, nullptr));
-            run_ops(s, ops);
-        }
-    };
-    if (pieces.size() == 1 && pieces[0].long_term < 0) {  // whole slices, several per plan
-        const int per = std::max(1, std::min(n_slices, kTrotterPlanGates / int(pieces[0].gates.size())));
-        const FusionPlan plan = plan_of(pieces[0].gates, per);
-        const int rest = n_slices % per;
-        DFScope df(s, use_df(s) && n_slices > per);  // one plan folds the layout changes into its passes
-        for (int64_t r = 0; r + per <= n_slices; r += per) apply(plan, pieces[0].gates, per);
-        if (rest) apply(plan_of(pieces[0].gates, rest), pieces[0].gates, rest);
-        return;
-    }
-    std::vector<FusionPlan> plans(pieces.size());
-    for (size_t i = 0; i < pieces.size(); i++)
-        if (pieces[i].long_term < 0) plans[i] = plan_of(pieces[i].gates, 1);
+    const bool whole = parts.empty();
+    flush(whole);
+    if (parts.empty()) return;  // done as one run
+    if (parts.size() == 1 && !parts[0].fused) return trotter_by_terms(s, parts[0].ops, n_slices);
     DFScope df(s, use_df(s));
     for (int r = 0; r < n_slices; r++)
-        for (size_t i = 0; i < pieces.size(); i++) {
-            if (pieces[i].long_term < 0)
-                apply(plans[i], pieces[i].gates, 1);
-            else
-                launch_op_arith(trotter_op(H, pieces[i].long_term, angle, n_slices), s->data, s->n, arith_of(s),
-                                s->stream, stage_of(s));
+        for (const TrotterPart& p : parts) {
+            if (p.fused) apply(p.plan, p.ops, 1);
+            else run_ops(s, p.ops);
         }
 }
 
@@ -1336,7 +1375,9 @@ qs_status qs_apply_observable_rotation(qs_state* s, const qs_pauli_obs* H, doubl
     } else if (trotter_fused(s, H, angle)) {
         trotter_by_blocks(s, H, angle, n_slices);
     } else {
-        trotter_by_terms(s, H, angle, n_slices);
+        std::vector<Op> ops;
+        for (int k = 0; k < H->n_terms; k++) ops.push_back(trotter_op(H, k, angle, n_slices));
+        trotter_by_terms(s, ops, n_slices);
     }
     API_END
 }

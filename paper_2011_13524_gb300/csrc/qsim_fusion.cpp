@@ -534,7 +534,8 @@ void clear_partition_cache() {
     g_part_cache.clear();
 }
 
-FusionPlan plan_fusion(const qs_circuit* c, int k, const double* theta) {
+namespace {
+std::vector<OpenBlock> partition_of(const qs_circuit* c, int k) {
     QS_REQUIRE(c != nullptr, "null circuit");
     QS_REQUIRE(c->n >= 1 && c->n <= QS_MAX_QUBITS, "qubit count out of range");
     QS_REQUIRE(c->n_gates >= 0 && (c->n_gates == 0 || c->gates != nullptr), "null gate array");
@@ -548,12 +549,23 @@ FusionPlan plan_fusion(const qs_circuit* c, int k, const double* theta) {
         masks[i] = gate_mask(g);
         tags[i] = gate_tags(g, c->n);
     }
+    return partition(c, masks, tags, k);
+}
+}  // namespace
+
+std::vector<BlockShape> plan_shapes(const qs_circuit* c, int k) {
+    std::vector<BlockShape> out;
+    for (const OpenBlock& b : partition_of(c, k)) out.push_back(BlockShape{b.gates, __builtin_popcountll(b.mask)});
+    return out;
+}
+
+FusionPlan plan_fusion(const qs_circuit* c, int k, const double* theta) {
+    const std::vector<OpenBlock> parts = partition_of(c, k);
     FusionPlan plan;
     plan.n = c->n;
     plan.k = k;
     plan.n_source_gates = c->n_gates;
     // block matrices: independent of each other, built by several host threads for long plans
-    const std::vector<OpenBlock> parts = partition(c, masks, tags, k);
     plan.blocks.resize(parts.size());
     size_t work = 0;
     for (const OpenBlock& blk : parts) work += blk.gates.size() << (2 * __builtin_popcountll(blk.mask));

@@ -234,6 +234,7 @@ struct GatePass {
 constexpr int kPassCostQubits = 20;
 int gate_pass_bits(int n, Arith ar);
 std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith ar);
+double scheduled_cost(const std::vector<Op>& ops, int n, Arith ar);  // of all passes, in light full passes
 // ieee_in / ieee_out (double-float): psi holds / is left in IEEE complex128
 void launch_gate_pass(const GatePass& p, const std::vector<Op>& ops, void* psi, int n, Arith ar, bool ieee_in,
                       bool ieee_out, cudaStream_t st);
@@ -475,6 +476,12 @@ struct FusionPlan {
 // theta (optional): parameter vector overriding the angles of parametric gates
 // forgets the cached partitions (planning starts afresh for every circuit)
 void clear_partition_cache();
+// the blocks that plan_fusion makes, without their matrices
+struct BlockShape {
+    std::vector<int> gates;
+    int width;
+};
+std::vector<BlockShape> plan_shapes(const qs_circuit* c, int k);
 FusionPlan plan_fusion(const qs_circuit* c, int k, const double* theta = nullptr);
 void apply_plan(qs_state* s, const FusionPlan& p);
 

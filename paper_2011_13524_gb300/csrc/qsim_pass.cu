@@ -578,6 +578,7 @@ std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith a
         GatePass p;
         if (!fits_alone(ops[rem[0]], q[rem[0]])) {
             p.ops.push_back(rem[0]);
+            p.alone = op_pass_cost(ops[rem[0]], ar).alone;
             out.push_back(std::move(p));
             rem.erase(rem.begin());
             continue;
@@ -612,6 +613,12 @@ std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith a
         rem.swap(keep);
     }
     return out;
+}
+
+double scheduled_cost(const std::vector<Op>& ops, int n, Arith ar) {
+    double t = 0.0;
+    for (const GatePass& p : schedule_passes(ops, n, ar)) t += p.local ? std::min(p.alone, p.tile) : p.alone;
+    return t;
 }
 
 void launch_gate_pass(const GatePass& p, const std::vector<Op>& ops, void* psi, int n, Arith ar, bool ieee_in,
