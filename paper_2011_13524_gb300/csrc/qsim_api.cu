@@ -1392,7 +1392,13 @@ qs_status qs_apply_observable_rotation(qs_state* s, const qs_pauli_obs* H, doubl
 // gradient's error against 64 bits falls (n = 14, 8 layers, rms: 1.5e-14 to 0.9e-14); passes in
 // double-float took 866 us at n = 16 but raised it to 2.1e-14. complex64 keeps its blocks: in it the
 // order of the roundings shows.
+// A fixed gate of three or more targets is a launch of its own there, from four on with an upload that
+// is waited for, where a plan uploads all of them at once: with 8 / 20 / 60 of them in four layers, fused
+// against passes, n = 16: 3 targets 1.55 / 1.98 / 3.65 ms against 1.40 / 2.01 / 4.22, 4 targets 1.82 / 2.92 / 5.37
+// against 1.76 / 2.97 / 7.14, 6 targets 4.0 / 7.4 / 15.9 against 3.3 / 6.7 / 18.2. From 16 on the blocks
+// serve.
 constexpr int kForwardPassQubits = 16;
+constexpr int kForwardWideGates = 16;
 
 qs_status qs_adjoint_grad(const qs_circuit* c, const double* theta, const qs_pauli_obs* H, qs_dtype dt, void* stream,
                           double* energy, double* grad) {
@@ -1662,10 +1668,16 @@ qs_status qs_adjoint_grad(const qs_circuit* c, const double* theta, const qs_pau
                    : ar == Arith::F32 && tensor_c64x_enabled() ? 6
                    : ar == Arith::F32                           ? 4
                                                                 : 2;
+    std::vector<Op> ops;
+    int wide = 0;
     if (ar != Arith::F32 && c->n <= kForwardPassQubits) {
-        std::vector<Op> ops;
         ops.reserve(size_t(c->n_gates));
-        for (int i = 0; i < c->n_gates; i++) ops.push_back(op_of_gate(c->gates[i], c->n, theta));
+        for (int i = 0; i < c->n_gates; i++) {
+            ops.push_back(op_of_gate(c->gates[i], c->n, theta));
+            wide += ops.back().kind == OpKind::Dense && ops.back().targets.size() > 2;
+        }
+    }
+    if (!ops.empty() && wide < kForwardWideGates) {
         psi->df = 0;
         launch_set_basis_arith(psi->data, c->n, Arith::F64, 0, st);
         run_ops(psi, ops, true);

@@ -28,3 +28,25 @@ def test_forward_of_gradient(n, math):
     assert abs(e - oracle.energy(c, obs)) < TOL * n
     idx = [0, 1, n, 2 * n - 1, 2 * n, 3 * n, 4 * n - 1]
     assert float(np.max(np.abs(g[idx] - oracle.grad_parameter_shift(c, obs, idx)))) < TOL * n
+
+
+@pytest.mark.parametrize("count", [0, 15, 16, 40])
+def test_forward_with_wide_gates(count):
+    """Fixed gates of 3..6 targets, fewer and more than gate passes serve, and no gate at all."""
+    import paper_2011_13524_gb300 as qs
+    n = 9
+    rng = W.SplitMix64(count)
+    h = W.hea_circuit(n, 2, 3)
+    gates = list(h.gates) if count else []
+    for j in range(count):
+        m = 3 + j % 4
+        gates.insert((j * 7) % len(gates), W.Gate("DENSE", tuple((3 * j + 2 * i) % n for i in range(m)), matrix=W.random_unitary(1 << m, rng)))
+    c = W.Circuit(n, gates, n_params=h.n_params)
+    obs = W.random_pauli_observable(n, 6, 3)
+    e, g = qs.adjoint_grad(c, obs)
+    assert abs(e - oracle.energy(c, obs)) < TOL * n
+    if not count:
+        assert not np.any(g)
+        return
+    idx = [0, 1, n, 2 * n - 1, 2 * n, 3 * n, 4 * n - 1]
+    assert float(np.max(np.abs(g[idx] - oracle.grad_parameter_shift(c, obs, idx)))) < TOL * n
