@@ -191,16 +191,15 @@ struct TileRot<DFArith> {
 // for eight rotations). Four CTAs per SM (64 registers, 150 bytes spilled) and three (85) differ by less
 // than the runs.
 constexpr int kAdjTileBits = 10;
-constexpr int kAdjMaxRot = 10;
 template <typename P>
 struct AdjTileParams {
     uint64_t n_tiles;
     uint64_t dep_hi[1 << (kAdjTileBits - 8)];  // address bits of local bits 8..t-1
     int32_t t, nr;
     uint8_t lq[kAdjTileBits];                  // local bit -> qubit, ascending
-    uint8_t bit[kAdjMaxRot];                   // local bit of rotation r
-    uint8_t axis[kAdjMaxRot];
-    typename P::K U[kAdjMaxRot][4];            // R_r^+
+    uint8_t bit[kAdjMaxRotations];                   // local bit of rotation r
+    uint8_t axis[kAdjMaxRotations];
+    typename P::K U[kAdjMaxRotations][4];            // R_r^+
 };
 
 __device__ __forceinline__ uint32_t adj_insert(uint32_t j, int p) {
@@ -566,7 +565,7 @@ void launch_tile(void* psi, void* lam, int n, int nr, const int* qubit, const in
     const size_t smem = 2 * (sizeof(typename P::C) << t) + sizeof(typename GradSlot<P>::T) * kAdjThreads * size_t(nr);
     static PerDevice setup;
     setup.once([](int) {
-        constexpr size_t most = 2 * (sizeof(typename P::C) << kAdjTileBits) + 8 * kAdjThreads * kAdjMaxRot;
+        constexpr size_t most = 2 * (sizeof(typename P::C) << kAdjTileBits) + 8 * kAdjThreads * kAdjMaxRotations;
         QS_TRY_CUDA(cudaFuncSetAttribute(k_adj_tile<P>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(most)));
     });
     k_adj_tile<P><<<grid, kAdjThreads, smem, st>>>(reinterpret_cast<typename P::C*>(psi),
@@ -584,13 +583,14 @@ unsigned adj_grid(int n) {
 }
 
 bool adjoint_rotations_fit(uint64_t qubits, int n) {
-    return __builtin_popcountll(qubits) <= kAdjMaxRot &&
+    return __builtin_popcountll(qubits) <= kAdjMaxRotations &&
            __builtin_popcountll(qubits | adj_low(n)) <= std::min(n, kAdjTileBits);
 }
 
 void launch_adjoint_rotations(void* psi, void* lam, int n, Arith ar, int nr, const int* qubit, const int* axis,
                               const double* theta, double* part, unsigned grid, cudaStream_t st) {
-    QS_REQUIRE(nr >= 1 && nr <= kAdjMaxRot, "rotations per pass out of range");
+    QS_REQUIRE(nr >= 1 && nr <= kAdjMaxRotations, "rotations per pass out of range");
+    for (int r = 0; r < nr; r++) QS_REQUIRE(axis[r] == 1 || axis[r] == 2, "rotations that share a pass are about X or Y");
     switch (ar) {
         case Arith::F32: launch_tile<NativeArith<float>>(psi, lam, n, nr, qubit, axis, theta, part, grid, st); break;
         case Arith::F64: launch_tile<NativeArith<double>>(psi, lam, n, nr, qubit, axis, theta, part, grid, st); break;

@@ -379,7 +379,7 @@ void launch_expect_pass(const TileParams& P, const void* psi, Arith ar, double* 
 void launch_apply_observable(const std::vector<PauliGroup>& groups, const void* psi, void* lam, int n,
                              Arith ar, cudaStream_t st);
 
-// Fused adjoint steps for uncontrolled rotations exp(i theta P/2), P = X/Y/Z (axis 1/2/3): per-block
+// Fused adjoint steps for uncontrolled rotations exp(i theta P/2), P = X/Y (axis 1/2; Z is diagonal): per-block
 // partials of Im <lam|P|psi>, then psi, lam <- R^+ psi, R^+ lam.
 unsigned adj_grid(int n);
 // Consecutive rotation steps on distinct qubits (qubit[0] first, the latest in the circuit) in one pass:
