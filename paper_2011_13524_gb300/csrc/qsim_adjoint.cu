@@ -1,6 +1,6 @@
 // Fused reverse steps of the adjoint gradient: for single-qubit rotations (below) and for runs of
 // diagonal gates (second half of the file). A rotation is
-// R_P(theta) = exp(+i theta P / 2), P in {X, Y, Z} (the paper's gate table sign).
+// R_P(theta) = exp(+i theta P / 2), P in {X, Y} (the paper's gate table sign).
 //
 // At gate j of the reverse sweep psi holds psi_j (the state after the gate) and lambda holds
 // lambda_j = U_{j+1}^+ ... U_G^+ H psi_G. Then dE/dtheta_j = -Im <lambda_j|P|psi_j>; afterwards
@@ -18,16 +18,14 @@ namespace {
 
 constexpr int kAdjThreads = 256;
 
-// accumulators of conj(l) * p for each arithmetic policy, FP64-class in all three
+// accumulators of Im conj(l) * p for each arithmetic policy, FP64-class in all three
 template <typename P>
 struct GradAcc;
 
 template <>
 struct GradAcc<NativeArith<double>> {
-    double re = 0.0, im = 0.0;
+    double im = 0.0;
     __device__ void add(double2 l, double2 p) {
-        re = fma(l.x, p.x, re);
-        re = fma(l.y, p.y, re);
         im = fma(l.x, p.y, im);
         im = fma(-l.y, p.x, im);
     }
@@ -57,12 +55,9 @@ __device__ __forceinline__ void rot_step(typename P::C& a, typename P::C& b, typ
     if (axis == 1) {
         g.add(la, b);
         g.add(lb, a);
-    } else if (axis == 2) {
+    } else {
         g.add(la, P::ipow(b, 3));
         g.add(lb, P::ipow(a, 1));
-    } else {
-        g.add(la, a);
-        g.add(lb, P::ipow(b, 2));
     }
     typename P::Acc r0 = P::first(U[0], a), r1 = P::first(U[2], a), s0 = P::first(U[0], la), s1 = P::first(U[2], la);
     P::mac(r0, U[1], b);
@@ -135,9 +130,9 @@ struct TileRot<DFArith> {
     __device__ __forceinline__ static Pair2 conj_swap(const Pair2& v) {  // (im, -re)
         return Pair2{make_float2(v.h.y, -v.h.x), make_float2(v.l.y, -v.l.x)};
     }
-    // (df_dot2 gives {re_hi, re_lo, im_hi, im_lo})
+    // (pair_dot gives {re_hi, re_lo, im_hi, im_lo})
     __device__ __forceinline__ static C dot(float2 xh, float2 xl, const Pair2& a, float2 yh, float2 yl, const Pair2& b) {
-        return order(df_dot2(xh, xl, a, yh, yl, b));
+        return order(pair_dot(xh, xl, a, yh, yl, b));
     }
     __device__ __forceinline__ static void update(C& a, C& b, int axis, float ch, float cl, float sh, float sl) {
         const Pair2 va = pair(a), vb = pair(b);
@@ -197,15 +192,10 @@ struct AdjTileParams {
     uint64_t dep_hi[1 << (kAdjTileBits - 8)];  // address bits of local bits 8..t-1
     int32_t t, nr;
     uint8_t lq[kAdjTileBits];                  // local bit -> qubit, ascending
-    uint8_t bit[kAdjMaxRotations];                   // local bit of rotation r
+    uint8_t bit[kAdjMaxRotations];             // local bit of rotation r
     uint8_t axis[kAdjMaxRotations];
-    typename P::K U[kAdjMaxRotations][4];            // R_r^+
+    typename P::K U[kAdjMaxRotations][4];      // R_r^+
 };
-
-__device__ __forceinline__ uint32_t adj_insert(uint32_t j, int p) {
-    const uint32_t lo = j & ((1u << p) - 1u);
-    return ((j ^ lo) << 1) | lo;
-}
 
 template <typename P>
 __global__ void __launch_bounds__(kAdjThreads, 4) k_adj_tile(typename P::C* __restrict__ psi, typename P::C* __restrict__ lam,
@@ -255,7 +245,7 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_adj_tile(typename P::C* __re
                 const int b0 = A.bit[r], b1 = A.bit[r + 1];
                 const int blo = min(b0, b1), bhi = max(b0, b1);
                 if (tid < N / 4) {  // N / 4 <= kAdjThreads
-                    const uint32_t l = adj_insert(adj_insert(tid, blo), bhi);
+                    const uint32_t l = insert_zero(insert_zero(tid, blo), bhi);
                     const uint32_t m0 = 1u << b0, m1 = 1u << b1;
                     C v[4] = {sp[l], sp[l | m0], sp[l | m1], sp[l | m0 | m1]};
                     C u[4] = {sl[l], sl[l | m0], sl[l | m1], sl[l | m0 | m1]};
@@ -280,7 +270,7 @@ __global__ void __launch_bounds__(kAdjThreads, 4) k_adj_tile(typename P::C* __re
                 const uint32_t m0 = 1u << A.bit[r];
                 typename R::Acc g;
                 for (uint32_t j = tid; j < N / 2; j += kAdjThreads) {
-                    const uint32_t l = adj_insert(j, A.bit[r]);
+                    const uint32_t l = insert_zero(j, A.bit[r]);
                     C a = sp[l], b = sp[l | m0], la = sl[l], lb = sl[l | m0];
                     R::step(a, b, la, lb, A.axis[r], A.U[r], g);
                     sp[l] = a;
@@ -521,12 +511,11 @@ size_t adj_diag_smem(int ntab, Arith ar) {
     return ((size_t(ntab) * kernel_entry_bytes(ar) + 15) & ~size_t(15)) + rs * (kAdjThreads / 32) * 32;
 }
 
-// R_P(theta)^+ = cos(theta/2) I - i sin(theta/2) P as a row-major 2x2 matrix
+// R_P(theta)^+ = cos(theta/2) I - i sin(theta/2) P as a row-major 2x2 matrix, P = X (axis 1) or Y
 void rot_dagger(int axis, double theta, cplx (&U)[4]) {
     const double c = std::cos(theta / 2), s = std::sin(theta / 2);
     if (axis == 1) { U[0] = c; U[1] = cplx(0, -s); U[2] = cplx(0, -s); U[3] = c; }
-    else if (axis == 2) { U[0] = c; U[1] = -s; U[2] = s; U[3] = c; }
-    else { U[0] = cplx(c, -s); U[1] = 0.0; U[2] = 0.0; U[3] = cplx(c, s); }
+    else { U[0] = c; U[1] = -s; U[2] = s; U[3] = c; }
 }
 
 // qubits 0 and 1 always lie in the tile: runs of 64 bytes (double-float)

@@ -311,11 +311,11 @@ WideMats upload_wide(qs_state* s, Arith ar, std::vector<Op>& ops) {
     for (size_t b = 0; b < ops.size(); b++) {
         if (ops[b].kind != OpKind::Dense || ops[b].targets.size() < 4) continue;
         if (ar == Arith::F32 && (ops[b].targets.size() == 5 || ops[b].targets.size() == 6) && tensor_c64x_enabled()) {
-            if (!std::is_sorted(ops[b].targets.begin(), ops[b].targets.end())) ops[b] = sort_targets(ops[b]);
+            ops[b] = sort_targets(std::move(ops[b]));
             oz[b] = char(10 + ops[b].targets.size());  // the complex64 form, 15 or 16
         }
         if (ar == Arith::DF && (ops[b].targets.size() == 4 || ops[b].targets.size() == 5) && tensor_c128_enabled()) {
-            if (!std::is_sorted(ops[b].targets.begin(), ops[b].targets.end())) ops[b] = sort_targets(ops[b]);
+            ops[b] = sort_targets(std::move(ops[b]));
             oz[b] = char(ops[b].targets.size());
         }
         offs[b] = total;

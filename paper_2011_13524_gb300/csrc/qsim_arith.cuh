@@ -314,7 +314,7 @@ __device__ __forceinline__ void dprod2(float2& s, float2& c, float2 ah, float2 a
     s = t;
     c = __fadd2_rn(c, __fadd2_rn(d, e));
 }
-__device__ __forceinline__ float4 df_dot2(float2 xh, float2 xl, const Pair2& a, float2 yh, float2 yl, const Pair2& b) {
+__device__ __forceinline__ float4 pair_dot(float2 xh, float2 xl, const Pair2& a, float2 yh, float2 yl, const Pair2& b) {
     float2 s, c;
     dprod2(s, c, xh, xl, a.h, a.l, true);
     dprod2(s, c, yh, yl, b.h, b.l, false);

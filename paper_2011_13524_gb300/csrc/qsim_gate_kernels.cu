@@ -899,13 +899,10 @@ void launch_from_df(void* psi, int n, cudaStream_t st) {
     QS_TRY_CUDA(cudaGetLastError());
 }
 
-Op sort_targets(const Op& op) {
-    if (std::is_sorted(op.targets.begin(), op.targets.end())) {
-        Op r = op;
-        r.dmat = nullptr;
-        r.dmat_oz = false;
-        return r;
-    }
+Op sort_targets(Op op) {
+    op.dmat = nullptr;
+    op.dmat_oz = false;
+    if (std::is_sorted(op.targets.begin(), op.targets.end())) return op;
     const int m = int(op.targets.size());
     std::vector<int> perm(m);
     for (int j = 0; j < m; j++) perm[j] = j;
@@ -923,8 +920,6 @@ Op sort_targets(const Op& op) {
         for (int z = 0; z < D; z++)
             for (int w = 0; w < D; w++) r.data[size_t(z) * D + w] = op.data[size_t(old_index(z)) * D + old_index(w)];
     }
-    r.dmat = nullptr;
-    r.dmat_oz = false;
     return r;
 }
 

@@ -425,7 +425,7 @@ void launch_slot_sums(const double* part, int nslots, unsigned nb, double* out, 
 // slices with exact FP32 accumulation).
 bool tensor_c128_enabled();
 // the same op with its targets ascending (matrix local bits permuted to match)
-Op sort_targets(const Op& op);
+Op sort_targets(Op op);
 // host image of the sliced operand of a 16 x 16 matrix (stacked bf16 slices, row scales)
 size_t oz4_matrix_bytes();
 void prepare_oz4_matrix(const std::vector<cplx>& K, unsigned char* host_out);

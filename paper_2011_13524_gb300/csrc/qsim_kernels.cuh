@@ -95,6 +95,12 @@ __device__ __forceinline__ void df_add_prod(DFAcc& acc, float a, float b) {
 }
 __device__ __forceinline__ double df_value(const DFAcc& a) { return double(a.hi) + double(a.lo); }
 
+// j with a zero inserted at bit p
+__device__ __forceinline__ uint32_t insert_zero(uint32_t j, int p) {
+    const uint32_t lo = j & ((1u << p) - 1u);
+    return ((j ^ lo) << 1) | lo;
+}
+
 // ---- block reductions (deterministic order)
 template <int NT>
 __device__ __forceinline__ double block_sum(double v, double* sh) {

@@ -67,8 +67,8 @@ struct PassParams {
     typename P::K data[NDATA];
 };
 
-// (a, b) <- K (a, b). Real matrices and those with a real diagonal and an imaginary off-diagonal
-// skip the products by zero.
+// (a, b) <- K (a, b). In FP64 and double-float, real matrices and those with a real diagonal and an imaginary
+// off-diagonal (mode 1, 2) skip the products by zero.
 template <typename P>
 __device__ __forceinline__ void pass_pair(const typename P::K* K, int, typename P::C& a, typename P::C& b) {
     typename P::Acc r0 = P::first(K[0], a), r1 = P::first(K[2], a);
@@ -99,12 +99,12 @@ __device__ __forceinline__ void pass_pair<DFArith>(const float4* K, int mode, fl
         a = df_mul_add2(K[0], K[1], va, wa, vb, wb);
         b = df_mul_add2(K[2], K[3], va, wa, vb, wb);
     } else if (mode == 1) {
-        a = df_dot2(dup(K[0].x), dup(K[0].y), va, dup(K[1].x), dup(K[1].y), vb);
-        b = df_dot2(dup(K[2].x), dup(K[2].y), va, dup(K[3].x), dup(K[3].y), vb);
+        a = pair_dot(dup(K[0].x), dup(K[0].y), va, dup(K[1].x), dup(K[1].y), vb);
+        b = pair_dot(dup(K[2].x), dup(K[2].y), va, dup(K[3].x), dup(K[3].y), vb);
     } else {  // i y b = (-y b.im, y b.re)
         const Pair2 wa = swapped(va), wb = swapped(vb);
-        a = df_dot2(dup(K[0].x), dup(K[0].y), va, mp(K[1].z), mp(K[1].w), wb);
-        b = df_dot2(mp(K[2].z), mp(K[2].w), wa, dup(K[3].x), dup(K[3].y), vb);
+        a = pair_dot(dup(K[0].x), dup(K[0].y), va, mp(K[1].z), mp(K[1].w), wb);
+        b = pair_dot(mp(K[2].z), mp(K[2].w), wa, dup(K[3].x), dup(K[3].y), vb);
     }
 }
 template <>
@@ -138,11 +138,6 @@ struct Tile {
     __device__ __forceinline__ C get(uint32_t l) const { return tile_order(s[l]); }
     __device__ __forceinline__ void put(uint32_t l, C v) const { s[l] = tile_order(v); }
 };
-
-__device__ __forceinline__ uint32_t insert_zero(uint32_t j, int p) {
-    const uint32_t lo = j & ((1u << p) - 1u);
-    return ((j ^ lo) << 1) | lo;
-}
 
 // k v, rounded as k_phase and k_diag do
 template <typename P>
