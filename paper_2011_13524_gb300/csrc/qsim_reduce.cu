@@ -777,31 +777,26 @@ SingleTerm single_term(const HeavyChunk& c) {
 }
 ExpectLaunches expectation_launches(const ExpectPlan& plan, int n, Arith ar, size_t cap) {
     auto is_single = [&](const HeavyChunk& c) { return c.g->xmask && c.g->coef.size() == 1 && ar != Arith::DF; };
-    auto build = [&](bool take_light) {
-        ExpectLaunches L;
-        if (plan.diag) L.pass_grid.push_back(expect_diag_grid(n, ar));
-        for (size_t p = 0; p < plan.passes.size(); p++) {
-            const auto& ch = plan.chunks[p];
-            if (take_light && ch.size() == 1 && is_single(ch[0])) {
-                L.singles.push_back(single_term(ch[0]));
-                continue;
-            }
-            L.passes.push_back(p);
-            L.pass_grid.push_back(expect_pass_grid(plan.passes[p], ar));
+    ExpectLaunches L;
+    if (plan.diag) L.pass_grid.push_back(expect_diag_grid(n, ar));
+    for (size_t p = 0; p < plan.passes.size(); p++) {
+        const auto& ch = plan.chunks[p];
+        if (ch.size() == 1 && is_single(ch[0])) {
+            L.singles.push_back(single_term(ch[0]));
+            continue;
         }
-        for (size_t h = 0; h < plan.heavy.size(); h++) {
-            if (is_single(plan.heavy[h])) {
-                L.singles.push_back(single_term(plan.heavy[h]));
-                continue;
-            }
-            L.heavy.push_back(h);
-            L.heavy_grid.push_back(red_grid((1ull << n) >> (plan.heavy[h].g->xmask ? 1 : 0)));
+        L.passes.push_back(p);
+        L.pass_grid.push_back(expect_pass_grid(plan.passes[p], ar));
+    }
+    for (size_t h = 0; h < plan.heavy.size(); h++) {
+        if (is_single(plan.heavy[h])) {
+            L.singles.push_back(single_term(plan.heavy[h]));
+            continue;
         }
-        return L;
-    };
-    ExpectLaunches L = build(true);
-    auto launches = [&]() { return L.pass_grid.size() + L.heavy_grid.size() + L.singles.size(); };
-    if (launches() > cap) L = build(false);
+        L.heavy.push_back(h);
+        L.heavy_grid.push_back(red_grid((1ull << n) >> (plan.heavy[h].g->xmask ? 1 : 0)));
+    }
+    const size_t launches = L.pass_grid.size() + L.heavy_grid.size() + L.singles.size();
     if (!L.singles.empty()) {
         // eight pairs per thread, at most 256 blocks per term unless few terms leave the GPU idle (2432
         // blocks per term measured no faster on states beyond L2: 25.4 / 25.9 ms for 24 strings at n = 28)
@@ -813,9 +808,8 @@ ExpectLaunches expectation_launches(const ExpectPlan& plan, int n, Arith ar, siz
     for (unsigned g : L.pass_grid) tot += g;
     for (unsigned g : L.heavy_grid) tot += g;
     if (tot > cap) {
-        const size_t nl = launches();
-        QS_REQUIRE(nl <= cap, "observable needs more kernel launches than the partial-sum scratch holds");
-        const size_t per = cap / nl;
+        QS_REQUIRE(launches <= cap, "observable needs more kernel launches than the partial-sum scratch holds");
+        const size_t per = cap / launches;
         for (unsigned& g : L.pass_grid) g = unsigned(std::min<size_t>(g, per));
         for (unsigned& g : L.heavy_grid) g = unsigned(std::min<size_t>(g, per));
         L.single_grid = unsigned(std::min<size_t>(L.single_grid, per));
