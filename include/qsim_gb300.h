@@ -270,8 +270,8 @@ qs_status qs_fused_layout_passes(const qs_fused_circuit* f, qs_dtype dt, int* pa
  * after every block; block_ms[b] receives the device time of block b. Synchronises. */
 qs_status qs_apply_fused_circuit_timed(qs_state* s, const qs_fused_circuit* f, float* block_ms);
 /* Fusion-width autotuner: plans c for every width 1..6, predicts each plan's device time from
- * per-kernel costs measured on this GPU (timed once per process on a scratch state of
- * min(n, 24) qubits and scaled by 2^n), and returns the fastest width in *best_k. pred_ms
+ * per-kernel costs measured on this GPU (timed once per process and size on a
+ * scratch state of min(n, 24) qubits, complex64 25, and scaled by 2^n beyond), and returns the fastest width in *best_k. pred_ms
  * (optional, 7 entries): index 0 = gate by gate, at one pass per gate (an upper estimate: a run
  * applies several gates per pass), 1..6 = fused widths. */
 qs_status qs_autotune_fusion(const qs_circuit* c, qs_dtype dt, int* best_k, double* pred_ms);

@@ -639,11 +639,11 @@ void trotter_by_blocks(qs_state* s, const qs_pauli_obs* H, double angle, int n_s
 }  // namespace
 
 // ------------------------------------------------------------------ autotuner
-// Seconds per algorithmic byte of each kernel form, measured once per process and device
-// on a scratch state, keyed by (device, dtype, c128 arithmetic, kernel, targets).
+// Seconds per algorithmic byte of each kernel form, measured once per process, device and probe size
+// on a scratch state, keyed by (device, dtype, c128 arithmetic, kernel, targets, qubits of the state).
 namespace {
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int, int, bool>, double> g_cost;
+std::map<std::tuple<int, int, int, int, int, bool, int>, double> g_cost;
 
 double measure_cost(int dev, qs_dtype dt, const Op& probe_op, int np_) {
     qs_state* s = nullptr;
@@ -762,8 +762,9 @@ double predicted_seconds(const Op& op, int n, qs_dtype dt) {
     int dev = 0;
     cudaGetDevice(&dev);
     const int width = op.kind == OpKind::Dense || op.kind == OpKind::Diag ? int(op.targets.size()) : 0;
+    const int np_ = std::max(8, std::min(n, dt == QS_C64 ? 25 : 24));
     auto key = std::make_tuple(dev, int(dt), dt == QS_C128 ? c128_math() : cur_tensor() & QS_TENSOR_C64X,
-                               kernel, width, touches_low(op));
+                               kernel, width, touches_low(op), np_);
     // (the kernel id already tells the tensor-core forms apart)
     double per_byte;
     {
@@ -772,7 +773,6 @@ double predicted_seconds(const Op& op, int n, qs_dtype dt) {
         if (it != g_cost.end()) {
             per_byte = it->second;
         } else {
-            const int np_ = std::max(8, std::min(n, dt == QS_C64 ? 25 : 24));
             per_byte = measure_cost(dev, dt, probe_like(op, np_), np_);
             g_cost[key] = per_byte;
         }
