@@ -270,10 +270,10 @@ qs_status qs_fused_layout_passes(const qs_fused_circuit* f, qs_dtype dt, int* pa
  * after every block; block_ms[b] receives the device time of block b. Synchronises. */
 qs_status qs_apply_fused_circuit_timed(qs_state* s, const qs_fused_circuit* f, float* block_ms);
 /* Fusion-width autotuner: plans c for every width 1..6, predicts each plan's device time from
- * per-kernel costs measured on this GPU (timed once per process and size on a
- * scratch state of min(n, 24) qubits, complex64 25, and scaled by 2^n beyond), and returns the fastest width in *best_k. pred_ms
- * (optional, 7 entries): index 0 = gate by gate, at one pass per gate (an upper estimate: a run
- * applies several gates per pass), 1..6 = fused widths. */
+ * per-kernel costs measured on this GPU (timed once per process and size on a scratch state of
+ * min(n, 24) qubits, complex64 25, and scaled by 2^n beyond), and returns the fastest width in *best_k. pred_ms
+ * (optional, 7 entries): index 0 = gate by gate, in the passes that such a run takes, 1..6 = fused
+ * widths. */
 qs_status qs_autotune_fusion(const qs_circuit* c, qs_dtype dt, int* best_k, double* pred_ms);
 /* Tile shape of the shared-memory dense kernel (QS_KERNEL_DENSE_SMEM: 4..6 targets on the CUDA
  * cores): output rows per thread, 4, 8 or 16 (the tile holds 256 rows / 2^m groups per row of

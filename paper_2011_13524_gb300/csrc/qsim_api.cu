@@ -199,6 +199,14 @@ void apply_single(qs_state* s, const Op& op) {
 // the costs of their kinds. Below, launches count more than traffic. A double-float run's first and last
 // passes also save a conversion pass as tiles, kConversionCost.
 constexpr double kConversionCost = 0.9;
+// whether passes[i] is launched gate by gate (`converts`: the run changes the layout at its ends)
+bool launched_alone(const std::vector<GatePass>& passes, size_t i, int n, Arith ar, bool converts) {
+    const GatePass& p = passes[i];
+    if (!p.local) return true;
+    const int ends = converts ? int(i == 0) + int(i + 1 == passes.size()) : 0;
+    if (n < kPassCostQubits) return p.ops.size() == 1 && !ends;
+    return p.alone < tile_cost(p, ar) - kConversionCost * ends;
+}
 // `fp64`: in IEEE doubles also where double-float is set.
 void run_ops(qs_state* s, const std::vector<Op>& ops, bool fp64 = false) {
     const bool df_run = use_df(s) && !s->df && !fp64;
@@ -208,13 +216,7 @@ void run_ops(qs_state* s, const std::vector<Op>& ops, bool fp64 = false) {
         DFScope df(s, df_run);
         return;
     }
-    auto single = [&](size_t i) {
-        const GatePass& p = passes[i];
-        if (!p.local) return true;
-        const int converts = df_run ? int(i == 0) + int(i + 1 == passes.size()) : 0;
-        if (s->n < kPassCostQubits) return p.ops.size() == 1 && !converts;
-        return p.alone < p.tile - kConversionCost * converts;
-    };
+    auto single = [&](size_t i) { return launched_alone(passes, i, s->n, ar, df_run); };
     // a double-float run changes the layout in its first and last passes where those are tile passes
     const bool in = df_run && !single(0), out = df_run && !single(passes.size() - 1);
     DFScope df(s, df_run, in);
@@ -754,6 +756,10 @@ Op probe_like(const Op& op, int np_) {
     return p;
 }
 
+// the settings that a measured cost depends on
+int cost_settings(qs_dtype dt) { return dt == QS_C128 ? c128_math() : cur_tensor() & QS_TENSOR_C64X; }
+int probe_qubits(int n, qs_dtype dt) { return std::max(8, std::min(n, dt == QS_C64 ? 25 : 24)); }
+
 double predicted_seconds(const Op& op, int n, qs_dtype dt) {
     int kernel = 0, launches = 0;
     double bytes = 0;
@@ -762,9 +768,8 @@ double predicted_seconds(const Op& op, int n, qs_dtype dt) {
     int dev = 0;
     cudaGetDevice(&dev);
     const int width = op.kind == OpKind::Dense || op.kind == OpKind::Diag ? int(op.targets.size()) : 0;
-    const int np_ = std::max(8, std::min(n, dt == QS_C64 ? 25 : 24));
-    auto key = std::make_tuple(dev, int(dt), dt == QS_C128 ? c128_math() : cur_tensor() & QS_TENSOR_C64X,
-                               kernel, width, touches_low(op), np_);
+    const int np_ = probe_qubits(n, dt);
+    auto key = std::make_tuple(dev, int(dt), cost_settings(dt), kernel, width, touches_low(op), np_);
     // (the kernel id already tells the tensor-core forms apart)
     double per_byte;
     {
@@ -786,9 +791,66 @@ double predict_plan(const FusionPlan& p, qs_dtype dt) {
     return t;
 }
 
+// seconds of a tile pass of `gates` general one-qubit gates on a probe state, best of three after a warm-up
+double measure_pass(qs_dtype dt, int np_, int gates) {
+    const Arith ar = dt == QS_C64 ? Arith::F32 : (c128_math() == QS_MATH_DF ? Arith::DF : Arith::F64);
+    const auto s = scratch_state(np_, dt, nullptr);
+    QS_TRY_CUDA(cudaMemsetAsync(s->data, 0, (size_t(1) << np_) * amp_bytes(dt), s->stream));
+    std::vector<Op> ops(static_cast<size_t>(gates));
+    for (int j = 0; j < gates; j++) {
+        ops[j].kind = OpKind::Dense;
+        ops[j].targets = {j % 8};
+        ops[j].data = {std::polar(0.6, 0.1), std::polar(0.8, 0.4), std::polar(0.8, 0.7), std::polar(-0.6, 1.0)};
+    }
+    const std::vector<GatePass> passes = schedule_passes(ops, np_, ar);
+    cudaEvent_t e0, e1;
+    QS_TRY_CUDA(cudaEventCreate(&e0));
+    QS_TRY_CUDA(cudaEventCreate(&e1));
+    float best = 1e30f;
+    for (int r = 0; r < 4; r++) {
+        QS_TRY_CUDA(cudaEventRecord(e0, s->stream));
+        launch_gate_pass(passes[0], ops, s->data, np_, ar, false, false, s->stream);
+        QS_TRY_CUDA(cudaEventRecord(e1, s->stream));
+        QS_TRY_CUDA(cudaEventSynchronize(e1));
+        float ms = 0;
+        QS_TRY_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+        if (r > 0) best = std::min(best, ms);
+    }
+    cudaEventDestroy(e0);
+    cudaEventDestroy(e1);
+    return 1e-3 * best;
+}
+
+// A tile pass: its staging and, by GatePass::inside, its gates, from probes of 1 and 9 gates
+double predicted_pass_seconds(const GatePass& p, int n, qs_dtype dt, Arith ar) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int np_ = probe_qubits(n, dt);
+    auto probe = [&](int gates) {  // (kernel id -1: a tile pass)
+        const auto key = std::make_tuple(dev, int(dt), cost_settings(dt), -1, gates, false, np_);
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        auto it = g_cost.find(key);
+        return it != g_cost.end() ? it->second : (g_cost[key] = measure_pass(dt, np_, gates));
+    };
+    const double one = probe(1), gate = std::max(0.0, (probe(9) - one) / 8.0);
+    const double t = std::max(0.0, one - gate) + gate * p.inside / kPassGateInside[int(ar)];
+    return t * std::ldexp(1.0, n - np_) + 2e-6;
+}
+
+// a run gate by gate, in the passes that it takes
 double predict_unfused(const qs_circuit* c, qs_dtype dt) {
+    const Arith ar = dt == QS_C64 ? Arith::F32 : (c128_math() == QS_MATH_DF ? Arith::DF : Arith::F64);
+    std::vector<Op> ops;
+    for (int i = 0; i < c->n_gates; i++) ops.push_back(op_of_gate(c->gates[i], c->n, nullptr));
+    const std::vector<GatePass> passes = schedule_passes(ops, c->n, ar);
     double t = 0;
-    for (int i = 0; i < c->n_gates; i++) t += predicted_seconds(op_of_gate(c->gates[i], c->n, nullptr), c->n, dt);
+    for (size_t i = 0; i < passes.size(); i++) {
+        if (launched_alone(passes, i, c->n, ar, ar == Arith::DF)) {
+            for (size_t k : passes[i].ops) t += predicted_seconds(ops[k], c->n, dt);
+        } else {
+            t += predicted_pass_seconds(passes[i], c->n, dt, ar);
+        }
+    }
     return t;
 }
 

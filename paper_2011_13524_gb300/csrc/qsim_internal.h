@@ -228,10 +228,13 @@ struct GatePass {
     std::vector<size_t> ops;  // indices into the run's ops
     uint64_t local = 0;       // the tile's qubits
     size_t data = 0;          // matrix entries
-    double alone = 0.0;       // estimated cost of the ops as launches of their own, and
-    double tile = 0.0;        // as this pass, in light full passes over the state (measured from 20 qubits on)
+    // estimated cost of the ops as launches of their own, and inside a tile beside its staging, in light
+    // full passes over the state (measured from kPassCostQubits on)
+    double alone = 0.0, inside = 0.0;
 };
 constexpr int kPassCostQubits = 20;
+constexpr double kPassGateInside[3] = {0.45, 2.55, 0.72};  // `inside` of a general one-qubit gate, by Arith
+double tile_cost(const GatePass& p, Arith ar);
 int gate_pass_bits(int n, Arith ar);
 std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith ar);
 double scheduled_cost(const std::vector<Op>& ops, int n, Arith ar);  // of all passes, in light full passes

@@ -359,9 +359,9 @@ struct ClassCost {
     double alone, inside;
 };
 constexpr ClassCost kClassCost[3][kOpClasses] = {  // by Arith
-    {{1.0, 0.45}, {1.0, 0.45}, {1.3, 0.75}, {1.1, 0.38}, {1.05, 1.1}, {1.9, 0.35}, {1.05, 0.45}, {1.05, 0.5}},    // F32
-    {{2.9, 2.55}, {1.5, 1.4}, {5.8, 5.0}, {1.0, 0.2}, {1.45, 1.5}, {1.6, 0.25}, {1.0, 0.3}, {2.0, 2.1}},         // F64
-    {{1.0, 0.72}, {1.0, 0.45}, {1.15, 1.25}, {1.2, 0.28}, {1.0, 1.0}, {1.4, 0.25}, {0.95, 0.38}, {1.05, 0.55}},  // DF
+    {{1.0, kPassGateInside[0]}, {1.0, 0.45}, {1.3, 0.75}, {1.1, 0.38}, {1.05, 1.1}, {1.9, 0.35}, {1.05, 0.45}, {1.05, 0.5}},    // F32
+    {{2.9, kPassGateInside[1]}, {1.5, 1.4}, {5.8, 5.0}, {1.0, 0.2}, {1.45, 1.5}, {1.6, 0.25}, {1.0, 0.3}, {2.0, 2.1}},         // F64
+    {{1.0, kPassGateInside[2]}, {1.0, 0.45}, {1.15, 1.25}, {1.2, 0.28}, {1.0, 1.0}, {1.4, 0.25}, {0.95, 0.38}, {1.05, 0.55}},  // DF
 };
 static_assert(int(Arith::F32) == 0 && int(Arith::F64) == 1 && int(Arith::DF) == 2, "order of kClassCost");
 constexpr double kPassBase[3] = {0.95, 1.1, 1.1};
@@ -580,7 +580,6 @@ std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith a
         }
         uint64_t L = low, bx = 0, bd = 0;
         size_t data = 0;
-        p.tile = kPassBase[int(ar)];
         keep.clear();
         bool ended = false;
         for (size_t i : rem) {
@@ -592,7 +591,7 @@ std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith a
                 data += e;
                 const ClassCost cost = op_pass_cost(op, ar);
                 p.alone += cost.alone;
-                p.tile += cost.inside;
+                p.inside += cost.inside;
                 p.ops.push_back(i);
             } else {
                 bx |= q[i].x;
@@ -610,9 +609,11 @@ std::vector<GatePass> schedule_passes(const std::vector<Op>& ops, int n, Arith a
     return out;
 }
 
+double tile_cost(const GatePass& p, Arith ar) { return kPassBase[int(ar)] + p.inside; }
+
 double scheduled_cost(const std::vector<Op>& ops, int n, Arith ar) {
     double t = 0.0;
-    for (const GatePass& p : schedule_passes(ops, n, ar)) t += p.local ? std::min(p.alone, p.tile) : p.alone;
+    for (const GatePass& p : schedule_passes(ops, n, ar)) t += p.local ? std::min(p.alone, tile_cost(p, ar)) : p.alone;
     return t;
 }
 

@@ -29,3 +29,14 @@ def test_small_probe_does_not_serve_large_states(dtype):
     c = W.u3cz_circuit(22, 4, 2)
     pred = qs.autotune_fusion(c, dtype)[1]
     assert pred[4] < 10.0 * measured_ms(qs, c, dtype, 4)  # (8192 times too long otherwise)
+
+
+@pytest.mark.parametrize("dtype", [2, 1])
+@pytest.mark.parametrize("n", [12, 20, 23])
+def test_unfused_prediction_counts_passes(n, dtype):
+    """Index 0 follows a run that applies several gates per pass (175 gates in 4 passes at n = 12), within
+    the host's share at small sizes and the spread of the gates' costs."""
+    import paper_2011_13524_gb300 as qs
+    c = W.u3cz_circuit(n, 10, 2)
+    pred, got = qs.autotune_fusion(c, dtype)[1][0], measured_ms(qs, c, dtype, 0)
+    assert got / 4.0 < pred < 2.0 * got
