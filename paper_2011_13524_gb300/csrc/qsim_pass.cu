@@ -541,9 +541,10 @@ void launch_pass_p(const Op* const* ops, int nops, size_t ndata, uint64_t local,
 
 // Tile bits: up to a 32 KB tile (fewer passes) once 2^8 tiles fill the SMs, never below 8 (9 in FP32)
 // bits: under that the extra passes cost more than the wider spread over SMs gives. Whole calls of the
-// depth-10 circuit with at least 7 / 8 / 9 bits: 147 / 142 / 152 us at n = 12 and 173 / 162 / 175 at
-// n = 14 in complex128, 138 / 123 / 124 us at n = 12 and 159 / 147 / 145 at n = 14 in complex64 (with
-// passes in any order).
+// depth-10 U3 + CZ circuit (and of four repetitions of RZ RX RZ + CNOT layers) with at least 7 / 8 / 9 / 10
+// bits: complex128 142 / 137 / 147 / 199 us (186 / 174 / 203 / 288) at n = 12, 173 / 162 / 173 / 226 (220 / 212 /
+// 236 / 335) at n = 14; complex64, whose passes end with the first gate that does not fit, 195 / 180 / 166 /
+// 175 (216 / 203 / 212 / 270) at n = 12 and 230 / 220 / 199 / 203 (257 / 240 / 251 / 324) at n = 14.
 int gate_pass_bits(int n, Arith ar) {
     const int most = ar == Arith::F32 ? 12 : 11, least = ar == Arith::F32 ? 9 : 8;
     return std::min(n, std::max(least, std::min(most, n - 8)));
