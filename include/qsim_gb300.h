@@ -199,7 +199,9 @@ qs_status qs_synchronize(const qs_state* s);
 /* ---------------------------------------------------------------- gates (Sec. 4.3) */
 /* psi <- K psi for one gate (Eq. update_mat; controlled, diagonal, Pauli and named forms).
  * complex128 dense gates of 3 or more targets use the double-float arithmetic (with its layout
- * change in and out) when it is selected; other gates use IEEE FP64 arithmetic, one pass. */
+ * change in and out) when it is selected; other gates use IEEE FP64 arithmetic, one pass. Products with
+ * an entry's zero real or imaginary part may be left out, here and where gates are merged: finite values
+ * are the same, an Inf or NaN may reach fewer components than 0 * Inf = NaN would carry it to. */
 qs_status qs_apply_gate(qs_state* s, const qs_gate* g);
 /* psi <- K psi for a dense k-qubit matrix (k in 1..6), as produced by gate fusion
  * (Sec. 5.4 merge). Equivalent to qs_apply_gate with a QS_GATE_DENSE gate. */

@@ -45,7 +45,8 @@ struct DenseRegParams {
 
 // One-qubit FP64 gates are bound by the FP64 rate (GB300: 1/64 of FP32), eight multiply-adds per
 // amplitude in general; entries that are real (H, RY) or whose off-diagonal is imaginary (RX) need
-// four: 516 / 265 us at n = 25. The values are those of the general form, whose other products are zero.
+// four: 516 / 265 us at n = 25. Finite values are those of the general form, whose other products are zero
+// (an Inf or NaN stays in the component that 0 * Inf would have carried it from).
 __device__ __forceinline__ void pair_form(const double2* K, int form, double2 a, double2 b, double2& ra, double2& rb) {
     ra = make_double2(K[0].x * a.x, K[0].x * a.y);
     if (form == 1) {

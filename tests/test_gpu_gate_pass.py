@@ -133,3 +133,31 @@ def test_launches_between_passes(n, arith):
     assert float((a.tensor - b.tensor).abs().max()) < TOL[arith]
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("arith", ["f64", "c64"])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_not_finite(bad, arith):
+    """An amplitude that is not finite reaches the same amplitudes through passes as through single gates."""
+    import torch
+    import paper_2011_13524_gb300 as qs
+    n = 12
+    dt, tdt = (qs.QS_C64, torch.complex64) if arith == "c64" else (qs.QS_C128, torch.complex128)
+    v = random_tensor(n, tdt, 3)
+    v[77] = complex(bad, 0.5)
+    a, b = qs.State(n, dt, tensor=v.clone()), qs.State(n, dt, tensor=v)
+    for s in (a, b):
+        s.set_arith(math=qs.QS_MATH_FP64)
+    gates = [W.Gate("H", (0,)), W.Gate("RX", (5,), params=(0.3,)), W.Gate("RZ", (1,), params=(0.2,)), W.Gate("CZ", (0, 11)),
+             W.Gate("U3", (11,), params=(0.3, 0.2, 0.7)), W.Gate("SWAP", (3, 9)), W.Gate("PAULIROT", (2, 7), pauli=(1, 3), params=(0.4,))]
+    a.run(W.Circuit(n, gates), 0)
+    for g in gates:
+        b.apply_gate(g)
+    a.synchronize()
+    b.synchronize()
+    x, y = torch.view_as_real(a.tensor), torch.view_as_real(b.tensor)
+    fine = torch.isfinite(y)
+    assert torch.equal(torch.isfinite(x), fine) and 0 < int((~fine).sum()) < y.numel()
+    assert float((x - y)[fine].abs().max()) < TOL[arith]
+    a.close()
+    b.close()

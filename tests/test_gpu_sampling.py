@@ -71,3 +71,24 @@ def test_marginal_by_insertion_and_by_deposit():
         mv = [(val >> q) & 1 if (mask >> q) & 1 else 2 for q in range(n)]
         assert abs(st.marginal_probability(mv) - p[(x & mask) == val].sum()) < 1e-14
     st.close()
+
+
+@pytest.mark.parametrize("dtype", ["c128", "c64"])
+def test_outside_the_range_of_pairs(dtype):
+    """A state of large norm takes the FP64 search (the indices of the same state scaled down), and one
+    that is not finite is refused by either search."""
+    import paper_2011_13524_gb300 as qs
+    n = 14
+    st = qs.State(n, qs.QS_C64 if dtype == "c64" else qs.QS_C128)
+    v = make_vec("random", n, 3).astype(np.complex64).astype(np.complex128)
+    u = uniforms(2000, 4)
+    st.load(v)
+    ref = st.sample(u)
+    st.load(v * 2.0 ** 45)
+    assert np.array_equal(st.sample(u), ref)
+    v[321] = np.nan
+    st.load(v)
+    with pytest.raises(qs.QsError) as e:
+        st.sample(u)
+    assert e.value.code == qs.QS_ERR_NUMERIC
+    st.close()
