@@ -139,7 +139,8 @@ constexpr int kMaxSingles = 64;
 struct SingleTerm {
     uint64_t f, z;
     double coef;     // with the pair's factor +-2
-    int32_t pivot;   // lowest bit of f, clear in y
+    int32_t pivot;   // highest bit of f, clear in y: runs of y and y ^ f then fill their lines (a string that
+                     // flips qubits 0 and 25 at n = 26, complex128: 0.37 ms from the lowest bit, 0.24 from the highest)
     int32_t imag;    // 1: Im A
 };
 struct SingleParams {
@@ -769,7 +770,7 @@ SingleTerm single_term(const HeavyChunk& c) {
     SingleTerm t;
     t.f = c.g->xmask;
     t.z = c.g->zmask[c.t0];
-    t.pivot = __builtin_ctzll(t.f);
+    t.pivot = 63 - __builtin_clzll(t.f);
     const int nY = __builtin_popcountll(t.f & t.z);
     t.imag = nY & 1;
     t.coef = (((nY + 1) / 2) & 1) ? -2.0 * c.g->coef[c.t0] : 2.0 * c.g->coef[c.t0];
