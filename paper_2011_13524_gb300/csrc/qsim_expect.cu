@@ -716,7 +716,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_transition_tiled(const C* _
 // instructions per string and amplitude (seven in complex64) where the products take 40. Whatever else
 // the tile holds, w_y keeps 2^-45 of the components it is the sum of.
 // What bounds it: the FP32 pipe. Norms, inner product and the Ising chain's amplitude at n = 26
-// (complex128): 5.94 ms with the X terms in tiled reads, 4.25 ms here, about 2.0 of them for 26 strings.
+// (complex128): 5.94 ms with the X terms in tiled reads, 4.25 ms here, 2.15 of them for 26 strings (12, 9
+// and 5 in a read: 0.84, 0.73 and 0.58 ms).
 // Error of the amplitude on random states, rms: 2.3e-15 against 6.4e-15 at n = 12 (1.2e-15 / 2.4e-15 at
 // n = 15; complex64 2.2e-15 / 5.3e-15 and 1.0e-15 / 2.3e-15). Sums on one fixed-point grid per tile took 0.35
 // ms less, but a component's error was then 2^-49 of the tile's largest: beside an amplitude of 1, one of

@@ -132,9 +132,9 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_group(const C* __restric
 //    pair side by side in packed instructions; one FP64 conversion per thread. A pair with a product
 //    below 2^-100 (its rounding error can fall under FP32's range) or from 2^80 on goes to an FP64 sum
 //    instead, as the group kernel forms it.
-// 24 random strings, whole call, one launch per group / here: complex64 1.62 / 0.35 ms at n = 23 (300 us
-// of kernel, 15 of them for the range; L2 reads and packed FP32 arithmetic about equal) and 67.8 / 12.9 ms at n = 28, complex128
-// 0.75 / 0.36 ms at n = 22 and 50.9 / 25.4 ms at n = 28.
+// 24 random strings, whole call, one launch per group / here: complex64 1.62 / 0.36 ms at n = 23 (300 us
+// of kernel, 15 of them for the range; L2 reads and packed FP32 arithmetic about equal) and 67.8 / 9.7 ms
+// at n = 28, complex128 0.75 / 0.37 ms at n = 22 and 50.9 / 17.9 ms at n = 28.
 constexpr int kMaxSingles = 64;
 struct SingleTerm {
     uint64_t f, z;
@@ -755,9 +755,9 @@ void reduce_inner(const qs_state* a, const qs_state* b, double out[2]) {
 
 // Launches of one expectation: the tile passes, one launch per heavy chunk, and the terms that are
 // alone in their flip group together (k_expect_singles): those that fit no tile, and one that a tile
-// pass would stage the state for alone (whole calls, tile pass / single term: 173 / 135 us at n = 25 and
-// 1138 / 790 us at n = 28 in complex128, 111 / 86 and 654 / 433 us in complex64; with two terms the tile
-// pass is the faster one, 740 / 1052 us at n = 28 in complex64). With a
+// pass would stage the state for alone (whole calls, tile pass / single term: 173 / 142 us at n = 25 and
+// 1138 / 801 us at n = 28 in complex128, 111 / 99 and 654 / 463 us in complex64; two terms take the tile
+// pass, 740 us at n = 28 in complex64). With a
 // cap on the block partials the grids shrink proportionally (the kernels loop over their work).
 struct ExpectLaunches {
     std::vector<unsigned> pass_grid, heavy_grid;  // a diagonal observable: its one streaming pass in pass_grid
@@ -800,7 +800,7 @@ ExpectLaunches expectation_launches(const ExpectPlan& plan, int n, Arith ar, siz
     const size_t launches = L.pass_grid.size() + L.heavy_grid.size() + L.singles.size();
     if (!L.singles.empty()) {
         // eight pairs per thread, at most 256 blocks per term unless few terms leave the GPU idle (2432
-        // blocks per term measured no faster on states beyond L2: 25.4 / 25.9 ms for 24 strings at n = 28)
+        // blocks per term measured no faster on states beyond L2)
         const uint64_t want = ((1ull << (n - 1)) + kRedThreads * 8 - 1) / (kRedThreads * 8);
         const uint64_t most = std::max<uint64_t>(256, uint64_t(sms()) * 8 / L.singles.size());
         L.single_grid = unsigned(std::max<uint64_t>(1, std::min(want, most)));
