@@ -224,7 +224,11 @@ void run_ops(qs_state* s, const std::vector<Op>& ops, bool fp64 = false) {
         const GatePass& p = passes[i];
         const bool last = i + 1 == passes.size();
         if (single(i)) {
-            for (size_t k : p.ops) launch_op_arith(ops[k], s->data, s->n, ar, s->stream, stage_of(s));
+            for (size_t k : p.ops) {
+                // (only wide gates read their matrix from the staging buffer: the others allocate nothing)
+                const bool staged = ops[k].kind == OpKind::Dense && ops[k].targets.size() >= 4;
+                launch_op_arith(ops[k], s->data, s->n, ar, s->stream, staged ? stage_of(s) : nullptr);
+            }
         } else {
             launch_gate_pass(p, ops, s->data, s->n, ar, in && i == 0, out && last, s->stream);
             if (in && i == 0) df.entered();

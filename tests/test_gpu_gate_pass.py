@@ -161,3 +161,33 @@ def test_not_finite(bad, arith):
     assert float((x - y)[fine].abs().max()) < TOL[arith]
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("arith", ["df", "c64"])
+@pytest.mark.parametrize("n", [12, 21])
+def test_capture(n, arith):
+    """A run gate by gate on a new state is launches alone, whether its passes are tiles or launches."""
+    import torch
+    import paper_2011_13524_gb300 as qs
+    dt, tdt = (qs.QS_C64, torch.complex64) if arith == "c64" else (qs.QS_C128, torch.complex128)
+    st = torch.cuda.Stream()
+    v = random_tensor(n, tdt, n)
+    a, b = qs.State(n, dt, tensor=v.clone(), stream=st), qs.State(n, dt, tensor=v)
+    torch.cuda.synchronize()
+    rot = tuple(1 + q % 3 for q in range(6))
+    gates = [W.Gate("RZ", (3,), params=(0.2,)), W.Gate("PAULIROT", tuple(range(0, 12, 2)), pauli=rot, params=(0.3,)),
+             W.Gate("DIAG", (1, n - 1), matrix=np.exp(1j * np.arange(4))), W.Gate("CZ", (0, 5)), W.Gate("H", (2,)),
+             W.Gate("DENSE", (0, 4, n - 1), matrix=W.random_unitary(8, W.SplitMix64(5))), W.Gate("SWAP", (1, 2))]
+    c = W.Circuit(n, gates + W.u3cz_circuit(n, 2, 3).gates)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=st):
+        a.run(c, 0)
+    with torch.cuda.stream(st):
+        graph.replay()
+    b.run(c, 0)
+    a.synchronize()
+    b.synchronize()
+    torch.cuda.synchronize()
+    assert torch.equal(a.tensor, b.tensor)
+    a.close()
+    b.close()
