@@ -716,10 +716,10 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_transition_tiled(const C* _
 // instructions per string and amplitude (seven in complex64) where the products take 40. Whatever else
 // the tile holds, w_y keeps 2^-45 of the components it is the sum of.
 // What bounds it: the FP32 pipe. Norms, inner product and the Ising chain's amplitude at n = 26
-// (complex128): 5.94 ms with the X terms in tiled reads, 4.25 ms here, 2.15 of them for 26 strings (12, 9
-// and 5 in a read: 0.84, 0.73 and 0.58 ms).
+// (complex128): 5.94 ms with the X terms in tiled reads, 4.18 ms here, 2.08 of them for 26 strings (12, 9
+// and 5 in a read: 0.80, 0.69 and 0.59 ms).
 // Error of the amplitude on random states, rms: 2.3e-15 against 6.4e-15 at n = 12 (1.2e-15 / 2.4e-15 at
-// n = 15; complex64 2.2e-15 / 5.3e-15 and 1.0e-15 / 2.3e-15). Sums on one fixed-point grid per tile took 0.35
+// n = 15; complex64 2.2e-15 / 5.3e-15 and 1.0e-15 / 2.3e-15). Sums on one fixed-point grid per tile took 0.3
 // ms less, but a component's error was then 2^-49 of the tile's largest: beside an amplitude of 1, one of
 // 2^-40 was 20 % off.
 __device__ __forceinline__ float2 tile_hi(float4 v) { return make_float2(v.x, v.y); }
@@ -798,18 +798,23 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_xsum(const C* __restrict__ 
             for (int j = 0; j < kH; j++) b[j] = bra[at | P.dep_hi[hf * kH + j]];
             float2 ws[kH], wc[kH];
 #pragma unroll
-            for (int j = 0; j < kH; j++) ws[j] = wc[j] = make_float2(0.f, 0.f);
+            for (int j = 0; j < kH; j++) {  // (the first string is its own sum)
+                T x = T();
+                if (P.nf) x = tile[tid ^ P.f[0] ^ uint32_t(kTileThreads * (hf * kH + j))];
+                ws[j] = tile_hi(x);
+                wc[j] = tile_lo(x);
+            }
+            for (int g = 1; g < P.nf; g++) {
+                const uint32_t o = tid ^ P.f[g];
+#pragma unroll
+                for (int j = 0; j < kH; j++) acc_sum2(ws[j], wc[j], tile[o ^ uint32_t(kTileThreads * (hf * kH + j))]);
+            }
 #pragma unroll
             for (int q = 0; q < 4; q++)
                 if ((P.item >> q) & 1u) {
 #pragma unroll
                     for (int j = 0; j < kH; j++) acc_sum2(ws[j], wc[j], own[(hf * kH + j) ^ (1 << q)]);
                 }
-            for (int g = 0; g < P.nf; g++) {
-                const uint32_t o = tid ^ P.f[g];
-#pragma unroll
-                for (int j = 0; j < kH; j++) acc_sum2(ws[j], wc[j], tile[o ^ uint32_t(kTileThreads * (hf * kH + j))]);
-            }
 #pragma unroll
             for (int j = 0; j < kH; j++) {
                 float2 wl;
