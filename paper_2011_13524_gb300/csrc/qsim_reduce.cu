@@ -129,11 +129,11 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_group(const C* __restric
 //    seven per pair and term).
 //  * complex64: products exact in FP32 pairs, summed with two levels of compensation (TwoSum of the
 //    sums and of their errors: nothing above 2^-70 of a thread's sum is dropped), both components of a
-//    pair side by side in packed instructions; one FP64 conversion per thread. A pair with a product
-//    below 2^-100 (its rounding error can fall under FP32's range) or from 2^80 on goes to an FP64 sum
-//    instead, as the group kernel forms it.
+//    pair side by side in packed instructions; one FP64 conversion per thread. Where a product
+//    lies below 2^-100 (its rounding error can fall under FP32's range) or from 2^80 on, the four pairs
+//    loaded with it go to an FP64 sum instead, as the group kernel forms it.
 // 24 random strings, whole call, one launch per group / here: complex64 1.62 / 0.36 ms at n = 23 (300 us
-// of kernel, 15 of them for the range; L2 reads and packed FP32 arithmetic about equal) and 67.8 / 9.7 ms
+// of kernel, 15 of them for the range; L2 reads and packed FP32 arithmetic about equal) and 67.8 / 9.4 ms
 // at n = 28, complex128 0.75 / 0.37 ms at n = 22 and 50.9 / 17.9 ms at n = 28.
 constexpr int kMaxSingles = 64;
 struct SingleTerm {
@@ -171,16 +171,19 @@ struct SingleAccF {  // complex64
         const float2 p = __fmul2_rn(factor(a, imag, neg), b);
         return max(range(p.x), range(p.y)) < kRange;
     }
-    template <bool kInRange>
+    // the same, or a product that a factor makes zero, which is exact (real and sparse states: 24 strings at
+    // n = 28 10.8 ms, general ones 9.4, amplitudes spread over 97 binary orders 36, per group 75)
+    __device__ __forceinline__ static bool in_range_or_zero(float2 a, float2 b, bool imag, int neg) {
+        const float2 u = factor(a, imag, neg), p = __fmul2_rn(u, b);
+        return (range(p.x) < kRange || u.x == 0.f || b.x == 0.f) && (range(p.y) < kRange || u.y == 0.f || b.y == 0.f);
+    }
+    __device__ __forceinline__ void add_wide(float2 a, float2 b, bool imag, int neg) {
+        const float2 u = factor(a, imag, neg);
+        wide = fma(widen_float_int(u.x), widen_float_int(b.x), wide);
+        wide = fma(widen_float_int(u.y), widen_float_int(b.y), wide);
+    }
     __device__ __forceinline__ void add(float2 a, float2 b, bool imag, int neg) {
         const float2 u = factor(a, imag, neg), p = __fmul2_rn(u, b);
-        if constexpr (!kInRange) {  // (a product that a factor makes zero is exact)
-            if ((range(p.x) >= kRange && u.x != 0.f && b.x != 0.f) || (range(p.y) >= kRange && u.y != 0.f && b.y != 0.f)) {
-                wide = fma(double(u.x), double(b.x), wide);
-                wide = fma(double(u.y), double(b.y), wide);
-                return;
-            }
-        }
         float2 e, e2;
         s = two_sum2(s, p, e);
         e = __fadd2_rn(e, __ffma2_rn(u, b, make_float2(-p.x, -p.y)));
@@ -194,13 +197,14 @@ struct SingleAccF {  // complex64
 struct SingleAccD {  // complex128
     double s = 0.0, c = 0.0;
     __device__ __forceinline__ static bool in_range(double2, double2, bool, int) { return true; }
-    template <bool>
+    __device__ __forceinline__ static bool in_range_or_zero(double2, double2, bool, int) { return true; }
     __device__ __forceinline__ void add(double2 a, double2 b, bool imag, int neg) {
         const long long sg = static_cast<long long>(uint64_t(neg) << 63);
         const double ux = imag ? a.y : a.x, uy = imag ? -a.x : a.y;
         s = fma(__longlong_as_double(__double_as_longlong(ux) ^ sg), b.x, s);
         c = fma(__longlong_as_double(__double_as_longlong(uy) ^ sg), b.y, c);
     }
+    __device__ __forceinline__ void add_wide(double2 a, double2 b, bool imag, int neg) { add(a, b, imag, neg); }
     __device__ double value() const { return s + c; }
 };
 
@@ -225,19 +229,25 @@ __global__ void __launch_bounds__(kRedThreads) k_expect_singles(const C* __restr
             b[u] = psi[y ^ T.f];
             neg[u] = parity64(y & T.z);
         }
-        bool fast = i0 + (kU - 1) * stride < P.pairs;  // (one branch for the four: their sums interleave)
-        if (fast) {
+        const bool four = i0 + (kU - 1) * stride < P.pairs;
+        bool fast = four;  // (one branch for the four: their sums interleave)
+        if (four) {
 #pragma unroll
             for (int u = 0; u < kU; u++) fast &= Acc::in_range(a[u], b[u], imag, neg[u]);
+            if (!fast) {  // real or sparse states
+                fast = true;
+#pragma unroll
+                for (int u = 0; u < kU; u++) fast &= Acc::in_range_or_zero(a[u], b[u], imag, neg[u]);
+            }
         }
         if (fast) {
 #pragma unroll
-            for (int u = 0; u < kU; u++) acc.template add<true>(a[u], b[u], imag, neg[u]);
+            for (int u = 0; u < kU; u++) acc.add(a[u], b[u], imag, neg[u]);
         } else {
 #pragma unroll
             for (int u = 0; u < kU; u++) {
                 if (i0 + u * stride >= P.pairs) break;
-                acc.template add<false>(a[u], b[u], imag, neg[u]);
+                acc.add_wide(a[u], b[u], imag, neg[u]);
             }
         }
     }
